@@ -96,6 +96,7 @@ struct Plan {
     unsigned long long* acc = nullptr;  // fixed-point sums of the cluster-list dispersion pass
     unsigned long long* npairs = nullptr;  // pair count of the cluster-list dispersion pass
     float* vd = nullptr;                // C6 projections (v, dv) per atom of the cluster-list dispersion pass
+    int vd_images = 0;                  // image atoms have rows of vd of their own (cluster lists only)
 };
 
 // The plan's Work set up for a list mode (kernel arguments are taken by value).
@@ -104,6 +105,7 @@ void set_mode(Plan& P, int mode) {
     P.w.acc = mode == kClusterLists ? P.acc : nullptr;
     P.w.npairs = mode == kClusterLists ? P.npairs : nullptr;
     P.w.vd = mode == kClusterLists ? P.vd : nullptr;
+    P.w.vd_images = mode == kClusterLists ? P.vd_images : 0;  // without vd there are no rows to copy
 }
 
 }  // namespace
@@ -760,7 +762,8 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         if (!grow) {
             // image rows of v and dv are copies of their source's when that is cheap
             // (few images, or few types); otherwise the pass resolves each image's source
-            P.w.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
+            P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
+            set_mode(P, mode);
             P.sized[mode] = true;
             return tune_shapes(h, P, pos, types, st, mode);
         }

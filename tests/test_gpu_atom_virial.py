@@ -69,6 +69,26 @@ def test_atom_virial_vs_oracle(torch_cuda, oracle_mod, precision, case):
         assert_mixed_ok(plain, full, b.offsets)
 
 
+def test_atom_virial_wide_cell(torch_cuda):
+    """A cell so wide that its images are few (images x types <= 2 x atoms): the cluster lists then give
+    image atoms rows of their own, which the full lists of the per-atom virial do not have."""
+    from paper_2310_05279_gb300 import D3
+    g = np.random.Generator(np.random.PCG64(16))
+    b = wl.batch_of([wl.bilayer(10, 18, 3.4, wl.BOND, 20.0, 0.02, g)], wl.carbon_table(1000))
+    pos, typ = to_dev(b)
+    out = {}
+    for precision in ("mixed", "fp64"):
+        d3 = D3(b.tables, precision=precision)
+        d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc)  # sizes the other list mode first
+        out[precision] = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc, w_atom=True)
+        d3.sync_status()
+        if precision == "mixed":
+            stats = d3.list_stats()
+            assert stats["image_atoms"] * b.tables.ntypes <= 2 * stats["real_atoms"] and stats["list_mode"] == 0
+    wa, ref = (out[k]["w_atom"].cpu().numpy() for k in ("mixed", "fp64"))
+    assert np.abs(wa - ref).max() <= TOL_WA["mixed"] * np.abs(ref).max()
+
+
 def test_heat_current(torch_cuda):
     torch = torch_cuda
     from paper_2310_05279_gb300 import D3, heat_current
