@@ -16,6 +16,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/d3gb.h"
@@ -25,6 +26,8 @@ namespace d3gb {
 cudaError_t launch_build_impl(const Work& w, const double* pos, const int32_t* types, const double* rk_tab,
                               int* bsum, cudaStream_t st, cudaEvent_t* lmarks = nullptr);
 int64_t scan_scratch_ints(int64_t ncells);
+cudaError_t launch_plan_ids(const StructGeo* geo, const int64_t* offsets, int B, int64_t Nr, int64_t ncl, int64_t nfin,
+                            int* sid_in, int* clu_sid, int* fin_sid, cudaStream_t st);
 cudaError_t launch_backward(const Work& w, const Consts& c, const double* c6d, const dbl4* paird,
                             const double* cnref, const int* nref, const Tabs& tbm, const double* dLdE,
                             const double* dLdF, double* dLdp, double* dLdx, double* scratch, int B, bool mixed,
@@ -71,6 +74,57 @@ struct DevBuf {
     }
 };
 
+// One device allocation that the buffers of successive plans are laid out in.  A
+// new geometry that fits takes no cudaMalloc or cudaFree: with one of each per
+// buffer, five blocking copies, a second build and a graph capture, a call with a
+// new cell took 2.08 ms on a 6,912-atom box and takes 0.37 ms without them.  A
+// geometry that does not fit replaces the allocation with an eighth to spare, and
+// one that needs less than a quarter of a large allocation gives it back.
+struct Arena {
+    char* base = nullptr;
+    size_t cap = 0;
+    cudaError_t reserve(size_t n) {
+        constexpr size_t kLarge = (size_t)256 << 20;
+        if (n <= cap && !(cap > kLarge && n < cap / 4)) return cudaSuccess;
+        release();
+        const size_t want = n + n / 8;
+        cudaError_t e = cudaMalloc((void**)&base, want);
+        if (e == cudaSuccess) {
+            cap = want;
+            return e;
+        }
+        cudaGetLastError();
+        e = cudaMalloc((void**)&base, n);  // without the spare part
+        if (e == cudaSuccess) cap = n;
+        else base = nullptr;
+        return e;
+    }
+    void release() {
+        if (base) cudaFree(base);
+        base = nullptr;
+        cap = 0;
+    }
+};
+
+// Page-locked host memory for the plan upload and the sizing read-back.
+struct Pinned {
+    char* p = nullptr;
+    size_t cap = 0;
+    cudaError_t reserve(size_t n) {
+        if (n <= cap) return cudaSuccess;
+        release();
+        const cudaError_t e = cudaHostAlloc((void**)&p, n + n / 2, cudaHostAllocDefault);
+        if (e == cudaSuccess) cap = n + n / 2;
+        else p = nullptr;
+        return e;
+    }
+    void release() {
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        cap = 0;
+    }
+};
+
 // List layout of a build: the mixed form's forward takes its dispersion pairs
 // from cluster half lists (per-atom lists only within R_cn); the FP64 form, the
 // per-atom virial of Eq. 7 and the backward use full per-atom lists.
@@ -85,14 +139,14 @@ struct Plan {
     std::vector<double> cells;
     std::vector<int32_t> pbc;
     std::vector<StructGeo> geo;
+    std::vector<double> cap_est;  // [2 B] estimated CN and cluster list capacities
     int64_t Nr = 0, ncells = 0, list_disp = 0, list_cn = 0, list_cl = 0, ncl = 0;
     int ghost_cap = 0;
-    DevBuf mem;
+    Arena mem, bwd;  // the plan's buffers; the backward's scratch
+    cudaStream_t stream = nullptr;  // of the last work enqueued on them
     Work w{};
     int* bsum = nullptr;  // scan scratch
     int* gate = nullptr;  // list-reuse gate (device int)
-    double* bwd_scratch = nullptr;
-    int64_t bwd_scratch_n = 0;
     unsigned long long* acc = nullptr;  // fixed-point sums of the cluster-list dispersion pass
     unsigned long long* npairs = nullptr;  // pair count of the cluster-list dispersion pass
     float* vd = nullptr;                // C6 projections (v, dv) per atom of the cluster-list dispersion pass
@@ -139,6 +193,7 @@ struct d3_handle {
     std::string err;
     Plan plan;
     // staging buffers of the host-memory entry point
+    Pinned pin;  // plan upload and sizing read-back
     DevBuf stage;
     size_t stage_atoms = 0, stage_structs = 0;
     double *s_pos = nullptr, *s_E = nullptr, *s_F = nullptr, *s_W = nullptr;
@@ -159,6 +214,9 @@ struct d3_handle {
     int64_t glaunches = 0;         // kernels in the captured call
     const void* gkey[10] = {};     // pointers and generations the graph was captured with
     int64_t plan_gen = 0, param_gen = 0;
+    int64_t last_gen[2] = {-1, -1};  // plan_gen and param_gen of the previous call
+    // list capacities the sizing passes settled on, over plan_geometry's estimates (largest ratio seen)
+    double cap_ratio_cn = 1.0, cap_ratio_cl = 1.0;
     // launch shapes (d3_launch_shapes): chosen per size class by the autotuner unless fixed
     int32_t shape[4] = {kDefaultShape[0], kDefaultShape[1], kDefaultShape[2], kDefaultShape[3]};
     bool autotune = true;
@@ -273,6 +331,11 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
     const double rl = std::max(rld, rln);
     P.geo.assign(B, StructGeo{});
     ghost_est.assign(B, 0.0);
+    P.cap_est.assign(2 * (size_t)B, 0.0);
+    // structures streamed through one handle are alike: start from the ratios of the earlier ones, so
+    // that the sizing pass rarely has to regrow and build again (up to a size where memory matters)
+    const bool learn = offsets[B] <= ((int64_t)1 << 18);
+    const double ratio_cn = learn ? h->cap_ratio_cn : 1.0, ratio_cl = learn ? h->cap_ratio_cl : 1.0;
     int64_t cell_base = 0;
     for (int s = 0; s < B; ++s) {
         StructGeo& G = P.geo[s];
@@ -354,26 +417,31 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
         const double nd = four_thirds_pi * rld * rld * rld * rho, nn = four_thirds_pi * rln * rln * rln * rho;
         const double cap_all = (double)n * vol_factor + 8;
         G.cap_disp = round_cap(std::min(cap_all, std::ceil(1.3 * nd + 32.0)));
-        G.cap_cn = round_cap(std::min(cap_all, std::ceil(1.3 * nn + 16.0)));
+        const double cn_est = std::ceil(1.3 * nn + 16.0), cl_est = std::ceil(4.5 * nd + 64.0);
+        P.cap_est[2 * (size_t)s] = std::min(cap_all, cn_est);
+        P.cap_est[2 * (size_t)s + 1] = std::min(cap_all, cl_est);
+        G.cap_cn = round_cap(std::min(cap_all, std::ceil(ratio_cn * cn_est)));
         // a cluster list holds about half the atoms within the list radius of the
         // cluster's bounding box (regrown by the sizing pass when short)
-        G.cap_cl = round_cap(std::min(cap_all, std::ceil(4.5 * nd + 64.0)));
+        G.cap_cl = round_cap(std::min(cap_all, std::ceil(ratio_cl * cl_est)));
         ghost_est[s] = (double)n * (vol_factor - 1.0);
     }
     P.ncells = cell_base;
     return D3_OK;
 }
 
-// (Re)allocate every device buffer of the plan for the current capacities.
-d3_status plan_alloc(d3_handle* h, Plan& P) {
-    ++h->plan_gen;  // a captured graph refers to the old buffers
-    P.mem.release();
-    P.bwd_scratch = nullptr;
-    P.bwd_scratch_n = 0;
+// Lay out every device buffer of the plan for the current capacities and upload
+// its geometry on st.
+d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
+    ++h->plan_gen;  // a captured graph refers to the old layout
+    // work of earlier calls may still use the memory: calls on st are ordered, another stream's are waited for
+    if (P.mem.base && P.stream != st) {
+        const cudaError_t e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return cuda_fail(h, e, "synchronize before a new layout");
+    }
     const int B = P.B;
     const int64_t Nr = P.Nr, C = P.ncells, Ng = P.ghost_cap, Nt = Nr + Ng;
-    int64_t ld = 0, lc = 0, lcl = 0, ncl = 0;
-    std::vector<int> clu_sid;
+    int64_t ld = 0, lc = 0, lcl = 0, ncl = 0, nfin = 0, maxn = 0;
     for (int s = 0; s < B; ++s) {
         StructGeo& G = P.geo[s];
         G.list_base_disp = ld;
@@ -385,7 +453,9 @@ d3_status plan_alloc(d3_handle* h, Plan& P) {
         G.list_base_cl = lcl;
         ncl += k;
         lcl += k * (int64_t)G.cap_cl;
-        clu_sid.insert(clu_sid.end(), (size_t)k, s);
+        G.fin_base = nfin;
+        nfin += (G.natoms + kFinChunk - 1) / kFinChunk;
+        maxn = std::max<int64_t>(maxn, G.natoms);
     }
     P.list_disp = ld;
     P.list_cn = lc;
@@ -410,96 +480,94 @@ d3_status plan_alloc(d3_handle* h, Plan& P) {
     w.blk_disp = h->shape[1];
     w.blk_chain = h->shape[2];
     w.build_per_sm = h->shape[3];
-    const size_t rs = h->prm.precision == D3_MIXED ? sizeof(float) : sizeof(double);
+    w.max_natoms = maxn;
+    w.n_fin = nfin;
+    const bool mixed = h->prm.precision == D3_MIXED;
+    const size_t rs = mixed ? sizeof(float) : sizeof(double);
     StructGeo* dgeo = nullptr;
     int64_t* doff = nullptr;
-    DevBuf& m = P.mem;
-    cudaError_t e = cudaSuccess;
-#define A(ptr, T, n) \
-    if (e == cudaSuccess) e = m.alloc((T**)&(ptr), (size_t)(n))
-    A(dgeo, StructGeo, B);
-    A(doff, int64_t, B + 1);
-    int* dsid = nullptr;
-    A(dsid, int, Nr);
-    A(w.cnt_real, int, C + 1);
-    A(w.cnt_ghost, int, C + 1);
-    A(w.start_real, int, C + 1);
-    A(w.start_ghost, int, C + 1);
-    A(w.cell_of, int, Nr);
-    A(w.slot_of, int, Nr);
-    A(w.xw, double, 3 * Nr);
-    A(w.ghost_src, int, Ng);
-    A(w.ghost_shift, int, Ng);
-    A(w.ghost_cell, int, Ng);
-    A(w.ghost_slot, int, Ng);
-    A(w.ghost_sid, int, Ng);
-    A(w.ghost_count, int, 1);
-    A(w.sorted_src, int, Nr);
-    A(w.gsorted, int, Ng);
-    A(w.ginv, int, Ng);
-    A(w.gfirst, int, Nr);
-    A(w.gcnt, int, Nr);
-    A(w.usrc, int, Nr + Ng);
-    A(w.ukey, long long, Nr + Ng);
-    A(w.pos64, dbl4, Nt);
-    A(w.rec, float4, 2 * Nt);
-    A(w.hi, float4, Nt);
-    A(w.fw, float, 3 * Nr);
-    A(w.frange, int, 6 * (int64_t)B);
-    A(w.perm, int, Nr);
-    A(w.sid, int, Nr);
-    A(w.cell_sorted, int, Nr);
-    A(w.nbr_disp, int, ld);
-    A(w.nbr_cn, int, lc);
-    A(w.cnt_disp, int, Nr);
-    A(w.cnt_cn, int, Nr);
-    A(w.maxcnt, int, 3 * B);
-    A(w.work_ctr, int, 2);
-    A(w.skey, float, Nr);
-    int* dclu = nullptr;
-    A(dclu, int, std::max<int64_t>(1, ncl));
-    A(w.nbr_cl, int, lcl);
-    A(w.cnt_cl, int, std::max<int64_t>(1, ncl));
-    A(w.acc, unsigned long long, 8 * Nr);
-    A(w.npairs, unsigned long long, 1);
-    // rows of v and dv for real and image atoms (whether images get copies of their
-    // source's rows is decided after the sizing pass, from the image count)
-    if (h->prm.precision == D3_MIXED) A(w.vd, float, Nt * h->T * 2 * h->RP);
-    if (h->prm.precision == D3_MIXED) A(w.gcn, float, lc);
-    A(w.gate, int, 1);
-    A(w.xref, double, 3 * Nr);
-    A(w.wshift, double, 3 * Nr);
-    A(w.cn, double, Nr);
-    A(w.W, char, Nr * h->RP * rs);
-    A(w.dW, char, Nr * h->RP * rs);
-    A(w.v, char, Nr * h->T * h->RP * rs);
-    A(w.dEdn, char, Nr * rs);
-    A(w.Fd, char, Nr * 4 * rs);
-    A(w.eat, double, Nr);
-    A(w.wv, double, 6 * Nr);
-    A(w.Pv, char, Nr * 4 * rs);
-    int64_t maxn = 0;
-    for (int s = 0; s < B; ++s) maxn = std::max<int64_t>(maxn, P.geo[s].natoms);
-    w.max_natoms = maxn;
-    std::vector<int> fin_sid;
-    int64_t nfin = 0;
-    for (int s = 0; s < B; ++s) {
-        P.geo[s].fin_base = nfin;
-        const int64_t k = (P.geo[s].natoms + kFinChunk - 1) / kFinChunk;
-        nfin += k;
-        fin_sid.insert(fin_sid.end(), (size_t)k, s);
-    }
-    w.n_fin = nfin;
-    A(w.fin_part, double, 7 * std::max<int64_t>(1, nfin));
-    int* dfin = nullptr;
-    A(dfin, int, std::max<int64_t>(1, nfin));
-    A(P.bsum, int, scan_scratch_ints(C));
+    int *dsid = nullptr, *dclu = nullptr, *dfin = nullptr;
+    size_t total = 0;
+    // the buffers one after the other from base (nullptr: sizes only), each on a 256-byte boundary
+    auto lay_out = [&](char* base) {
+        size_t off = 0;
+        auto put = [&](auto*& p, size_t n, size_t size) {
+            p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base ? base + off : nullptr);
+            off += (std::max<size_t>(n, 1) * size + 255) & ~(size_t)255;
+        };
+#define A(ptr, T, n) put(ptr, (size_t)(n), sizeof(T))
+        A(dgeo, StructGeo, B);
+        A(doff, int64_t, B + 1);
+        A(dsid, int, Nr);
+        A(w.cnt_real, int, C + 1);
+        A(w.cnt_ghost, int, C + 1);
+        A(w.start_real, int, C + 1);
+        A(w.start_ghost, int, C + 1);
+        A(w.cell_of, int, Nr);
+        A(w.slot_of, int, Nr);
+        A(w.xw, double, 3 * Nr);
+        A(w.ghost_src, int, Ng);
+        A(w.ghost_shift, int, Ng);
+        A(w.ghost_cell, int, Ng);
+        A(w.ghost_slot, int, Ng);
+        A(w.ghost_sid, int, Ng);
+        A(w.maxcnt, int, 3 * (int64_t)B + 1);  // the sizing read-back: list maxima, then the image count
+        w.ghost_count = w.maxcnt ? w.maxcnt + 3 * (int64_t)B : nullptr;
+        A(w.sorted_src, int, Nr);
+        A(w.gsorted, int, Ng);
+        A(w.ginv, int, Ng);
+        A(w.gfirst, int, Nr);
+        A(w.gcnt, int, Nr);
+        A(w.usrc, int, Nr + Ng);
+        A(w.ukey, long long, Nr + Ng);
+        A(w.pos64, dbl4, Nt);
+        A(w.rec, float4, 2 * Nt);
+        A(w.hi, float4, Nt);
+        A(w.fw, float, 3 * Nr);
+        A(w.frange, int, 6 * (int64_t)B);
+        A(w.perm, int, Nr);
+        A(w.sid, int, Nr);
+        A(w.cell_sorted, int, Nr);
+        A(w.nbr_disp, int, ld);
+        A(w.nbr_cn, int, lc);
+        A(w.cnt_disp, int, Nr);
+        A(w.cnt_cn, int, Nr);
+        A(w.work_ctr, int, 2);
+        A(w.skey, float, Nr);
+        A(dclu, int, ncl);
+        A(w.nbr_cl, int, lcl);
+        A(w.cnt_cl, int, ncl);
+        A(w.acc, unsigned long long, 8 * Nr);
+        A(w.npairs, unsigned long long, 1);
+        // rows of v and dv for real and image atoms (whether images get copies of their
+        // source's rows is decided after the sizing pass, from the image count)
+        if (mixed) A(w.vd, float, Nt * h->T * 2 * h->RP);
+        if (mixed) A(w.gcn, float, lc);
+        A(w.gate, int, 1);
+        A(w.xref, double, 3 * Nr);
+        A(w.wshift, double, 3 * Nr);
+        A(w.cn, double, Nr);
+        put(w.W, (size_t)(Nr * h->RP), rs);
+        put(w.dW, (size_t)(Nr * h->RP), rs);
+        put(w.v, (size_t)(Nr * h->T * h->RP), rs);
+        put(w.dEdn, (size_t)Nr, rs);
+        put(w.Fd, (size_t)(Nr * 4), rs);
+        A(w.eat, double, Nr);
+        A(w.wv, double, 6 * Nr);
+        put(w.Pv, (size_t)(Nr * 4), rs);
+        A(w.fin_part, double, 7 * nfin);
+        A(dfin, int, nfin);
+        A(P.bsum, int, scan_scratch_ints(C));
 #undef A
+        total = off;
+    };
+    lay_out(nullptr);
+    cudaError_t e = P.mem.reserve(total);
     if (e != cudaSuccess) {
-        P.mem.release();
         P.valid = false;
         return cuda_fail(h, e, "workspace allocation");
     }
+    lay_out(P.mem.base);
     P.w.status = h->d_status;
     P.w.geo = dgeo;
     P.w.offsets = doff;
@@ -523,18 +591,16 @@ d3_status plan_alloc(d3_handle* h, Plan& P) {
     int* gate = w.gate;
     w.gate = nullptr;  // the plan's own Work builds unconditionally; enqueue_build gates a copy
     P.gate = gate;
-    e = cudaMemcpy(dgeo, P.geo.data(), sizeof(StructGeo) * B, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nfin > 0)
-        e = cudaMemcpy(dfin, fin_sid.data(), sizeof(int) * (size_t)nfin, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(doff, P.offsets.data(), sizeof(int64_t) * (B + 1), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && ncl > 0)
-        e = cudaMemcpy(dclu, clu_sid.data(), sizeof(int) * (size_t)ncl, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && Nr > 0) {
-        std::vector<int> sid((size_t)Nr);
-        for (int s = 0; s < B; ++s)
-            for (int64_t i = P.offsets[s]; i < P.offsets[s + 1]; ++i) sid[(size_t)i] = s;
-        e = cudaMemcpy(dsid, sid.data(), sizeof(int) * (size_t)Nr, cudaMemcpyHostToDevice);
-    }
+    // geometry and offsets through page-locked memory (free again: the sizing pass that follows
+    // every upload waits for the stream); the per-atom and per-cluster indices are formed on the device
+    const size_t ngeo = sizeof(StructGeo) * (size_t)B, noff = sizeof(int64_t) * ((size_t)B + 1);
+    e = h->pin.reserve(ngeo + noff + sizeof(int) * (3 * (size_t)B + 2));
+    if (e != cudaSuccess) return cuda_fail(h, e, "page-locked staging");
+    std::memcpy(h->pin.p, P.geo.data(), ngeo);
+    std::memcpy(h->pin.p + ngeo, P.offsets.data(), noff);
+    e = cudaMemcpyAsync(dgeo, h->pin.p, ngeo, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(doff, h->pin.p + ngeo, noff, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_plan_ids(dgeo, doff, B, Nr, ncl, nfin, dsid, dclu, dfin, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "geometry upload");
     return D3_OK;
 }
@@ -609,6 +675,7 @@ d3_status enqueue_build(d3_handle* h, Plan& P, const double* pos, const int32_t*
     if (P.last_mode != mode) gated = false;
     set_mode(P, mode);
     P.last_mode = mode;
+    P.stream = st;
     Work w = P.w;
     cudaError_t e = cudaSuccess;
     if (gated) {
@@ -710,9 +777,11 @@ d3_status tune_shapes(d3_handle* h, Plan& P, const double* pos, const int32_t* t
 
 // Make the plan match the geometry; on a new geometry run the build once
 // synchronously and grow image and list capacities until nothing overflows.
+// *built: the sizing pass left the lists of these positions (the caller need not build again).
 d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const double* pos, const int32_t* types,
-                      const double* cells, const int32_t* pbc, cudaStream_t st, int mode) {
+                      const double* cells, const int32_t* pbc, cudaStream_t st, int mode, bool* built) {
     Plan& P = h->plan;
+    *built = false;
     if (same_geometry(P, B, offsets, cells, pbc) && P.sized[mode]) return D3_OK;
     if (!same_geometry(P, B, offsets, cells, pbc)) {
         P.valid = false;
@@ -730,22 +799,28 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         for (double x : gest) g += 1.15 * x + 8.0;
         if (g > 2.0e9) return fail(h, D3_ERR_ARG, "too many periodic images");
         P.ghost_cap = (int)g;
-        s = plan_alloc(h, P);
+        s = plan_alloc(h, P, st);
         if (s != D3_OK) return s;
         P.valid = true;
+    }
+    if (P.Nr == 0) {  // no atoms: nothing to build or to measure
+        P.sized[mode] = true;
+        P.last_mode = mode;
+        *built = true;
+        return D3_OK;
     }
     for (int attempt = 0; attempt < 4; ++attempt) {
         cudaError_t e = cudaMemsetAsync(h->d_status, 0, sizeof(int), st);
         if (e != cudaSuccess) return cuda_fail(h, e, "status reset");
         d3_status s = enqueue_build(h, P, pos, types, st, mode);
         if (s != D3_OK) return s;
-        int gcount = 0, status = 0;
-        std::vector<int> mx(3 * (size_t)std::max(B, 1), 0);
-        e = cudaMemcpyAsync(&gcount, P.w.ghost_count, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && B > 0) e = cudaMemcpyAsync(mx.data(), P.w.maxcnt, sizeof(int) * 3 * B, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&status, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
+        int* mx = reinterpret_cast<int*>(h->pin.p + sizeof(StructGeo) * (size_t)B + sizeof(int64_t) * ((size_t)B + 1));
+        e = cudaMemcpyAsync(mx, P.w.maxcnt, sizeof(int) * (3 * (size_t)B + 1), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(mx + 3 * (size_t)B + 1, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(h, e, "sizing pass");
+        const int gcount = mx[3 * (size_t)B], status = mx[3 * (size_t)B + 1];
         if (status & ST_NONFINITE) return fail(h, D3_ERR_NONFINITE, "non-finite coordinate");
         if (status & ST_TYPE) return fail(h, D3_ERR_TYPE, "atom type out of range");
         bool grow = false;
@@ -756,8 +831,14 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         for (int s2 = 0; s2 < B; ++s2) {
             StructGeo& G = P.geo[s2];
             if (mx[3 * s2] > G.cap_disp) { G.cap_disp = round_cap(mx[3 * s2] * 1.1 + 16); grow = true; }
-            if (mx[3 * s2 + 1] > G.cap_cn) { G.cap_cn = round_cap(mx[3 * s2 + 1] * 1.1 + 8); grow = true; }
-            if (mx[3 * s2 + 2] > G.cap_cl) { G.cap_cl = round_cap(mx[3 * s2 + 2] * 1.1 + 16); grow = true; }
+            auto regrow = [&](int n, int32_t& cap, int spare, double est, double& ratio) {
+                if (n <= cap) return;
+                cap = round_cap(n * 1.1 + spare);
+                if (est > 0) ratio = std::min(8.0, std::max(ratio, n * 1.1 / est));
+                grow = true;
+            };
+            regrow(mx[3 * s2 + 1], G.cap_cn, 8, P.cap_est[2 * (size_t)s2], h->cap_ratio_cn);
+            regrow(mx[3 * s2 + 2], G.cap_cl, 16, P.cap_est[2 * (size_t)s2 + 1], h->cap_ratio_cl);
         }
         if (!grow) {
             // image rows of v and dv are copies of their source's when that is cheap
@@ -765,10 +846,11 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
             P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
             set_mode(P, mode);
             P.sized[mode] = true;
+            *built = true;
             return tune_shapes(h, P, pos, types, st, mode);
         }
-        P.sized[0] = P.sized[1] = false;  // the buffers are reallocated: both modes re-measure
-        s = plan_alloc(h, P);
+        P.sized[0] = P.sized[1] = false;  // the buffers are laid out again: both modes re-measure
+        s = plan_alloc(h, P, st);
         if (s != D3_OK) return s;
     }
     return fail(h, D3_ERR_CAPACITY, "workspace sizing did not converge");
@@ -792,9 +874,51 @@ int list_mode(const d3_handle* h, const double* w_atom) {
     return h->prm.precision == D3_MIXED && !w_atom ? kClusterLists : kFullLists;
 }
 
-d3_status forward(d3_handle* h, int32_t B, const int64_t* offsets, const double* pos, const int32_t* types,
-                  const double* cells, const int32_t* pbc, double* E, double* F, double* W, double* e_atom,
-                  double* cn, cudaStream_t st, double* w_atom = nullptr) {
+// Enqueue the build (unless the sizing pass has just run it for these positions)
+// and the passes of a call whose plan is sized.
+d3_status enqueue_forward(d3_handle* h, const double* pos, const int32_t* types, double* E, double* F, double* W,
+                          double* e_atom, double* cn, cudaStream_t st, double* w_atom, int mode, bool built) {
+    Plan& P = h->plan;
+    std::vector<cudaEvent_t> ev;
+    if (h->prof_on) {
+        ev = take_events(h, kEvents);
+        if (ev.size() == kEvents) cudaEventRecord(ev[0], st);
+        built = false;  // a profiled call times its build
+    }
+    if (!built) {
+        const d3_status s = enqueue_build(h, P, pos, types, st, mode, h->prm.skin_A > 0,
+                                          ev.size() == kEvents ? ev.data() + kStages + 1 : nullptr);
+        if (s != D3_OK) return s;
+    }
+    const Consts c = make_consts(h);
+    const bool mixed = h->prm.precision == D3_MIXED;
+    const Tabs tb = forward_tabs(h);
+    cudaError_t e = launch_forward(P.w, c, mixed, tb, E, F, W, e_atom, cn, w_atom, P.B, st,
+                                   ev.size() == kEvents ? ev.data() + 1 : nullptr);
+    if (e != cudaSuccess) return cuda_fail(h, e, "forward launch");
+    h->launches += (P.Nr > 0 ? kForwardLaunches + c.atm + (mode == kClusterLists ? 1 : 0) : 1);
+    if (ev.size() == kEvents) h->ev_pending.push_back(ev);
+    else for (cudaEvent_t x : ev) h->ev_pool.push_back(x);
+    return D3_OK;
+}
+
+// A call on a sized plan is the same sequence of kernels and memsets every time for
+// the same pointers and parameters, so it is captured once as a CUDA graph on an
+// internal stream and then replayed on the caller's stream with one launch.  The
+// first call of a geometry, or of a parameter set, enqueues its kernels directly:
+// capturing and instantiating a graph takes about 100 us of host time and pays only
+// when calls follow one another (a run whose cell changes in every call never gets
+// there).  Calls made while profiling, or while the caller's stream is itself being
+// captured, enqueue directly.
+bool same_key(const void* const (&a)[10], const void* const (&b)[10]) {
+    for (int i = 0; i < 10; ++i)
+        if (a[i] != b[i]) return false;
+    return true;
+}
+
+d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const double* pos, const int32_t* types,
+                        const double* cells, const int32_t* pbc, double* E, double* F, double* W, double* e_atom,
+                        double* cn, cudaStream_t st, double* w_atom) {
     d3_status s = check_batch_args(h, B, offsets, pos, types, cells, pbc);
     if (s != D3_OK) return s;
     if (B > 0 && (!E || !W)) return fail(h, D3_ERR_ARG, "NULL E or W");
@@ -805,78 +929,38 @@ d3_status forward(d3_handle* h, int32_t B, const int64_t* offsets, const double*
     h->last_stream = st;
     if (B == 0) return D3_OK;
     const int mode = list_mode(h, w_atom);
-    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode);
+    bool built = false;
+    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode, &built);
     if (s != D3_OK) return s;
-    Plan& P = h->plan;
-    std::vector<cudaEvent_t> ev;
-    if (h->prof_on) {
-        ev = take_events(h, kEvents);
-        if (ev.size() == kEvents) cudaEventRecord(ev[0], st);
-    }
-    s = enqueue_build(h, P, pos, types, st, mode, h->prm.skin_A > 0,
-                      ev.size() == kEvents ? ev.data() + kStages + 1 : nullptr);
-    if (s != D3_OK) return s;
-    const Consts c = make_consts(h);
-    const bool mixed = h->prm.precision == D3_MIXED;
-    const Tabs tb = forward_tabs(h);
-    cudaError_t e = launch_forward(P.w, c, mixed, tb, E, F, W, e_atom, cn, w_atom, B, st,
-                                   ev.size() == kEvents ? ev.data() + 1 : nullptr);
-    if (e != cudaSuccess) return cuda_fail(h, e, "forward launch");
-    h->launches += (P.Nr > 0 ? kForwardLaunches + c.atm + (mode == kClusterLists ? 1 : 0) : 1);
-    if (ev.size() == kEvents) h->ev_pending.push_back(ev);
-    else for (cudaEvent_t x : ev) h->ev_pool.push_back(x);
-    return D3_OK;
-}
-
-// The steady-state call (sized plan, no profiling) is the same sequence of
-// kernels and memsets every time for the same pointers and parameters, so it
-// is captured once as a CUDA graph on an internal stream and then replayed on
-// the caller's stream with one launch.  Calls made while the caller's stream
-// is itself being captured enqueue directly.
-bool graph_key_match(const d3_handle* h, const void* const (&k)[10]) {
-    if (!h->gexec) return false;
-    for (int i = 0; i < 10; ++i)
-        if (h->gkey[i] != k[i]) return false;
-    return true;
-}
-
-d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const double* pos, const int32_t* types,
-                        const double* cells, const int32_t* pbc, double* E, double* F, double* W, double* e_atom,
-                        double* cn, cudaStream_t st, double* w_atom) {
+    auto direct = [&]() { return enqueue_forward(h, pos, types, E, F, W, e_atom, cn, st, w_atom, mode, built); };
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool direct = !h->graphs || h->prof_on || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
-                        cs != cudaStreamCaptureStatusNone;
-    if (direct || B <= 0 || !offsets || offsets[B] <= 0)
-        return forward(h, B, offsets, pos, types, cells, pbc, E, F, W, e_atom, cn, st, w_atom);
-    d3_status s = check_batch_args(h, B, offsets, pos, types, cells, pbc);
-    if (s != D3_OK) return s;
-    if (!E || !W || !F) return fail(h, D3_ERR_ARG, "NULL E, F or W");
-    const int mode = list_mode(h, w_atom);
-    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode);
-    if (s != D3_OK) return s;
-    h->last_stream = st;
-    // the last build was in the other list mode: rebuild once directly (a
-    // replayed graph would take the list-reuse decision on stale lists)
-    if (h->plan.last_mode != mode)
-        return forward(h, B, offsets, pos, types, cells, pbc, E, F, W, e_atom, cn, st, w_atom);
+    if (!h->graphs || h->prof_on || offsets[B] <= 0 || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
+        cs != cudaStreamCaptureStatusNone)
+        return direct();
     const void* key[10] = {pos, types, E, F, W, e_atom, cn, w_atom, (const void*)(intptr_t)h->plan_gen,
                            (const void*)(intptr_t)(h->param_gen * 2 + (h->accumulate ? 1 : 0))};
-    if (!graph_key_match(h, key)) {
+    const bool again = h->last_gen[0] == h->plan_gen && h->last_gen[1] == h->param_gen;  // as in the previous call
+    h->last_gen[0] = h->plan_gen;
+    h->last_gen[1] = h->param_gen;
+    // (the last build was in the other list mode: rebuild once directly, a
+    // replayed graph would take the list-reuse decision on stale lists)
+    const bool captured_before = h->gexec && same_key(key, h->gkey);
+    if (built || h->plan.last_mode != mode || !(captured_before || again)) return direct();
+    if (!captured_before) {
         if (!h->cap_stream && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
             h->graphs = false;
-            return forward(h, B, offsets, pos, types, cells, pbc, E, F, W, e_atom, cn, st, w_atom);
+            return direct();
         }
         // the captured work must start after everything already on the caller's stream
         cudaGraph_t g = nullptr;
         const int64_t before = h->launches;
         cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            s = forward(h, B, offsets, pos, types, cells, pbc, E, F, W, e_atom, cn, h->cap_stream, w_atom);
+            s = enqueue_forward(h, pos, types, E, F, W, e_atom, cn, h->cap_stream, w_atom, mode, false);
             e = cudaStreamEndCapture(h->cap_stream, &g);
         }
         const int64_t captured = h->launches - before;
         h->launches = before;
-        h->last_stream = st;
         cudaGraphExec_t x = nullptr;
         if (e == cudaSuccess && s == D3_OK && g) e = cudaGraphInstantiate(&x, g, 0);
         if (g) cudaGraphDestroy(g);
@@ -884,13 +968,14 @@ d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const d
             cudaGetLastError();
             if (x) cudaGraphExecDestroy(x);
             h->graphs = false;  // fall back to direct enqueueing for this handle
-            return forward(h, B, offsets, pos, types, cells, pbc, E, F, W, e_atom, cn, st, w_atom);
+            return direct();
         }
         if (h->gexec) cudaGraphExecDestroy(h->gexec);
         h->gexec = x;
         h->glaunches = captured;
         for (int i = 0; i < 10; ++i) h->gkey[i] = key[i];
     }
+    h->plan.stream = st;
     cudaError_t e = cudaGraphLaunch(h->gexec, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "graph launch");
     h->launches += h->glaunches;
@@ -1028,6 +1113,8 @@ void d3_destroy(d3_handle* h) {
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     h->plan.mem.release();
+    h->plan.bwd.release();
+    h->pin.release();
     h->stage.release();
     h->tabmem.release();
     if (h->h_status) cudaFreeHost(h->h_status);
@@ -1038,6 +1125,7 @@ d3_status d3_set_damping(d3_handle* h, double s6, double s8, double a1, double a
     if (!h) return D3_ERR_ARG;
     if (!std::isfinite(s6) || !std::isfinite(s8) || !std::isfinite(a1) || !std::isfinite(a2_bohr))
         return fail(h, D3_ERR_ARG, "non-finite damping parameter");
+    if (s6 == h->prm.s6 && s8 == h->prm.s8 && a1 == h->prm.a1 && a2_bohr == h->prm.a2_bohr) return D3_OK;
     if (h->last_stream) cudaStreamSynchronize(h->last_stream);
     h->prm.s6 = s6;
     h->prm.s8 = s8;
@@ -1110,9 +1198,10 @@ d3_status d3_build_neighbors(d3_handle* h, int32_t B, const int64_t* offsets, co
     h->last_stream = st;
     if (B == 0) return D3_OK;
     const int mode = list_mode(h, nullptr);
-    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode);
+    bool built = false;
+    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode, &built);
     if (s != D3_OK) return s;
-    s = enqueue_build(h, h->plan, pos, types, st, mode);
+    if (!built) s = enqueue_build(h, h->plan, pos, types, st, mode);
     if (s != D3_OK) return s;
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(h, e, "build");
@@ -1219,18 +1308,16 @@ d3_status d3_backward(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         }
         return D3_OK;
     }
-    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, kFullLists);
+    bool built = false;
+    s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, kFullLists, &built);
     if (s != D3_OK) return s;
     Plan& P = h->plan;
-    s = enqueue_build(h, P, pos, types, st, kFullLists);
+    if (!built) s = enqueue_build(h, P, pos, types, st, kFullLists);
     if (s != D3_OK) return s;
-    const int64_t need = backward_scratch_doubles(P.w, B);
-    if (need > P.bwd_scratch_n) {
-        double* p = nullptr;
-        cudaError_t e = P.mem.alloc(&p, (size_t)need);
+    const size_t need = (size_t)backward_scratch_doubles(P.w, B) * sizeof(double);
+    if (need > P.bwd.cap) {  // (otherwise kept: a captured call must not lose the memory it refers to)
+        const cudaError_t e = P.bwd.reserve(need);
         if (e != cudaSuccess) return cuda_fail(h, e, "backward scratch");
-        P.bwd_scratch = p;
-        P.bwd_scratch_n = need;
     }
     Consts c = make_consts(h);
     Tabs tbm{};  // FP32 tables of the mixed form
@@ -1241,7 +1328,7 @@ d3_status d3_backward(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     tbm.cnref2 = h->d_cnref2;
     tbm.dcr = h->d_dcr;
     cudaError_t e = launch_backward(P.w, c, h->d_c6d, h->d_pairb, h->d_cnref, h->d_nref, tbm, dLdE, dLdF, dLdparams,
-                                    dLdpos, P.bwd_scratch, B, h->prm.precision == D3_MIXED, st);
+                                    dLdpos, reinterpret_cast<double*>(P.bwd.base), B, h->prm.precision == D3_MIXED, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "backward launch");
     return D3_OK;
 }

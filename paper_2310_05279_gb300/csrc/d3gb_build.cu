@@ -909,6 +909,34 @@ cudaError_t launch_build_impl(const Work& w, const double* pos, const int32_t* t
     return cudaGetLastError();
 }
 
+// Structure of every atom, cluster and chunk of the per-structure sums.
+__global__ void __launch_bounds__(256) k_plan_ids(const StructGeo* __restrict__ geo, const int64_t* __restrict__ off, int B,
+                                                  int64_t Nr, int64_t ncl, int64_t nfin, int* __restrict__ sid_in,
+                                                  int* __restrict__ clu_sid, int* __restrict__ fin_sid) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < Nr) sid_in[i] = struct_of(off, B, i);
+    if (i >= ncl && i >= nfin) return;
+    // the last structure whose clusters (chunks) begin at or before i: empty structures own none
+    int lo = 0, hi = B, lf = 0, hf = B;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (geo[mid].clu_base <= i) lo = mid; else hi = mid;
+    }
+    while (hf - lf > 1) {
+        const int mid = (lf + hf) >> 1;
+        if (geo[mid].fin_base <= i) lf = mid; else hf = mid;
+    }
+    if (i < ncl) clu_sid[i] = lo;
+    if (i < nfin) fin_sid[i] = lf;
+}
+
+cudaError_t launch_plan_ids(const StructGeo* geo, const int64_t* offsets, int B, int64_t Nr, int64_t ncl, int64_t nfin,
+                            int* sid_in, int* clu_sid, int* fin_sid, cudaStream_t st) {
+    // (a structure has at least one atom per cluster and per chunk: Nr threads cover all three)
+    if (Nr > 0) k_plan_ids<<<nblk(Nr, 256), 256, 0, st>>>(geo, offsets, B, Nr, ncl, nfin, sid_in, clu_sid, fin_sid);
+    return cudaGetLastError();
+}
+
 int64_t scan_scratch_ints(int64_t ncells) { return 2 * nblk(ncells, kScanBlock) + 2; }
 
 cudaError_t launch_check(const Work& w, const double* pos, cudaStream_t st) {
