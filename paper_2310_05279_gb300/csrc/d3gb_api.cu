@@ -150,6 +150,7 @@ struct Plan {
     unsigned long long* acc = nullptr;  // fixed-point sums of the cluster-list dispersion pass
     unsigned long long* npairs = nullptr;  // pair count of the cluster-list dispersion pass
     float* vd = nullptr;                // C6 projections (v, dv) per atom of the cluster-list dispersion pass
+    int split_on = 0;                   // some cluster's list is longer than w.split_min
     int vd_images = 0;                  // image atoms have rows of vd of their own (cluster lists only)
 };
 
@@ -160,6 +161,7 @@ void set_mode(Plan& P, int mode) {
     P.w.npairs = mode == kClusterLists ? P.npairs : nullptr;
     P.w.vd = mode == kClusterLists ? P.vd : nullptr;
     P.w.vd_images = mode == kClusterLists ? P.vd_images : 0;  // without vd there are no rows to copy
+    P.w.split_on = P.split_on;
 }
 
 }  // namespace
@@ -482,6 +484,11 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     w.build_per_sm = h->shape[3];
     w.max_natoms = maxn;
     w.n_fin = nfin;
+    // Lists longer than this are split over a block (k_disp_cl_split) where clusters are few: 64
+    // entries (one chunk) when every warp of the chip could take a part, up to 1024 while a single
+    // long list can outlast the rest (6,912-atom box, 864 clusters, lists of 471 entries on average
+    // and 2,258 at most: 372 us unsplit, 309 from 142 entries on, 296 from 473 on).
+    w.split_min = (int)std::min<int64_t>(1024, std::max<int64_t>(64, ncl * 333 / (4 * (int64_t)w.num_sms)));
     const bool mixed = h->prm.precision == D3_MIXED;
     const size_t rs = mixed ? sizeof(float) : sizeof(double);
     StructGeo* dgeo = nullptr;
@@ -532,11 +539,12 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
         A(w.nbr_cn, int, lc);
         A(w.cnt_disp, int, Nr);
         A(w.cnt_cn, int, Nr);
-        A(w.work_ctr, int, 2);
+        A(w.work_ctr, int, 3);
         A(w.skey, float, Nr);
         A(dclu, int, ncl);
         A(w.nbr_cl, int, lcl);
         A(w.cnt_cl, int, ncl);
+        A(w.split_q, int, ncl);
         A(w.acc, unsigned long long, 8 * Nr);
         A(w.npairs, unsigned long long, 1);
         // rows of v and dv for real and image atoms (whether images get copies of their
@@ -844,6 +852,12 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
             // image rows of v and dv are copies of their source's when that is cheap
             // (few images, or few types); otherwise the pass resolves each image's source
             P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
+            if (mode == kClusterLists) {
+                P.split_on = 0;
+                // (with more clusters the long lists hide behind the others, and leaving them out costs 2%)
+                if (P.ncl <= 128 * (int64_t)P.w.num_sms)
+                    for (int s2 = 0; s2 < B; ++s2) P.split_on |= mx[3 * s2 + 2] > P.w.split_min ? 1 : 0;
+            }
             set_mode(P, mode);
             P.sized[mode] = true;
             *built = true;

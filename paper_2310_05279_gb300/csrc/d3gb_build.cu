@@ -400,6 +400,7 @@ __global__ void k_reset(Work w) {
         *w.ghost_count = 0;
         w.work_ctr[0] = 0;
         w.work_ctr[1] = 0;
+        w.work_ctr[2] = 0;
         atomicAdd(w.nbuild, 1ull);
     }
 }
@@ -853,6 +854,7 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
             }
         if (lane == 0) {
             w.cnt_cl[I] = min(n, cap);
+            if (min(n, cap) > w.split_min) w.split_q[atomicAdd(w.work_ctr + 2, 1)] = (int)I;
             if (n > cap || mc > capc) atomicOr(w.status, ST_LIST_CAP);
             atomicMax(&w.maxcnt[3 * s + 2], n);
             atomicMax(&w.maxcnt[3 * s + 1], mc);

@@ -84,10 +84,17 @@ __device__ __forceinline__ void load_j(const Work& w, const float* __restrict__ 
     load_vec<R>(r + (R <= 4 ? 4 : 8), J.dv);
 }
 
+// Split form: the steps of one chunk (16) of the force terms on i, and the chunk's
+// partial sums (dE/dn_i, energy, virial), one float per lane each.
+constexpr int kChunkSteps = 16;
+constexpr int kSplitForce = kChunkSteps * 3 * 32;
+constexpr int kSplitFloats = kSplitForce + 8 * 32;  // per warp
+
 // The lane's i atom and its running sums.  step2() evaluates two steps (8 i atoms x
 // 4 list entries each) written as one block, so that their dependency chains
-// interleave.
-template <int R, bool SITE>
+// interleave.  SPLIT: the warp evaluates single chunks of the list, and the force
+// terms of each step are left in fbuf, to be subtracted in list order by one warp.
+template <int R, bool SITE, bool SPLIT>
 struct ClusterPass {
     Site<true> S;
     float Wi[R], dWi[R];
@@ -99,6 +106,7 @@ struct ClusterPass {
     unsigned long long* acc;
     bool bad = false;     // a fixed-point value out of range (ST_SUM_RANGE at the end)
     unsigned npairs = 0;  // used pairs of the warp (warp-uniform)
+    float* fbuf = nullptr;  // SPLIT: the lane's slots of the chunk
     // running sums of the lane's i
     float fx = 0.f, fy = 0.f, fz = 0.f;
     float dnc = 0.f, dnh = 0.f, dnl = 0.f;            // dE/dn_i: chunk partial and compensated sum
@@ -132,7 +140,7 @@ struct ClusterPass {
 
     // pair terms of a used pair (zero weight otherwise) and the i-side sums; returns
     // the j-side values: force on j (nt), dE/dn_j, energy share
-    __device__ __forceinline__ void pair(const JData<R>& J, float dx, float dy, float dz, float r2, bool use,
+    __device__ __forceinline__ void pair(const JData<R>& J, int step, float dx, float dy, float dz, float r2, bool use,
                                          float& ntx, float& nty, float& ntz, float& dnj, float& e) {
         const float4 tb = trow[__float_as_int(J.h.w) & 15];
         float C6 = 0.f, dC6i = 0.f, dC6j = 0.f;
@@ -152,7 +160,12 @@ struct ClusterPass {
         // F_i = -(de/dr) d/r = -nfc d, nfc = -C6 (6 r^4 t6 i6 + 8 r^6 t8 i8); the force on j is nfc d
         const float nfc = use ? -C6 * fmaf(6.0f * r4, t6 * i6, 8.0f * r6 * (t8 * i8)) : 0.f;
         ntx = nfc * dx; nty = nfc * dy; ntz = nfc * dz;
-        fx -= ntx; fy -= nty; fz -= ntz;
+        if constexpr (SPLIT) {
+            float* f = fbuf + step * 96;
+            f[0] = ntx; f[32] = nty; f[64] = ntz;
+        } else {
+            fx -= ntx; fy -= nty; fz -= ntz;
+        }
         dnc = fmaf(mg, dC6i, dnc);
         ec += e;
         sv[0] = fmaf(ntx, dx, sv[0]); sv[1] = fmaf(nty, dy, sv[1]); sv[2] = fmaf(ntz, dz, sv[2]);
@@ -199,7 +212,8 @@ struct ClusterPass {
         red_add_if((um >> fshift) & 0xffu, acc + 8 * (int64_t)(tsq >> 4) + 2 * b0 + b1, x);
     }
 
-    __device__ __forceinline__ void step2(const JData<R>& A, const JData<R>& B) {
+    // (step: place of A in its chunk, used by SPLIT)
+    __device__ __forceinline__ void step2(const JData<R>& A, const JData<R>& B, int step) {
         float ax, ay, az, ar2, bx, by, bz, br2;
         bool ause, anear, buse, bnear;
         pair_vec(A, ax, ay, az, ar2, ause, anear);
@@ -209,11 +223,17 @@ struct ClusterPass {
             if (bnear) buse = S.inside(B.q, br2, rc2, rc2d);
         }
         const unsigned uma = __ballot_sync(0xffffffffu, ause), umb = __ballot_sync(0xffffffffu, buse);
-        if ((uma | umb) == 0u) return;
+        if ((uma | umb) == 0u) {
+            if constexpr (SPLIT) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) fbuf[step * 96 + 32 * k] = 0.f;
+            }
+            return;
+        }
         npairs += __popc(uma) + __popc(umb);
         float atx, aty, atz, adn, ae, btx, bty, btz, bdn, be;
-        pair(A, ax, ay, az, ar2, ause, atx, aty, atz, adn, ae);
-        pair(B, bx, by, bz, br2, buse, btx, bty, btz, bdn, be);
+        pair(A, step, ax, ay, az, ar2, ause, atx, aty, atz, adn, ae);
+        pair(B, step + 1, bx, by, bz, br2, buse, btx, bty, btz, bdn, be);
         if constexpr (SITE) {
             flush_j(__float_as_int(A.h.w), uma, atx, aty, atz, adn, ae);
             flush_j(__float_as_int(B.h.w), umb, btx, bty, btz, bdn, be);
@@ -224,11 +244,164 @@ struct ClusterPass {
     }
 };
 
+// The lane's part of cluster I: its atom (il = lane % 8) and the row of its list.
+struct ClusterRow {
+    int64_t p0, p;
+    bool ilive;
+    const int* row;
+    int cnt;
+};
+
+template <int R, bool SITE, bool SPLIT>
+__device__ __forceinline__ ClusterRow cluster_row(const Work& w, int64_t I, int il) {
+    ClusterRow C;
+    const StructGeo& G = w.geo[w.clu_sid[I]];
+    C.p0 = G.atom_base + (I - G.clu_base) * kClusterAtoms;
+    const int64_t rem = G.atom_base + G.natoms - C.p0;
+    const int nI = rem < kClusterAtoms ? (int)rem : kClusterAtoms;
+    C.ilive = il < nI;
+    C.p = C.p0 + (C.ilive ? il : 0);  // lanes past the cluster's end mirror its first atom, unused
+    C.row = w.nbr_cl + G.list_base_cl + (I - G.clu_base) * (int64_t)G.cap_cl;
+    C.cnt = w.cnt_cl[I];
+    return C;
+}
+
+template <int R, bool SITE, bool SPLIT>
+__device__ __forceinline__ void cluster_setup(ClusterPass<R, SITE, SPLIT>& P, const Work& w, const Consts& c,
+                                              const ClusterRow& C, const float4* tab, int lane) {
+    const int ti = P.S.tsrc() & 15;
+    load_vec<R>((const float*)w.W + C.p * c.RP, P.Wi);
+    load_vec<R>((const float*)w.dW + C.p * c.RP, P.dWi);
+    P.trow = tab + ti * c.T;
+    P.pthr = C.ilive ? (int)C.p : 0x7fffffff;
+    P.rc2 = c.rc_disp2f;
+    P.band = 4e-6f * c.rc_disp2f;  // FP32 error band of the cutoff test (as Site::inside)
+    P.rc2d = c.rc_disp2;
+    P.b0 = lane & 1;
+    P.b1 = (lane >> 1) & 1;
+    P.il = lane & 7;
+    P.fshift = lane & 24;
+    P.acc = w.acc;
+}
+
+// Blocks [b0, b1) of the list (8 steps each).  List entries of steps 8b..8b+7 come from
+// one coalesced load, lane k holding entry 32b + k, together with the entry's source
+// atom (itself for a real atom; with IMGSRC, an image's source from its compact
+// record), a block ahead.  The neighbour data of the next two steps is loaded while two
+// steps compute.  Whole blocks are processed: entries past the end of the list are -1
+// (unused).
+template <int R, bool SITE, bool IMGSRC, bool SPLIT>
+__device__ __forceinline__ void cluster_blocks(ClusterPass<R, SITE, SPLIT>& P, const Work& w, const Consts& c,
+                                               const ClusterRow& C, int lane, int b0, int b1) {
+    constexpr int RPc = R <= 4 ? 4 : 8;
+    const int js = lane >> 3;
+    const int rows = c.T * 2 * RPc;                         // floats of v/dv rows per atom
+    const float* vdb = w.vd + (P.S.tsrc() & 15) * 2 * RPc;  // the rows for partner type t_i
+    const int end = SPLIT ? min(C.cnt, 32 * b1) : C.cnt;
+    const int nr = (int)w.Nr;
+    auto src_of = [&](int q) { return IMGSRC && q >= nr ? (__float_as_int(__ldg(&w.hi[q].w)) >> 4) : q; };
+    auto entry = [&](int k) { return k < end ? __ldg(C.row + k) : -1; };
+    int qa = entry(32 * b0 + lane);
+    int qb = entry(32 * b0 + 32 + lane);
+    int sa = src_of(qa), sb = src_of(qb);
+    // this lane's entry of step s (0..7) of the current block
+    auto load = [&](int st, JData<R>& J) {
+        const int from = (st << 2) + js;
+        const int q = __shfl_sync(0xffffffffu, qa, from);
+        const int src = IMGSRC ? __shfl_sync(0xffffffffu, sa, from) : q;
+        load_j<R>(w, vdb, rows, q, src, J);
+    };
+    JData<R> A, B, CC, D;
+    load(0, A);
+    load(1, B);
+    for (int b = b0; b < b1; ++b) {
+        const int s0 = (b & 1) * 8;
+        load(2, CC);
+        load(3, D);
+        P.step2(A, B, s0);
+        load(4, A);
+        load(5, B);
+        P.step2(CC, D, s0 + 2);
+        load(6, CC);
+        load(7, D);
+        P.step2(A, B, s0 + 4);
+        // next block: its entries become current, the one after is loaded
+        qa = qb;
+        sa = sb;
+        qb = entry(32 * (b + 2) + lane);
+        sb = src_of(qb);
+        load(0, A);
+        load(1, B);
+        P.step2(CC, D, s0 + 6);
+        if (!SPLIT && (b & 1)) P.chunk();  // every 16 steps
+    }
+}
+
+// The cluster's sums, held by one warp: the i side summed over the 4 lanes of each i
+// (fixed order) and added to the accumulators, then the virial and (without SITE) the
+// energy, -sum_pairs fc d (x) d (the partials are of nfc d (x) d): compensated float
+// pairs summed over the warp in a fixed order, then lane m converts value m to FP64
+// (one conversion for all seven: the FP64 pipe takes a whole warp instruction however
+// few lanes are active) and writes it on the cluster's first atom; zero on the others.
+template <int R, bool SITE, bool SPLIT>
+__device__ __forceinline__ void cluster_finish(ClusterPass<R, SITE, SPLIT>& P, const Work& w, const ClusterRow& C,
+                                               int lane) {
+    const int il = lane & 7, js = lane >> 3;
+    float fx = P.fx, fy = P.fy, fz = P.fz, dnh = P.dnh, dnl = P.dnl, Eh = P.Eh, El = P.El;
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        fx += __shfl_xor_sync(0xffffffffu, fx, o);
+        fy += __shfl_xor_sync(0xffffffffu, fy, o);
+        fz += __shfl_xor_sync(0xffffffffu, fz, o);
+        dnh += __shfl_xor_sync(0xffffffffu, dnh, o);
+        dnl += __shfl_xor_sync(0xffffffffu, dnl, o);
+        if (SITE) {
+            Eh += __shfl_xor_sync(0xffffffffu, Eh, o);
+            El += __shfl_xor_sync(0xffffffffu, El, o);
+        }
+    }
+    if (js == 0 && C.ilive) {
+        unsigned long long* ai = w.acc + 8 * C.p;
+        red_add(ai + 0, fix40(fx, P.bad));
+        red_add(ai + 1, fix40(fy, P.bad));
+        red_add(ai + 2, fix40(fz, P.bad));
+        red_add(ai + 3, fix40(dnh, P.bad) + fix40(dnl, P.bad));
+        if (SITE) red_add(ai + 4, fix40(Eh, P.bad) + fix40(El, P.bad));
+    }
+    float hm = 0.f, lm = 0.f;
+#pragma unroll
+    for (int m = 0; m < 7; ++m) {
+        if (m == 6 && SITE) break;
+        float h = m < 6 ? P.Vh[m] : P.Eh, l = m < 6 ? P.Vl[m] : P.El;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            h += __shfl_xor_sync(0xffffffffu, h, o);
+            l += __shfl_xor_sync(0xffffffffu, l, o);
+        }
+        if (lane == m) {
+            hm = h;
+            lm = l;
+        }
+    }
+    const double Vm = (double)hm + (double)lm;
+    if (lane < 6) w.wv[6 * C.p0 + lane] = Vm;
+    if (!SITE && lane == 6) w.eat[C.p0] = Vm;
+    if (js == 0 && C.ilive && il > 0) {
+        double* wv = w.wv + 6 * C.p;
+#pragma unroll
+        for (int m = 0; m < 6; ++m) wv[m] = 0.0;
+        if (!SITE) w.eat[C.p] = 0.0;
+    }
+}
+
 // IMGSRC: image atoms have no rows of their own; each list entry's source atom is
 // resolved once per block of 32 entries (from the image's compact record).
 // The bound (128, 3) holds every instantiation to 168 registers, so that three
 // 128-thread blocks (12 warps) stay resident per SM whatever R is.
-template <int R, bool SITE, bool IMGSRC>
+// BESIDE: clusters with more than w.split_min entries are left to k_disp_cl_split, which
+// runs at the same time: this kernel is launched without waiting for it and waits before
+// it ends, so that what follows sees both.
+template <int R, bool SITE, bool IMGSRC, bool BESIDE>
 __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const float4* __restrict__ pair_tab) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* tab = reinterpret_cast<float4*>(smem_raw);
@@ -244,7 +417,7 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
     const int nI = rem < kClusterAtoms ? (int)rem : kClusterAtoms;
     const bool ilive = il < nI;
     const int64_t p = p0 + (ilive ? il : 0);  // lanes past the cluster's end mirror its first atom, unused
-    ClusterPass<R, SITE> P(w, p);
+    ClusterPass<R, SITE, false> P(w, p);
     const int ti = P.S.tsrc() & 15;
     load_vec<R>((const float*)w.W + p * c.RP, P.Wi);
     load_vec<R>((const float*)w.dW + p * c.RP, P.dWi);
@@ -263,6 +436,10 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
     const float* vdb = w.vd + ti * 2 * RPc;  // the rows for partner type t_i
     const int* row = w.nbr_cl + G.list_base_cl + (I - G.clu_base) * (int64_t)G.cap_cl;
     const int cnt = w.cnt_cl[I];
+    if (BESIDE && cnt > w.split_min) {
+        grid_dependency_wait();
+        return;
+    }
     const int nsteps = (cnt + 3) >> 2;
     // list entries of steps 8b..8b+7 (block b) come from one coalesced load, lane k
     // holding entry 32b + k, together with the entry's source atom (itself for a real
@@ -288,13 +465,13 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
     for (int b = 0; b < nblocks; ++b) {
         load(2, C);
         load(3, D);
-        P.step2(A, B);
+        P.step2(A, B, 0);
         load(4, A);
         load(5, B);
-        P.step2(C, D);
+        P.step2(C, D, 0);
         load(6, C);
         load(7, D);
-        P.step2(A, B);
+        P.step2(A, B, 0);
         // next block: its entries become current, the one after is loaded
         qa = qb;
         sa = sb;
@@ -303,7 +480,7 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
         sb = src_of(qb);
         load(0, A);
         load(1, B);
-        P.step2(C, D);
+        P.step2(C, D, 0);
         if (b & 1) P.chunk();  // every 16 steps
     }
     P.chunk();
@@ -361,6 +538,102 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
         for (int m = 0; m < 6; ++m) wv[m] = 0.0;
         if (!SITE) w.eat[p] = 0.0;
     }
+    if (BESIDE) grid_dependency_wait();
+}
+
+// One block per cluster with more than w.split_min entries (the list builder queues
+// them): its warps take the list's chunks of 16 steps in turn, and the sums are then
+// formed chunk by chunk in list order, so every result is the one that a single warp
+// would give, bit for bit.  A chunk takes a warp about 4 us whatever else runs, so a
+// list of thousands of entries (a cluster in a sparse row at the edge of the occupied
+// cells spans the whole row) or a batch of few clusters is bound by that chain: the
+// dispersion stage of a 6,912-atom box took 153 us and takes 92, a batch of 64
+// structures (63,709 atoms) 277 us and 190.
+template <int R, bool SITE, bool IMGSRC>
+__global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, const float4* __restrict__ pair_tab) {
+    grid_dependency_launch();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float4* tab = reinterpret_cast<float4*>(smem_raw);
+    float* buf = reinterpret_cast<float*>(tab + c.T * c.T);
+    for (int k = threadIdx.x; k < c.T * c.T; k += blockDim.x) tab[k] = pair_tab[k];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nq = w.work_ctr[2];
+    for (int k = blockIdx.x; k < nq; k += gridDim.x) {
+        const ClusterRow C = cluster_row<R, SITE, true>(w, w.split_q[k], lane & 7);
+        ClusterPass<R, SITE, true> P(w, C.p);
+        cluster_setup(P, w, c, C, tab, lane);
+        const int nblocks = (C.cnt + 31) >> 5, nchunks = (nblocks + 1) >> 1;
+        float* mine = buf + wid * kSplitFloats + lane;
+        for (int c0 = 0; c0 < nchunks; c0 += nw) {
+            const int ch = c0 + wid;
+            if (ch < nchunks) {
+                P.fbuf = mine;
+                P.dnc = P.ec = 0.f;
+#pragma unroll
+                for (int m = 0; m < 6; ++m) P.sv[m] = 0.f;
+                const int b1 = min(nblocks, 2 * ch + 2);
+                cluster_blocks<R, SITE, IMGSRC, true>(P, w, c, C, lane, 2 * ch, b1);
+                if (b1 == 2 * ch + 1)  // the last chunk has 8 steps
+#pragma unroll
+                    for (int s = 8 * 3; s < kChunkSteps * 3; ++s) mine[s * 32] = 0.f;
+                float* q = mine + kSplitForce;
+                q[0] = P.dnc;
+                q[32] = P.ec;
+#pragma unroll
+                for (int m = 0; m < 6; ++m) q[64 + 32 * m] = P.sv[m];
+            }
+            __syncthreads();
+            // warp t = 0, 1, 2 adds force component t and some of the other sums, chunk by chunk
+            if (wid < 3) {
+                const int n = min(nw, nchunks - c0);
+                for (int r = 0; r < n; ++r) {
+                    const float* f = buf + r * kSplitFloats + 32 * wid + lane;
+                    float x = P.fx;
+#pragma unroll
+                    for (int s = 0; s < kChunkSteps; ++s) x = __fsub_rn(x, f[s * 96]);
+                    P.fx = x;
+                    const float* q = buf + r * kSplitFloats + kSplitForce + lane;
+                    if (wid == 0) {
+                        acc_add(P.dnh, P.dnl, q[0]);
+                        acc_add(P.Eh, P.El, q[32]);
+                    } else {
+                        const float* v = q + 64 + 96 * (wid - 1);
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) acc_add(P.Vh[m], P.Vl[m], v[32 * m]);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+        // everything to warp 0
+        if (wid == 1 || wid == 2) {
+            float* o = buf + wid * kSplitFloats + lane;
+            o[0] = P.fx;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                o[32 + 64 * m] = P.Vh[m];
+                o[64 + 64 * m] = P.Vl[m];
+            }
+        }
+        __syncthreads();
+        if (wid == 0) {
+            const float *o1 = buf + kSplitFloats + lane, *o2 = buf + 2 * kSplitFloats + lane;
+            P.fy = o1[0];
+            P.fz = o2[0];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                P.Vh[m] = o1[32 + 64 * m];
+                P.Vl[m] = o1[64 + 64 * m];
+                P.Vh[3 + m] = o2[32 + 64 * m];
+                P.Vl[3 + m] = o2[64 + 64 * m];
+            }
+            cluster_finish(P, w, C, lane);
+        }
+        if (lane == 0 && w.npairs) atomicAdd(w.npairs, (unsigned long long)P.npairs);
+        if (P.bad) atomicOr(w.status, ST_SUM_RANGE);
+        __syncthreads();  // the buffer is reused by the next cluster
+    }
 }
 
 // Per atom: the fixed-point totals of the dispersion pass into the arrays the
@@ -388,15 +661,30 @@ cudaError_t launch_disp_cl(const Work& w, const Consts& c, const void* pair_tab,
         const int TB = w.blk_disp;  // 64 or 128 threads: 2 or 4 clusters per block
         const unsigned grid = nblk(w.ncl, TB / 32);
         const size_t sm = (size_t)c.T * c.T * sizeof(float4);
+        const int nw = w.ncl <= w.num_sms ? 8 : 4;  // fewer clusters than SMs: more warps for each
+        const size_t sms = sm + (size_t)nw * kSplitFloats * sizeof(float);
+        const unsigned gs = (unsigned)(w.ncl < 8 * (int64_t)w.num_sms ? w.ncl : 8 * (int64_t)w.num_sms);
         const float4* pt = (const float4*)pair_tab;
-#define D3_CL(RR)                                                                  \
-    if (w.vd_images) {                                                             \
-        if (site) k_disp_cl<RR, true, false><<<grid, TB, sm, st>>>(w, c, pt);     \
-        else k_disp_cl<RR, false, false><<<grid, TB, sm, st>>>(w, c, pt);         \
-    } else {                                                                       \
-        if (site) k_disp_cl<RR, true, true><<<grid, TB, sm, st>>>(w, c, pt);      \
-        else k_disp_cl<RR, false, true><<<grid, TB, sm, st>>>(w, c, pt);          \
-    }                                                                              \
+        cudaError_t e = cudaSuccess;
+#define D3_CL1(RR, S, I)                                                                                   \
+    {                                                                                                      \
+        if (w.split_on) {                                                                                  \
+            e = cudaFuncSetAttribute(k_disp_cl_split<RR, S, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms); \
+            if (e != cudaSuccess) return e;                                                                \
+            k_disp_cl_split<RR, S, I><<<gs, 32 * nw, sms, st>>>(w, c, pt);                                 \
+            e = launch_overlapped(k_disp_cl<RR, S, I, true>, grid, TB, sm, st, w, c, pt);                         \
+        } else {                                                                                           \
+            k_disp_cl<RR, S, I, false><<<grid, TB, sm, st>>>(w, c, pt);                                           \
+        }                                                                                                  \
+    }
+#define D3_CL(RR)                                  \
+    if (w.vd_images) {                             \
+        if (site) D3_CL1(RR, true, false)          \
+        else D3_CL1(RR, false, false)              \
+    } else {                                       \
+        if (site) D3_CL1(RR, true, true)           \
+        else D3_CL1(RR, false, true)               \
+    }                                              \
     break
         switch (c.R) {
             case 1: D3_CL(1);
@@ -408,6 +696,8 @@ cudaError_t launch_disp_cl(const Work& w, const Consts& c, const void* pair_tab,
             default: D3_CL(7);
         }
 #undef D3_CL
+#undef D3_CL1
+        if (e != cudaSuccess) return e;
     }
     k_disp_fin<<<nblk(w.Nr, 256), 256, 0, st>>>(w, site ? 1 : 0);
     return cudaGetLastError();

@@ -152,13 +152,16 @@ struct Work {
     int* cnt_disp;           // [Nr]
     int* cnt_cn;             // [Nr]
     int* maxcnt;             // [3*B] max list length per structure (disp, cn, cluster)
-    int* work_ctr;           // [2] persistent-kernel work counters (zeroed before each build)
+    int* work_ctr;           // [3] persistent-kernel work counters, length of split_q (zeroed before each build)
     // cluster lists of the dispersion pass (mixed form)
     int cl_mode;             // build: 1 = CN per-atom lists and cluster lists, 0 = both per-atom lists
     int64_t ncl;             // clusters over the batch
     const int* clu_sid;      // [ncl] structure of each cluster
     int* nbr_cl;             // rows of cap_cl entries per cluster
     int* cnt_cl;             // [ncl]
+    int* split_q;            // [ncl] clusters with more than split_min entries (work_ctr[2] of them)
+    int split_min;           // entries up to which one warp takes a cluster's whole list
+    int split_on;            // some cluster of the plan has more
     unsigned long long* acc; // [Nr][8] fixed-point sums of the dispersion pass: F (3), dE/dn, site energy
     float* gcn;              // mixed form: per CN-list entry, the chain coefficient f'(r)/r of Eq. 4
                              // (written by the CN pass, 0 outside R_cn; read by the chain pass)
@@ -240,6 +243,25 @@ __device__ __forceinline__ void rec_load(const Work& w, int64_t q, float4& hi, f
 }
 __device__ __forceinline__ float4 rec_hi(const Work& w, int64_t q) { return __ldg(w.rec + 2 * q); }
 __device__ __forceinline__ int rec_tsrc(const Work& w, int64_t q) { return __float_as_int(__ldg(&w.rec[2 * q].w)); }
+
+// Two kernels of a stream at once: the first lets the second start (launch), the
+// second, launched by launch_overlapped, waits for the first's results (wait).
+__device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_overlapped(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, a...);
+}
 
 struct ListView {
     const int* p;  // the atom's row (list_row)
