@@ -593,7 +593,8 @@ __device__ __forceinline__ int64_t next_chunk(const Work& w, int lane, int ctr) 
 __global__ void __launch_bounds__(128) k_build_lists(Work w) {
     if (skip_build(w)) return;
     const int lane = threadIdx.x & 31;
-    const float rd2 = w.rl_disp2, rn2 = w.rl_cn2;
+    // (an entry of the CN list is one of the dispersion list first, also where R_cn is the larger)
+    const float rn2 = w.rl_cn2, rd2 = fmaxf(w.rl_disp2, rn2);
     const float4* __restrict__ H = w.hi;
     __shared__ __align__(16) int stage[2][128][8];
     for (;;) {

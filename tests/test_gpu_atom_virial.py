@@ -6,7 +6,7 @@ import pytest
 
 from paper_2310_05279_gb300 import workloads as wl
 
-from ._helpers import assert_mixed_ok, to_dev
+from ._helpers import assert_fp64_ok, assert_mixed_ok, to_dev
 
 pytestmark = pytest.mark.gpu
 PRM = dict(wl.PBE_BJ)
@@ -87,6 +87,19 @@ def test_atom_virial_wide_cell(torch_cuda):
             assert stats["image_atoms"] * b.tables.ntypes <= 2 * stats["real_atoms"] and stats["list_mode"] == 0
     wa, ref = (out[k]["w_atom"].cpu().numpy() for k in ("mixed", "fp64"))
     assert np.abs(wa - ref).max() <= TOL_WA["mixed"] * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_cn_cutoff_beyond_rpot(torch_cuda, oracle_mod, precision):
+    """R_cn > R_pot: the CN lists reach beyond the dispersion pairs."""
+    from paper_2310_05279_gb300 import D3
+    b = wl.uneven_batch(seed=18, nstruct=3, n_range=(20, 120))
+    prm = dict(PRM, rc_disp=5.0, rc_cn=6.0)
+    d3 = D3(b.tables, prm, precision=precision)
+    pos, typ = to_dev(b)
+    out = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc, w_atom=True)
+    d3.sync_status()
+    (assert_fp64_ok if precision == "fp64" else assert_mixed_ok)(out, oracle_mod.compute_batch(b, prm), b.offsets)
 
 
 def test_heat_current(torch_cuda):
