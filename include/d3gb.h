@@ -74,7 +74,9 @@ enum { D3_FP64 = 0, D3_MIXED = 1 };
  * the positions are refreshed.  No host synchronisation is involved either way.
  * precision: D3_MIXED evaluates distances, damping, the C6 interpolation and
  * the coordination-number terms in FP32 with FP64 accumulation of energies,
- * virials and dE/dn; D3_FP64 evaluates everything in FP64. */
+ * virials and dE/dn; D3_FP64 evaluates everything with FP64 accuracy (the
+ * dispersion pass forms its C6 interpolation and its sums in 64-bit fixed
+ * point, scaled so that they round less than FP64 does). */
 typedef struct d3_params {
     double s6, s8, a1, a2_bohr;
     double k1, k2, k3;

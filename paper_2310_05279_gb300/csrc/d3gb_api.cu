@@ -125,9 +125,10 @@ struct Pinned {
     }
 };
 
-// List layout of a build: the mixed form's forward takes its dispersion pairs
-// from cluster half lists (per-atom lists only within R_cn); the FP64 form, the
-// per-atom virial of Eq. 7 and the backward use full per-atom lists.
+// List layout of a build: the forward takes its dispersion pairs from cluster
+// half lists (per-atom lists only within R_cn); the per-atom virial of Eq. 7, the
+// backward, and the FP64 form with parameters outside its fixed-point bounds use
+// full per-atom lists.
 enum ListMode { kFullLists = 0, kClusterLists = 1 };
 
 struct Plan {
@@ -149,6 +150,7 @@ struct Plan {
     int* gate = nullptr;  // list-reuse gate (device int)
     unsigned long long* acc = nullptr;  // fixed-point sums of the cluster-list dispersion pass
     unsigned long long* npairs = nullptr;  // pair count of the cluster-list dispersion pass
+    long long *ipos = nullptr, *row64 = nullptr;  // FP64 form over cluster lists
     float* vd = nullptr;                // C6 projections (v, dv) per atom of the cluster-list dispersion pass
     int split_on = 0;                   // some cluster's list is longer than w.split_min
     int vd_images = 0;                  // image atoms have rows of vd of their own (cluster lists only)
@@ -162,6 +164,8 @@ void set_mode(Plan& P, int mode) {
     P.w.vd = mode == kClusterLists ? P.vd : nullptr;
     P.w.vd_images = mode == kClusterLists ? P.vd_images : 0;  // without vd there are no rows to copy
     P.w.split_on = P.split_on;
+    P.w.ipos = mode == kClusterLists ? P.ipos : nullptr;
+    P.w.row64 = mode == kClusterLists ? P.row64 : nullptr;
 }
 
 }  // namespace
@@ -188,6 +192,12 @@ struct d3_handle {
     float4* d_rcpair = nullptr;  // k2 (Rcov_i + Rcov_j) and its square, FP32 hi + lo
     float2* d_exptab = nullptr;  // 2^(j/64), j = 0..63, FP32 hi + lo
     double* d_rk = nullptr;
+    double* d_k1rc = nullptr;    // k1 k2 (Rcov_i + Rcov_j)
+    double* d_exptab64 = nullptr;  // 2^(j/64), j = 0..63
+    // bounds of the FP64 form over cluster lists (Consts::fx_*); fx_ok: finite and positive
+    bool fx_ok = false;
+    int fx_e[5] = {}, fx_dsh = 0;
+    float fx_ratio = 1.0f;
     int* d_status = nullptr;
     int* h_status = nullptr;                 // pinned host word for the status read of the host-buffer path
     unsigned long long* d_nbuild = nullptr;  // builds executed on the device
@@ -249,9 +259,62 @@ double det3(const double* H) {
     return H[0] * (H[4] * H[8] - H[5] * H[7]) - H[1] * (H[3] * H[8] - H[5] * H[6]) + H[2] * (H[3] * H[7] - H[4] * H[6]);
 }
 
+// Bounds on one pair's terms over all element pairs and distances (FP64 form over
+// cluster lists): with C the largest |C6 reference| of the pair, x = |s6|, y = |s8| R0^2,
+//   de/dC6          x / R^6 + y / R^8                               (at r = 0)
+//   |C6 de/dC6|     C times that
+//   |de/dr|         C (1.56 x / R^7 + 2.03 y / R^9)                  (6 u^5/(1 + u^6)^2 <= 1.56, 8 u^7/(1 + u^8)^2 <= 2.03)
+//   r |de/dr|       C (1.5 x / R^6 + 2 y / R^8)                      (at r = R)
+//   |de/dr| / r     C (1.69 x / R^8 + 2.14 y / R^10)                 (6 u^4/(1 + u^6)^2, 8 u^6/(1 + u^8)^2)
+// and fx_ratio the largest ratio of a pair's terms at r >= R_cn to these bounds (every
+// term falls with r beyond R).  Exponents e with bound < 2^e.
+void fixed_point_bounds(d3_handle* h) {
+    const int T = h->T, R = h->R;
+    double mx[5] = {}, far[4] = {};
+    bool ok = true;
+    const double rcn = h->prm.rc_cn_A / kBohrA;
+    for (int a = 0; a < T; ++a)
+        for (int b = 0; b < T; ++b) {
+            double C = 0.0;
+            for (int k = 0; k < R * R; ++k) C = std::max(C, std::fabs(h->c6[((size_t)a * T + b) * R * R + k]));
+            const double q = 3.0 * h->sqrtq[a] * h->sqrtq[b], Rd = std::fabs(h->prm.a1 * std::sqrt(q) + h->prm.a2_bohr);
+            const double x = std::fabs(h->prm.s6), y = std::fabs(h->prm.s8) * q;
+            const double R2 = Rd * Rd, R6 = R2 * R2 * R2, R8 = R6 * R2;
+            const double r = std::max(rcn, Rd), r2 = r * r, r6 = r2 * r2 * r2, r8 = r6 * r2;
+            const double d6 = r6 + R6, d8 = r8 + R8, n6 = rcn * rcn * rcn * rcn * rcn * rcn;
+            const double v[4] = {C * (1.56 * x / (R6 * Rd) + 2.03 * y / (R8 * Rd)), C * (x / R6 + y / R8),
+                                 C * (1.5 * x / R6 + 2.0 * y / R8), x / R6 + y / R8};
+            const double g = x / (n6 + R6) + y / (n6 * rcn * rcn + R8);
+            const double f = 6.0 * x * r6 / r / (d6 * d6) + 8.0 * y * r8 / r / (d8 * d8);
+            const double u[4] = {C * f, C * g, C * f * r, g};
+            for (int k = 0; k < 4; ++k) {
+                ok = ok && std::isfinite(v[k]) && std::isfinite(u[k]);
+                mx[k] = std::max(mx[k], v[k]);
+                far[k] = std::max(far[k], u[k]);
+            }
+            mx[4] = std::max(mx[4], C * (1.69 * x / R8 + 2.14 * y / (R8 * R2)));
+            ok = ok && R8 > 1e-200;
+        }
+    double ratio = 0.0;
+    for (int k = 0; k < 5; ++k) {
+        ok = ok && mx[k] > 1e-100 && mx[k] < 1e100;
+        if (!ok) continue;
+        h->fx_e[k] = std::ilogb(mx[k]) + 1;
+        if (k < 4) ratio = std::max(ratio, far[k] / mx[k]);
+    }
+    // pair vectors (units of 2^-50 bohr, below 2^dexp bohr) are shifted left to at most 62 bits, and by no
+    // more than leaves a lane's virial sum, in units 2^(14 - dsh) of the force's, below 2^58
+    const int dexp = std::ilogb(h->prm.rc_disp_A / kBohrA) + 1;
+    h->fx_dsh = ok ? std::min(12 - dexp, 11 - (h->fx_e[2] - h->fx_e[0])) : 0;
+    ok = ok && h->fx_dsh >= 0;
+    h->fx_ok = ok;
+    h->fx_ratio = ok ? (float)std::min(1.0, 1.01 * ratio) : 1.0f;
+}
+
 // Upload the damping table (R^6, R^8, s6, s8 R0^2 per element pair) in both precisions.
 d3_status upload_pair_table(d3_handle* h) {
     const int T = h->T;
+    fixed_point_bounds(h);
     std::vector<dbl4> pd(T * T), pb(T * T);
     std::vector<float4> pf(T * T);
     std::vector<double> rd(T * T);
@@ -312,6 +375,13 @@ Consts make_consts(const d3_handle* h) {
     c.alpha9f = (float)c.alpha9;
     c.alpha9_3f = (float)(c.alpha9 / 3.0);
     c.rc3_2f = (float)c.rc3_2;
+    c.fx_eF = h->fx_e[0];
+    c.fx_eE = h->fx_e[1];
+    c.fx_eV = h->fx_e[2];
+    c.fx_eG = h->fx_e[3];
+    c.fx_eM = h->fx_e[4];
+    c.fx_dsh = h->fx_dsh;
+    c.fx_ratio = h->fx_ratio;
     return c;
 }
 
@@ -545,12 +615,19 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
         A(w.nbr_cl, int, lcl);
         A(w.cnt_cl, int, ncl);
         A(w.split_q, int, ncl);
-        A(w.acc, unsigned long long, 8 * Nr);
+        A(w.acc, unsigned long long, (mixed ? 8 : 16) * Nr);
         A(w.npairs, unsigned long long, 1);
         // rows of v and dv for real and image atoms (whether images get copies of their
         // source's rows is decided after the sizing pass, from the image count)
         if (mixed) A(w.vd, float, Nt * h->T * 2 * h->RP);
         if (mixed) A(w.gcn, float, lc);
+        if (!mixed) {
+            A(w.gcnd, double, lc);
+            A(w.ipos, long long, 4 * Nt);
+            A(w.row64, long long, Nr * h->T * row64_len(h->R));
+            A(w.i64, long long, Nr * row64_len(h->R));
+            A(w.kd, int, Nr);
+        }
         A(w.gate, int, 1);
         A(w.xref, double, 3 * Nr);
         A(w.wshift, double, 3 * Nr);
@@ -587,8 +664,11 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     P.npairs = w.npairs;
     P.w.npairs = nullptr;
     P.vd = w.vd;
+    P.ipos = w.ipos;
+    P.row64 = w.row64;
     P.w.acc = nullptr;
     P.w.vd = nullptr;
+    P.w.ipos = P.w.row64 = nullptr;
     P.w.cl_mode = 0;
     const double rld = list_radius(h, h->prm.rc_disp_A), rln = list_radius(h, h->prm.rc_cn_A);
     w.rl_disp2 = (float)(rld * rld);
@@ -640,6 +720,8 @@ Tabs forward_tabs(const d3_handle* h) {
     tb.nref = h->d_nref;
     tb.rcpair = h->d_rcpair;
     tb.exptab = h->d_exptab;
+    tb.k1rc = h->d_k1rc;
+    tb.exptab64 = h->d_exptab64;
     tb.rtab = mixed ? (const void*)h->d_rtabf : (const void*)h->d_rtabd;
     return tb;
 }
@@ -838,7 +920,7 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         }
         for (int s2 = 0; s2 < B; ++s2) {
             StructGeo& G = P.geo[s2];
-            if (mx[3 * s2] > G.cap_disp) { G.cap_disp = round_cap(mx[3 * s2] * 1.1 + 16); grow = true; }
+            if (mode == kFullLists && mx[3 * s2] > G.cap_disp) { G.cap_disp = round_cap(mx[3 * s2] * 1.1 + 16); grow = true; }
             auto regrow = [&](int n, int32_t& cap, int spare, double est, double& ratio) {
                 if (n <= cap) return;
                 cap = round_cap(n * 1.1 + spare);
@@ -882,10 +964,11 @@ d3_status check_batch_args(d3_handle* h, int32_t B, const int64_t* offsets, cons
     return D3_OK;
 }
 
-// List mode of a forward call: cluster lists for the mixed form, full per-atom
-// lists for the FP64 form and for the per-atom virial of Eq. 7.
+// List mode of a forward call: cluster lists, but full per-atom lists for the
+// per-atom virial of Eq. 7 and for the FP64 form where a pair's terms have no usable
+// bounds (a damping radius of zero, all-zero C6 references).
 int list_mode(const d3_handle* h, const double* w_atom) {
-    return h->prm.precision == D3_MIXED && !w_atom ? kClusterLists : kFullLists;
+    return (h->prm.precision == D3_MIXED || h->fx_ok) && !w_atom ? kClusterLists : kFullLists;
 }
 
 // Enqueue the build (unless the sizing pass has just run it for these positions)
@@ -1064,6 +1147,8 @@ d3_status d3_create(const d3_params* params, const d3_tables* tables, d3_handle*
     if (e == cudaSuccess) e = m.alloc(&h->d_rcpair, T * T);
     if (e == cudaSuccess) e = m.alloc(&h->d_exptab, 64);
     if (e == cudaSuccess) e = m.alloc(&h->d_rk, T);
+    if (e == cudaSuccess) e = m.alloc(&h->d_k1rc, T * T);
+    if (e == cudaSuccess) e = m.alloc(&h->d_exptab64, 64);
     if (e == cudaSuccess) e = m.alloc(&h->d_status, 1);
     if (e == cudaSuccess) e = m.alloc(&h->d_nbuild, 1);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_nref, h->nref.data(), T * sizeof(int), cudaMemcpyHostToDevice);
@@ -1085,6 +1170,11 @@ d3_status d3_create(const d3_params* params, const d3_tables* tables, d3_handle*
     if (e == cudaSuccess) e = cudaMemcpy(h->d_c6f, c6f.data(), c6f.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_c6d, h->c6.data(), h->c6.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_rk, rk.data(), T * sizeof(double), cudaMemcpyHostToDevice);
+    std::vector<double> k1rc(T * T), ex64(64);
+    for (int k = 0; k < T * T; ++k) k1rc[k] = p.k1 * p.k2 * (h->rcov[k / T] + h->rcov[k % T]);
+    for (int j = 0; j < 64; ++j) ex64[j] = std::exp2(j / 64.0);
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_k1rc, k1rc.data(), k1rc.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_exptab64, ex64.data(), 64 * sizeof(double), cudaMemcpyHostToDevice);
     std::vector<float4> rcp(T * T);
     for (int a2 = 0; a2 < T; ++a2)
         for (int b2 = 0; b2 < T; ++b2) {

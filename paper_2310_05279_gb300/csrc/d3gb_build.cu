@@ -444,6 +444,16 @@ __device__ inline void split_pos(const double x[3], float (&h)[3], float (&l)[3]
         l[a] = (xh - h[a]) + xl;
     }
 }
+// Positions of the FP64 form over cluster lists, in units of 2^-50 bohr: exact for
+// |x| >= 4 bohr, where an FP64 ulp is no smaller, and rounded by at most 2^-51 below
+// (the FP64 difference of two positions some bohr apart rounds by as much).
+__device__ inline void store_ipos(Work& w, int64_t q, const double x[3], int tsrc) {
+    if (!w.ipos) return;
+    longlong2* d = reinterpret_cast<longlong2*>(w.ipos + 4 * q);
+    const double u = 1125899906842624.0;
+    d[0] = make_longlong2(__double2ll_rn(x[0] * u), __double2ll_rn(x[1] * u));
+    d[1] = make_longlong2(__double2ll_rn(x[2] * u), (long long)tsrc);
+}
 __device__ inline void store_pos(Work& w, int64_t q, const double x[3], double rk, int tsrc) {
     w.pos64[q] = dbl4_make(x[0], x[1], x[2], rk);
     float h[3], l[3];
@@ -451,6 +461,7 @@ __device__ inline void store_pos(Work& w, int64_t q, const double x[3], double r
     w.rec[2 * q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
     w.rec[2 * q + 1] = make_float4(l[0], l[1], l[2], (float)rk);
     w.hi[q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
+    store_ipos(w, q, x, tsrc);
 }
 
 // Sorted positions: threads [0, Nr) fill the real atoms' slots, the next ones the
@@ -503,6 +514,7 @@ __global__ void k_fill(Work w, const int32_t* __restrict__ types, const double* 
     w.rec[2 * (w.Nr + q)] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
     w.rec[2 * (w.Nr + q) + 1] = make_float4(l[0], l[1], l[2], (float)rk);
     w.hi[w.Nr + q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
+    store_ipos(w, w.Nr + q, x, tsrc);
 }
 
 // ---- per-atom lists within the two list radii ------------------------------
@@ -722,6 +734,7 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
         int n = 0;
         int nc[kClusterAtoms] = {0, 0, 0, 0, 0, 0, 0, 0};  // CN list lengths (warp-uniform)
         int ns = 0;                                        // staged CN candidates (warp-uniform)
+        int nwin = 0;                                      // atoms of the window (this lane's ranges)
         // per-atom CN lists of the cluster's atoms from the first m staged candidates
         auto cn_round = [&](int m) {
             __syncwarp();
@@ -768,6 +781,7 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
                 if ((r & 1) == 0) {
                     b = __ldg(&w.start_real[cf]);
                     len = __ldg(&w.start_real[cl + 1]) - b;
+                    nwin += len;
                     if (b + len <= (int)p0) {  // the whole row precedes the cluster: CN candidates only
                         if (y < yc0 || y > yc1 || z < zc0 || z > zc1) {
                             len = 0;
@@ -780,6 +794,7 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
                 } else {
                     b = (int)w.Nr + __ldg(&w.start_ghost[cf]);
                     len = (int)w.Nr + __ldg(&w.start_ghost[cl + 1]) - b;
+                    nwin += len;
                 }
             }
             int incl = len;  // inclusive scan of the lengths over the lanes
@@ -853,6 +868,10 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
                 mc = max(mc, nc[i]);
                 if (lane == i) w.cnt_cn[first + i] = min(nc[i], capc);
             }
+        if (w.ipos) {  // bounds the number of pairs of an atom (FP64 form)
+            nwin = __reduce_add_sync(full, nwin);
+            if (lane == 0) atomicMax(&w.maxcnt[3 * s], nwin);
+        }
         if (lane == 0) {
             w.cnt_cl[I] = min(n, cap);
             if (min(n, cap) > w.split_min) w.split_q[atomicAdd(w.work_ctr + 2, 1)] = (int)I;

@@ -1,0 +1,313 @@
+// d3gb_cluster64.cu -- dispersion pass of the FP64 form over cluster half lists
+// (arXiv 2310.05279, Sec. II A, Eq. 2 with the C6 of Eq. 3).
+//
+// GB300 runs FP64 at 1/64 of the FP32 rate: one FP64 warp instruction occupies its pipe
+// for about 80 issue slots, so the FP64 form is bound by their number and by the lanes
+// they leave idle.  The per-atom-list pass (k_disp) takes about 60 of them per ordered
+// pair.  This pass
+//   * evaluates each unordered pair instance once (the half lists of the mixed form);
+//   * keeps the lanes full: lane = i + 8 j keeps one atom i of the warp's cluster and
+//     tests its quarter of the list in FP32 (FP64 inside the error band of R_pot);
+//     what passes goes into a ring of the lane's own, and the pairs are evaluated when
+//     every lane has one;
+//   * leaves to the FP64 pipe only the damping function (18 instructions a pair).
+//     Pair vectors, r^2, the C6 interpolation and all sums are formed on the integer
+//     pipe, with 64-bit mantissas scaled by powers of two: positions in units of
+//     2^-50 bohr; W, dW and the rows v, dv with one exponent per row (Work::i64,
+//     row64); products as the upper half of 64 x 64 bits.  Their relative errors are
+//     2^-57 and less (the C6 sums: 2^-61 of the row's largest value), below FP64's 2^-53;
+//   * adds everything to per-atom 64-bit fixed-point sums, which associate, so the
+//     result does not depend on the order in which warps and splits of a list run.
+//
+// Scales.  A pair's terms are bounded (Becke-Johnson damping is finite at r = 0), and
+// terms beyond R_cn are smaller by fx_ratio; with the longest CN list and the fullest
+// cluster window of the structure that bounds every atom's sum within a factor of about
+// ten (fix_log2_pairs).  The scale leaves 61 bits to that bound: one unit is some 2^-57
+// of an atom's largest sum.  dE/dn has its own scale per atom, from its own dC6/dn.
+// Parameters whose bounds are not finite and positive keep the per-atom-list pass.
+//
+// Measured on 128 x 1440 atoms (27.9 M pairs): 1.61 ms against 5.62 ms for the per-atom-list
+// pass, FP64 pipe 61% busy, 48% of issue slots used, 16 warps per SM (128 registers; at 142
+// registers and 12 warps 2.07 ms).
+#include "d3gb_pair.cuh"
+
+namespace d3gb {
+
+namespace {
+
+constexpr int kRing = 32;  // ring entries per lane
+constexpr int kTest = 8;   // entries tested per lane at a time
+
+// v 2^-s rounded to nearest, |v| < 2^62 (and the result below 2^62)
+__device__ __forceinline__ long long shr_rn(long long v, int s) {
+    if (s <= 0) return v << min(-s, 63);
+    s = min(s, 62);
+    return (v + (1LL << (s - 1))) >> s;
+}
+// a normal double as m 2^(e - 1085), |m| in [2^62, 2^63)
+__device__ __forceinline__ long long mantissa(double v, int& e) {
+    const long long b = __double_as_longlong(v);
+    e = (int)((unsigned long long)b >> 52) & 0x7ff;
+    const long long m = ((b & 0xfffffffffffffLL) | 0x10000000000000LL) << 10;
+    return b < 0 ? -m : m;
+}
+__device__ __forceinline__ void red_add64(unsigned long long* a, long long x) {
+    atomicAdd(a, (unsigned long long)x);  // result unused: a reduction, no return trip
+}
+
+// Scale exponents of a structure's force, energy and virial sums.
+struct FixScale {
+    int kF, kE, kV;  // kV: of a lane's sum; a cluster's has three bits less
+    int pv;          // bits that the virial's products take beyond the force sums'
+    __device__ FixScale(const Work& w, const Consts& c, int s) {
+        const int lg = fix_log2_pairs(w, c, s);
+        kF = min(61 - c.fx_eF - lg, 45 + c.fx_dsh - c.fx_eM);  // (the second: k_disp_cl64's sF stays above 0)
+        kE = 61 - c.fx_eE - lg;
+        pv = min(75 - c.fx_eV - lg - kF - c.fx_dsh, lg);  // (at least 3: fixed_point_bounds)
+        kV = kF + c.fx_dsh - 14 + pv;
+    }
+};
+
+// Damping constants of an element pair in shared memory: R^6, R^8, s6, s8 R0^2, 6 s6, 8 s8 R0^2.
+constexpr int kDamp = 6;
+
+template <int R, bool SITE>
+__global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const dbl4* __restrict__ pair_tab, int nsplit) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* tab = reinterpret_cast<double*>(smem_raw);
+    constexpr int S64 = row64_len(R);
+    // the clusters' rows W, dW (loaded again for every pair: they would take 20 registers)
+    long long* wsh = reinterpret_cast<long long*>(tab + kDamp * c.T * c.T) + (threadIdx.x >> 5) * (kClusterAtoms * S64);
+    int* rings = reinterpret_cast<int*>(reinterpret_cast<long long*>(tab + kDamp * c.T * c.T) + 4 * kClusterAtoms * S64);
+    for (int k = threadIdx.x; k < c.T * c.T; k += blockDim.x) {
+        const dbl4 t = pair_tab[k];
+        double* d = tab + kDamp * k;
+        d[0] = t.x; d[1] = t.y; d[2] = t.z; d[3] = t.w; d[4] = 6.0 * t.z; d[5] = 8.0 * t.w;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, il = lane & 7, js = lane >> 3;
+    const int64_t I = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (I >= w.ncl) return;  // whole warps
+    int* ring = rings + (threadIdx.x >> 5) * (kRing * 32) + lane;  // slot k at ring[32 k]
+    const int s = w.clu_sid[I];
+    const StructGeo& G = w.geo[s];
+    const int64_t p0 = G.atom_base + (I - G.clu_base) * kClusterAtoms;
+    const int64_t rem = G.atom_base + G.natoms - p0;
+    const int nI = rem < kClusterAtoms ? (int)rem : kClusterAtoms;
+    const bool ilive = il < nI;
+    const int64_t p = p0 + (ilive ? il : 0);
+    const int* row = w.nbr_cl + G.list_base_cl + (I - G.clu_base) * (int64_t)G.cap_cl;
+    const int cnt = w.cnt_cl[I];
+    const int nblocks = (cnt + 31) >> 5;
+    // this warp's share of the blocks of 32 entries (blockIdx.y of nsplit)
+    const int bb = (int)((int64_t)nblocks * blockIdx.y / nsplit), be = (int)((int64_t)nblocks * (blockIdx.y + 1) / nsplit);
+    if (bb >= be) return;
+    const Site<true> S(w, p);
+    const int ti = S.tsrc() & 15;
+    const int pthr = ilive ? (int)p : 0x7fffffff;  // a pair is used when q > pthr
+    const longlong2* xi2 = reinterpret_cast<const longlong2*>(w.ipos + 4 * p);
+    const longlong2 xa = xi2[0], xb = xi2[1];
+    for (int k = lane; k < nI * S64; k += 32) wsh[k] = w.i64[p0 * S64 + k];
+    __syncwarp();
+    const long long* wi = wsh + (int)(p - p0) * S64;
+    const int eW = (int)wi[2 * R];
+    const int kDi = w.kd[p];
+    const FixScale K(w, c, s);
+    const double* trow = tab + kDamp * ti * c.T;
+    const long long* rbase = w.row64 + ti * S64;
+    const int rstride = c.T * S64;
+    const float rc2 = c.rc_disp2f, band = 4e-6f * c.rc_disp2f;
+    long long aF[3] = {0, 0, 0}, aD = 0, aE = 0, aV[6] = {0, 0, 0, 0, 0, 0};
+    int head = 0, n = 0;  // the lane's ring: first entry and number of entries
+    unsigned npairs = 0;
+
+    auto eval = [&](int q) {
+        const longlong2* x2 = reinterpret_cast<const longlong2*>(w.ipos + 4 * (int64_t)q);
+        const longlong2 ya = __ldg(x2), yb = __ldg(x2 + 1);
+        const int tsq = (int)yb.y;
+        const int64_t src = tsq >> 4;
+        const longlong2* rp = reinterpret_cast<const longlong2*>(rbase + src * rstride);
+        long long rv[2 * R + 2];
+#pragma unroll
+        for (int a = 0; a < 2 * R + 1; a += 2) {
+            const longlong2 t = __ldg(rp + a / 2);
+            rv[a] = t.x;
+            rv[a + 1] = t.y;
+        }
+        const int ev = (int)rv[2 * R], ed = (int)(rv[2 * R] >> 32);
+        const int kDj = __ldg(w.kd + src);
+        // pair vector, and r^2 = r2u 2^(-36 - 2 sh) from it normalised by its largest component
+        long long dx = ya.x - xa.x, dy = ya.y - xa.y, dz = yb.x - xb.x;
+        const unsigned long long o = (unsigned long long)((dx ^ (dx >> 63)) | (dy ^ (dy >> 63)) | (dz ^ (dz >> 63)));
+        const int sh = __clzll((long long)o) - 1;
+        const long long nx = dx << sh, ny = dy << sh, nz = dz << sh;
+        const unsigned long long r2u = (unsigned long long)(__mul64hi(nx, nx) + __mul64hi(ny, ny)) +
+                                       (unsigned long long)__mul64hi(nz, nz);
+        const int lz = __clzll((long long)r2u);
+        const unsigned long long mant = r2u << lz;
+        const unsigned long long bits = ((unsigned long long)(unsigned)(1049 - 2 * sh - lz) << 52) + (mant >> 11) +
+                                        ((mant >> 10) & 1);  // (the leading bit adds one to the exponent)
+        const double r2 = r2u ? __longlong_as_double((long long)bits) : 0.0;
+        const double* t = trow + kDamp * (tsq & 15);
+        // damping: g = -de/dC6 = s6/(r^6 + R^6) + s8 R0^2/(r^8 + R^8), fc0 = (de/dr)/(C6 r)
+        const double r4 = r2 * r2, r6 = r4 * r2;
+        const double d6 = r6 + t[0], d8 = fma(r4, r4, t[1]);
+        const double pinv = rcp64(d6 * d8);
+        const double i6 = d8 * pinv, i8 = d6 * pinv;
+        const double g = fma(t[3], i8, t[2] * i6);
+        const double u6 = r2 * i6;
+        const double fc0 = fma(t[5], r6 * (i8 * i8), t[4] * (u6 * u6));
+        // C6 and both CN derivatives
+        long long C6 = (R + 1) / 2, dCi = 0, dCj = 0;  // (each product is rounded down)
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            const long long W = wi[a];
+            C6 += __mul64hi(W, rv[a]);            // units 2^(ev - 61)
+            dCi += __mul64hi(wi[R + a], rv[a]);   // 2^(eW + ev - 60)
+            dCj += __mul64hi(W, rv[R + a]);       // 2^(ed - 61)
+        }
+        C6 <<= 1;   // below 2^62 and a rounding error: the weights add up to 1
+        dCj <<= 1;
+        int eg, ef;
+        const long long mg = mantissa(g, eg), mf = mantissa(fc0, ef);
+        // energy and dE/dn
+        const int sE = 1083 - eg - ev - K.kE + (SITE ? 1 : 0);  // SITE: half of it to each atom
+        const long long e = shr_rn(__mul64hi(mg, C6), sE);
+        aE += e;
+        aD += shr_rn(__mul64hi(mg, dCi), 1081 - eg - eW - ev - kDi);
+        unsigned long long* aj = w.acc + 16 * src;
+        red_add64(aj + 3, shr_rn(__mul64hi(mg, dCj), 1083 - eg - ed - kDj));
+        if (SITE) red_add64(aj + 4, e);
+        // force, and the virial from it (rounded down: half a unit a pair is added at the end)
+        dx <<= c.fx_dsh; dy <<= c.fx_dsh; dz <<= c.fx_dsh;
+        const long long fC = __mul64hi(mf, C6) << 1;
+        // forces with pv bits more than their sums keep, for the virial
+        const int sF = min(1070 + c.fx_dsh - ef - ev - K.kF, 62) - K.pv;
+        const int dn = max(sF, 0), up = max(-sF, 0);
+        // (rounded: a half list's pair vectors do not cancel, so a bias would add up in the virial)
+        const long long h1 = (1LL << dn) >> 1, half = 1LL << (K.pv - 1);
+        const long long ux = (__mul64hi(fC, dx) + h1) >> dn << up, uy = (__mul64hi(fC, dy) + h1) >> dn << up,
+                        uz = (__mul64hi(fC, dz) + h1) >> dn << up;
+        const long long tx = (ux + half) >> K.pv, ty = (uy + half) >> K.pv, tz = (uz + half) >> K.pv;
+        aF[0] += tx; aF[1] += ty; aF[2] += tz;
+        red_add64(aj + 0, -tx);
+        red_add64(aj + 1, -ty);
+        red_add64(aj + 2, -tz);
+        aV[0] += __mul64hi(ux, dx);
+        aV[1] += __mul64hi(uy, dy);
+        aV[2] += __mul64hi(uz, dz);
+        aV[3] += __mul64hi(ux, dy);
+        aV[4] += __mul64hi(ux, dz);
+        aV[5] += __mul64hi(uy, dz);
+    };
+    auto evaluate = [&]() {  // one pair per lane that has one
+        if (n > 0) {
+            const int q = ring[32 * head];
+            head = (head + 1) & (kRing - 1);
+            --n;
+            eval(q);
+        }
+    };
+
+    for (int b = bb; b < be; ++b) {
+        const int k = 32 * b + lane;
+        const int qa = k < cnt ? __ldg(row + k) : -1;
+#pragma unroll
+        for (int st = 0; st < kTest; ++st) {
+            const int q = __shfl_sync(0xffffffffu, qa, (st << 2) + js);
+            float4 h, l;
+            rec_load(w, q >= 0 ? q : 0, h, l);
+            const float dx = (h.x - S.h.x) + (l.x - S.l.x);
+            const float dy = (h.y - S.h.y) + (l.y - S.l.y);
+            const float dz = (h.z - S.h.z) + (l.z - S.l.z);
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            bool use = q > pthr && r2 < rc2;
+            if (q > pthr && fabsf(r2 - rc2) <= band) use = S.inside(q, r2, rc2, c.rc_disp2);
+            if (use) {
+                ring[32 * ((head + n) & (kRing - 1))] = q;
+                ++n;
+            }
+            npairs += use ? 1u : 0u;
+        }
+        while (__all_sync(0xffffffffu, n > 0) || __any_sync(0xffffffffu, n > kRing - kTest)) evaluate();
+    }
+    while (__any_sync(0xffffffffu, n > 0)) evaluate();
+
+    const long long mine = npairs;  // the lane's pairs
+    npairs = __reduce_add_sync(0xffffffffu, npairs);
+    if (lane == 0 && w.npairs) atomicAdd(w.npairs, (unsigned long long)npairs);
+    if (ilive) {
+        unsigned long long* ai = w.acc + 16 * p;
+        red_add64(ai + 0, aF[0]);
+        red_add64(ai + 1, aF[1]);
+        red_add64(ai + 2, aF[2]);
+        red_add64(ai + 3, aD);
+        red_add64(ai + 4, aE);
+        // the virial, in half units for the half that each pair's rounding lost on average: a
+        // cluster's sum of 32 lanes' (and splits') would need more bits than a word has, so the
+        // last four are added up on their own (13 bits each: at most 15 x 512)
+        unsigned long long* av = w.acc + 16 * p0 + 5;
+        unsigned long long rest[2] = {0, 0};
+#pragma unroll
+        for (int m = 0; m < 6; ++m) {
+            const long long v = 2 * aV[m] + mine;
+            red_add64(av + m, v >> 4);
+            rest[m / 3] |= (unsigned long long)(v & 15) << (13 * (m % 3));
+        }
+        red_add64(av + 6, (long long)rest[0]);
+        red_add64(av + 7, (long long)rest[1]);
+    }
+}
+
+// Per atom: the fixed-point totals into the arrays the chain pass, the per-structure
+// sums (and the optional three-body pass) read.
+__global__ void __launch_bounds__(256) k_disp_fin64(Work w, Consts c) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= w.Nr) return;
+    const FixScale K(w, c, w.sid[p]);
+    const long long* a = reinterpret_cast<const long long*>(w.acc) + 16 * p;
+    auto value = [](long long v, int k) { return ldexp((double)v, -k); };
+    ((dbl4*)w.Fd)[p] = dbl4_make(value(a[0], K.kF), value(a[1], K.kF), value(a[2], K.kF), 0.0);
+    ((double*)w.dEdn)[p] = -value(a[3], w.kd[p]);
+    w.eat[p] = -value(a[4], K.kE);
+    double* wv = w.wv + 6 * p;
+#pragma unroll
+    for (int m = 0; m < 6; ++m) {  // (zero but on a cluster's first atom)
+        const long long rest = (a[11 + m / 3] >> (13 * (m % 3))) & 8191;
+        wv[m] = a[5 + m] | rest ? -ldexp((double)a[5 + m] + 0.0625 * (double)rest, 3 - K.kV) : 0.0;
+    }
+}
+
+inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
+
+}  // namespace
+
+cudaError_t launch_disp_cl64(const Work& w, const Consts& c, const dbl4* pair_tab, bool site, cudaStream_t st) {
+    if (w.Nr == 0) return cudaGetLastError();
+    if (w.ncl > 0) {
+        // 16 warps stay resident per SM; with fewer clusters than that each list goes to several warps
+        const int64_t want = 16 * (int64_t)w.num_sms;
+        const int nsplit = (int)(w.ncl >= want ? 1 : (want / w.ncl < 16 ? (want + w.ncl - 1) / w.ncl : 16));
+        const dim3 grid(nblk(w.ncl, 4), (unsigned)nsplit);
+        const size_t sm = (size_t)c.T * c.T * kDamp * sizeof(double) +
+                          4 * ((size_t)kClusterAtoms * row64_len(c.R) * sizeof(long long) + kRing * 32 * sizeof(int));
+#define D3_CL(RR)                                                                          \
+    if (site) k_disp_cl64<RR, true><<<grid, 128, sm, st>>>(w, c, pair_tab, nsplit);       \
+    else k_disp_cl64<RR, false><<<grid, 128, sm, st>>>(w, c, pair_tab, nsplit);           \
+    break
+        switch (c.R) {
+            case 1: D3_CL(1);
+            case 2: D3_CL(2);
+            case 3: D3_CL(3);
+            case 4: D3_CL(4);
+            case 5: D3_CL(5);
+            case 6: D3_CL(6);
+            default: D3_CL(7);
+        }
+#undef D3_CL
+    }
+    k_disp_fin64<<<nblk(w.Nr, 256), 256, 0, st>>>(w, c);
+    return cudaGetLastError();
+}
+
+}  // namespace d3gb

@@ -103,6 +103,8 @@ __host__ __device__ inline void row_cells(const StructGeo& G, int cy, int cz, in
     first = a < b ? a : b;
     last = a < b ? b : a;
 }
+// 64-bit words per row of Work::row64 and Work::i64 (2 R values and one word of exponents, whole sectors)
+__host__ __device__ constexpr int row64_len(int R) { return (2 * R + 1 + 3) & ~3; }
 // Atoms per cluster of the cluster lists (consecutive sorted real atoms of a structure).
 constexpr int kClusterAtoms = 8;
 
@@ -151,7 +153,8 @@ struct Work {
     int* nbr_cn;
     int* cnt_disp;           // [Nr]
     int* cnt_cn;             // [Nr]
-    int* maxcnt;             // [3*B] max list length per structure (disp, cn, cluster)
+    int* maxcnt;             // [3*B] per structure, the longest list of an atom or cluster: disp (cluster lists:
+                             // the most atoms in a cluster's window), cn, cluster
     int* work_ctr;           // [3] persistent-kernel work counters, length of split_q (zeroed before each build)
     // cluster lists of the dispersion pass (mixed form)
     int cl_mode;             // build: 1 = CN per-atom lists and cluster lists, 0 = both per-atom lists
@@ -162,7 +165,14 @@ struct Work {
     int* split_q;            // [ncl] clusters with more than split_min entries (work_ctr[2] of them)
     int split_min;           // entries up to which one warp takes a cluster's whole list
     int split_on;            // some cluster of the plan has more
-    unsigned long long* acc; // [Nr][8] fixed-point sums of the dispersion pass: F (3), dE/dn, site energy
+    unsigned long long* acc; // fixed-point sums of the dispersion pass: mixed [Nr][8] F (3), dE/dn, site energy;
+                             // FP64 [Nr][16] F (3), dE/dn, energy, and on a cluster's first atom its virial (6)
+    // FP64 form over cluster lists (d3gb_cluster64.cu): 64-bit integers scaled by powers of two
+    long long* ipos;         // [Nr + ghost_cap][4] x, y, z in units of 2^-50 bohr, type | (source << 4)
+    long long* row64;        // [Nr][T][row64_len(R)] rows v^(t), dv^(t) and their exponents
+    long long* i64;          // [Nr][row64_len(R)] W, dW/dn and its exponent
+    int* kd;                 // [Nr] scale exponent of the atom's dE/dn sum
+    double* gcnd;            // FP64 form: per CN-list entry, the chain coefficient f'(r)/r (as gcn)
     float* gcn;              // mixed form: per CN-list entry, the chain coefficient f'(r)/r of Eq. 4
                              // (written by the CN pass, 0 outside R_cn; read by the chain pass)
     float* vd;               // [Nr (+ ghost_cap)][T][2][RP] per atom q and partner type t: v_q^(t) and
@@ -214,6 +224,11 @@ struct Consts {
     float s9f, alpha9f, alpha9_3f, rc3_2f;  // FP32 copies (alpha9_3f = alpha9 / 3) for the mixed form
     float k1f, rc_cn2f, k3f;   // FP32 copies for the mixed form
     float k3h, k3l;            // k3 as a float pair (k3h + k3l)
+    // FP64 form over cluster lists: binary exponents that bound one pair's force, energy and virial
+    // terms, de/dC6 and (de/dr)/r (Eq. 2), and the ratio of the bounds beyond R_cn to those at any distance
+    int fx_eF, fx_eE, fx_eV, fx_eG, fx_eM;
+    int fx_dsh;                // pair vectors: units of 2^-(50 + fx_dsh) bohr
+    float fx_ratio;
 };
 
 // ---- neighbour lists: `cap` entries per atom (cap a multiple of 8).  The rows of
@@ -287,6 +302,14 @@ __host__ __device__ inline void unpack_shift(int s, int& a, int& b, int& c) {
     c = ((s >> 16) & 255) - 128;
 }
 
+// FP64 form over cluster lists: a bound on an atom's number of pairs of structure s,
+// weighted by the size their terms can have, as a binary logarithm (at least 5).  The
+// CN lists hold every partner within R_cn; beyond, terms are smaller by fx_ratio.
+__device__ __forceinline__ int fix_log2_pairs(const Work& w, const Consts& c, int s) {
+    const int n = w.maxcnt[3 * s + 1] + (int)(c.fx_ratio * (float)w.maxcnt[3 * s]) + 17;
+    return 32 - __clz(n);
+}
+
 // Structure of input atom i (binary search over offsets).
 __device__ inline int struct_of(const int64_t* off, int B, int64_t i) {
     int lo = 0, hi = B;  // off[lo] <= i < off[hi]
@@ -308,6 +331,8 @@ cudaError_t launch_build(const Work& w, const double* pos, const int32_t* types,
 cudaError_t launch_check(const Work& w, const double* pos, cudaStream_t st);
 // Device tables of one handle.
 struct Tabs {
+    const double* k1rc;    // [T][T] k1 k2 (Rcov_i + Rcov_j) (bohr), FP64 form
+    const double* exptab64;  // [64] 2^(j/64), FP64 form
     const void* c6;        // [T][T][R][R] real (float or double by precision)
     const void* pair;      // [T][T] real4: R^6, R^8, s6, s8 R0^2
     const double* cnref;   // [T][R]
@@ -330,6 +355,8 @@ cudaError_t launch_forward(const Work& w, const Consts& c, bool mixed, const Tab
 // false, w.eat holds per-cluster sums on each cluster's first atom instead of
 // site energies).
 cudaError_t launch_disp_cl(const Work& w, const Consts& c, const void* pair_tab, bool site, cudaStream_t st);
+// The same for the FP64 form (d3gb_cluster64.cu).
+cudaError_t launch_disp_cl64(const Work& w, const Consts& c, const dbl4* pair_tab, bool site, cudaStream_t st);
 // Optional three-body pass (d3gb_atm.cu): adds into w.eat, w.wv, w.Fd and
 // w.dEdn after the dispersion pass; rtab as Tabs::rtab in the handle's precision.
 cudaError_t launch_atm(const Work& w, const Consts& c, bool mixed, const void* rtab, cudaStream_t st);

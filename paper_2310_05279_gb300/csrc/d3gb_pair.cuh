@@ -32,6 +32,45 @@ __device__ __forceinline__ float rcp_nr(float x) {
     return fmaf(y, e, y);
 }
 
+// FP64 reciprocal, reciprocal square root and exponential for the FP64 form.  An
+// FP64 instruction occupies its pipe for about 80 issue slots on this GPU, so they
+// are written for few of them: the hardware's estimate (about 2^-20, not on that
+// pipe) and one step of Householder's iteration of third order, which leaves a
+// relative error near 2^-60 before the last rounding (3 and 5 instructions; the
+// IEEE division and square root take about 10 and 12).
+__device__ __forceinline__ double rcp64(double x) {  // 1/x for normal, finite x
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);  // 1/x = y (1 + e + e^2 + ...)
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) {  // x^(-1/2) for normal, finite x > 0
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);  // x^(-1/2) = y (1 + e/2 + 3 e^2/8 + ...)
+    return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+// exp(x) by the table-driven method named at cn_ds below: x = (64 m + j) L + r with
+// L = ln2/64 in two parts, exp(r) - 1 by its Taylor series to r^5 (|r| <= L/2: the rest
+// is below 2^-54), tab[j] = 2^(j/64) rounded to FP64.  |x| is clamped to 708.
+constexpr double kExp64L1 = 0.010830424696249145;  // ln2/64 rounded to FP64
+constexpr double kExp64L2 = 3.623510646634843e-19;  // and the rest
+__device__ __forceinline__ double exp64(double x, const double* __restrict__ tab) {
+    if ((__double2hiint(x) & 0x7fffffff) >= 0x40862000) x = copysign(708.0, x);
+    const double kb = fma(x, 92.33248261689366, 6755399441055744.0);  // 64/ln2; 1.5 2^52
+    const double kf = kb - 6755399441055744.0;
+    const int k = __double2loint(kb);
+    double r = fma(-kf, kExp64L1, x);
+    r = fma(-kf, kExp64L2, r);
+    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(r, p, 1.0 / 6.0);
+    p = fma(r, p, 0.5);
+    p = fma(r * r, p, r);
+    const double T = __ldg(tab + (k & 63));
+    const double v = fma(T, p, T);
+    return __hiloint2double(__double2hiint(v) + ((k >> 6) << 20), __double2loint(v));
+}
+
 // s + err == a + b exactly when |a| >= |b| (Dekker's Fast2Sum); s, err may alias a, b
 __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& err) {
     const float t = a + b;

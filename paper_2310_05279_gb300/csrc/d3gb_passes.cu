@@ -9,9 +9,9 @@
 //                     v_i^(t)_a = sum_b C6ref[t][t_i][a][b] W_ib, so that
 //                     C6_ij = sum_a W_ia v_j^(t_i)_a
 //   k_disp     Eq. 2  site energy, direct forces, virial and
-//                     dE/dn_i = sum_j (dE/dC6_ij)(dC6_ij/dn_i) (FP64 form and per-atom
-//                     virial; the mixed form's dispersion pass runs over cluster half
-//                     lists, d3gb_cluster.cu)
+//                     dE/dn_i = sum_j (dE/dC6_ij)(dC6_ij/dn_i) (per-atom virial, and the
+//                     FP64 form where its fixed-point bounds do not hold; otherwise the
+//                     pass runs over cluster half lists, d3gb_cluster.cu, d3gb_cluster64.cu)
 //   k_atm             optional three-body term (not part of the paper's model;
 //                     d3gb_atm.cu), between the dispersion and chain passes
 //   k_chain           forces and virial of the coordination-number dependence:
@@ -46,16 +46,8 @@ template <> struct PassAcc<false> {
     __device__ double total() const { return h; }
 };
 
-// Eq. 4 counting function f(r) and, optionally, df/dr, in FP64; r from 1/r.
-// (The mixed form evaluates it in double-single, cn_ds below.)
-__device__ __forceinline__ void cn_fun(double rinv, double rc_eff, double, double k1, double& f, double* dfdr) {
-    const double t = exp(-k1 * (rc_eff * rinv - 1.0));
-    f = 1.0 / (1.0 + t);
-    if (dfdr) *dfdr = -k1 * rc_eff * rinv * rinv * t * f * f;
-}
-__device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 __device__ __forceinline__ float recip(float x) { return rcp_approx(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ double recip(double x) { return rcp64(x); }
 
 // ------------------------------------------------------------------ Eq. 3
 // Per atom, right after its coordination number (fused into the CN pass): the
@@ -72,6 +64,23 @@ __device__ __forceinline__ void store_row(T* dst, const T (&v)[8], int rp) {
     if (rp > 4) d[1] = T4{v[4], v[5], v[6], v[7]};
 }
 
+// FP64 form over cluster lists: the value v (bits b) in units of 2^(e - bits), rounded,
+// for |v| < 2^e; e = fix_exponent of the largest value of the row.
+__device__ __forceinline__ int fix_exponent(const double* v, int n) {
+    int e = 0;
+    for (int a = 0; a < n; ++a) e = max(e, (__double2hiint(v[a]) >> 20) & 0x7ff);
+    return e - 1022;
+}
+__device__ __forceinline__ long long fix_value(double v, int e, int bits) {
+    const long long b = __double_as_longlong(v);
+    const int ev = (int)((unsigned long long)b >> 52) & 0x7ff;
+    long long m = ev ? ((b & 0xfffffffffffffLL) | 0x10000000000000LL) : 0;
+    const int s = ev - 1075 + bits - e;  // v = m 2^(ev - 1075)
+    if (s >= 0) m <<= min(s, 10);        // s <= bits - 53 <= 10: m < 2^53
+    else m = s < -60 ? 0 : (m + (1LL << (-s - 1))) >> -s;
+    return b < 0 ? -m : m;
+}
+
 // W and dW/dn rows of atom p and its projections v_p^(u)_a = sum_b C6ref[u][t][a][b] W_b
 // (and, for the cluster-list dispersion pass, the same rows next to
 // dv_p^(u)_a = sum_b C6ref[u][t][a][b] dW_b in w.vd)
@@ -82,6 +91,8 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
     store_row<T>((T*)w.dW + p * c.RP, dWr, c.RP);
     T* vp = (T*)w.v + p * c.T * c.RP;
     T* dvp = (sizeof(T) == 4 && w.vd) ? (T*)w.vd + p * c.T * 2 * c.RP : nullptr;  // [T][2][RP] per atom
+    constexpr int S64 = row64_len(R);
+    int edmax = -1022;  // FP64 form: |dv| < 2^edmax over all rows
     for (int u = 0; u < c.T; ++u) {
         const T* cu = c6 + ((size_t)(u * c.T + t) * R) * R;  // C6ref[u][t][a][b]
         T vr[8], dvr[8];
@@ -99,16 +110,45 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
             dvr[a] = ds;
         }
         store_row<T>(vp + u * c.RP, vr, c.RP);
+        if constexpr (sizeof(T) == 8) {
+            if (w.row64) {
+                long long* r64 = w.row64 + (p * c.T + u) * S64;
+                const int ev = fix_exponent(vr, R), ed = fix_exponent(dvr, R);
+                edmax = max(edmax, ed);
+#pragma unroll
+                for (int a = 0; a < R; ++a) {
+                    r64[a] = fix_value(vr[a], ev, 63);
+                    r64[R + a] = fix_value(dvr[a], ed, 63);
+                }
+                r64[2 * R] = (long long)(unsigned)ev | ((long long)ed << 32);
+            }
+        }
         if (dvp) {
             store_row<T>(dvp + 2 * u * c.RP, vr, c.RP);
             store_row<T>(dvp + (2 * u + 1) * c.RP, dvr, c.RP);
         }
     }
+    if constexpr (sizeof(T) == 8) {
+        if (w.row64) {
+            long long* q = w.i64 + p * S64;
+            const int ew = fix_exponent(dWr, R);
+#pragma unroll
+            for (int a = 0; a < R; ++a) {
+                q[a] = fix_value(Wr[a], 0, 62);
+                q[R + a] = fix_value(dWr[a], ew, 61);
+            }
+            q[2 * R] = ew;
+            // |dC6/dn_p| < 2^edmax for any partner (the weights of Eq. 3 add up to 1)
+            w.kd[p] = min(900, 61 - (edmax + c.fx_eG + fix_log2_pairs(w, c, w.sid[p])));
+        }
+    }
     if (p == 0 && w.npairs) *w.npairs = 0ull;  // pair count of this call's dispersion pass
     if (w.acc) {  // clear the atom's fixed-point sums of the cluster-list dispersion pass
-        ulonglong2* a = reinterpret_cast<ulonglong2*>(w.acc + 8 * p);
+        constexpr int n = sizeof(T) == 8 ? 8 : 4;
+        ulonglong2* a = reinterpret_cast<ulonglong2*>(w.acc + 2 * n * p);
         const ulonglong2 z = make_ulonglong2(0ull, 0ull);
-        a[0] = z; a[1] = z; a[2] = z; a[3] = z;
+#pragma unroll
+        for (int k = 0; k < n; ++k) a[k] = z;
     }
 }
 
@@ -240,7 +280,8 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
                                            const float2* __restrict__ exptab, const double* __restrict__ cnref,
                                            const float2* __restrict__ cnref2, const float* __restrict__ dcr,
                                            const int* __restrict__ nref,
-                                           const typename Real<MIXED>::T* __restrict__ c6) {
+                                           const typename Real<MIXED>::T* __restrict__ c6,
+                                           const double* __restrict__ k1rc, const double* __restrict__ exptab64) {
     using T = typename Real<MIXED>::T;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= w.Nr) return;
@@ -303,16 +344,34 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
             }
         }
     } else {
-        const T rki = S.rk();
-        LV.for_each(0, cnt, [&](int q) {
-            T dx, dy, dz, r2, rkq;
+        // f = 1/(1 + t), t = exp(-k1 (rc/r - 1)), and the coefficient f'(r)/r = -k1 rc t f^2 / r^3,
+        // kept for the chain pass (33 FP64 instructions a pair, 83% of the FP64 pipe; on 9.4 M entries
+        // 0.76 ms, and the chain pass that reads it 0.30 ms: 0.91 and 1.22 ms with the library's exp,
+        // square root and divisions in both)
+        const double* krow = k1rc + (S.tsrc() & 15) * c.T;
+        double* grow = w.gcnd + (LV.p - w.nbr_cn);
+        auto term = [&](int q) -> double {
+            double dx, dy, dz, r2, rkq;
             int tq;
             S.dist(q, dx, dy, dz, r2, tq, rkq);
-            if (!S.inside(q, r2, rc2, c.rc_cn2)) return;
-            T f;
-            cn_fun(inv_sqrt(r2), rki + rkq, (T)0, k1, f, (T*)nullptr);
+            if (!(r2 < c.rc_cn2)) return 0.0;
+            // (coincident atoms: r = 0, t = 0)
+            const double rinv = __double2hiint(r2) > 0x00100000 ? rsqrt64(r2) : 1.0 / sqrt(r2);
+            const double a = krow[tq & 15];
+            const double t = exp64(fma(-a, rinv, c.k1), exptab64);
+            const double f = rcp64(1.0 + t);
             nh += f;
-        });
+            return -(a * (rinv * rinv)) * (rinv * (t * f * f));
+        };
+        for (int k = 0; k < cnt; k += 4) {
+            const int4 q4 = __ldg(reinterpret_cast<const int4*>(LV.p + list_off(k)));
+            dbl4 g;
+            g.x = term(q4.x);
+            g.y = k + 1 < cnt ? term(q4.y) : 0.0;
+            g.z = k + 2 < cnt ? term(q4.z) : 0.0;
+            g.w = k + 3 < cnt ? term(q4.w) : 0.0;
+            *reinterpret_cast<dbl4*>(grow + list_off(k)) = g;
+        }
         w.cn[p] = (double)nh;
         weights_atom<MIXED, R>(w, c, cnref, nref, c6, p, S.tsrc() & 15, (double)nh);
     }
@@ -439,10 +498,15 @@ __global__ void __launch_bounds__(128) k_chain(Work w, Consts c, const float4* _
         T tm[6] = {0, 0, 0, 0, 0, 0}, gv[3] = {0, 0, 0}, mm[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
         // one pair's chain-rule terms: pair vector d, coefficient g = f'(r)/r, partner's dE/dn
         auto add_pair = [&](T dx, T dy, T dz, T g, T dnq, int srcq) {
-            const T coef = (dni + dnq) * g;
-            fx += coef * dx; fy += coef * dy; fz += coef * dz;
             // per-atom geometric sum for the virial (scaled by dE/dn_i below)
             const T gx = g * dx, gy = g * dy, gz = g * dz;
+            if constexpr (MIXED) {
+                const T coef = (dni + dnq) * g;
+                fx += coef * dx; fy += coef * dy; fz += coef * dz;
+            } else {
+                const T dn2 = dni + dnq;
+                fx = fma(dn2, gx, fx); fy = fma(dn2, gy, fy); fz = fma(dn2, gz, fz);
+            }
             sxx = fma(gx, dx, sxx); syy = fma(gy, dy, syy); szz = fma(gz, dz, szz);
             sxy = fma(gx, dy, sxy); sxz = fma(gx, dz, sxz); syz = fma(gy, dz, syz);
             if constexpr (ATOMV) {
@@ -493,17 +557,21 @@ __global__ void __launch_bounds__(128) k_chain(Work w, Consts c, const float4* _
                 for (int e = 0; e < kGroup; ++e) add_pair(D[e][0], D[e][1], D[e][2], g[e], dn[e], src[e]);
             }
         } else {
-            LV.for_each(k0, k1e, [&](int q) {
-                T dx, dy, dz, r2, rkq;
-                int tsq;
-                S.dist(q, dx, dy, dz, r2, tsq, rkq);
-                if (!S.inside(q, r2, rc2, c.rc_cn2)) return;
-                const T rinv = inv_sqrt(r2);
-                T f, dfdr;
-                cn_fun(rinv, S.rk() + rkq, (T)0, k1, f, &dfdr);
-                const int srcq = tsq >> 4;
-                add_pair(dx, dy, dz, dfdr * rinv, dEdn[srcq], srcq);
-            });
+            const double* grow = w.gcnd + (LV.p - w.nbr_cn);
+            auto entry = [&](int q, double g) {
+                if (__double_as_longlong(g) == 0) return;  // outside R_cn
+                const dbl4 y = w.pos64[q];
+                const int srcq = rec_tsrc(w, q) >> 4;
+                add_pair(y.x - S.x.x, y.y - S.x.y, y.z - S.x.z, g, dEdn[srcq], srcq);
+            };
+            for (int k = k0; k < k1e; k += 4) {
+                const int4 q4 = __ldg(reinterpret_cast<const int4*>(LV.p + list_off(k)));
+                const dbl4 g4 = *reinterpret_cast<const dbl4*>(grow + list_off(k));
+                entry(q4.x, g4.x);
+                if (k + 1 < k1e) entry(q4.y, g4.y);
+                if (k + 2 < k1e) entry(q4.z, g4.z);
+                if (k + 3 < k1e) entry(q4.w, g4.w);
+            }
         }
         Sxx += (double)sxx; Syy += (double)syy; Szz += (double)szz;
         Sxy += (double)sxy; Sxz += (double)sxz; Syz += (double)syz;
@@ -625,11 +693,12 @@ cudaError_t forward_impl(const Work& w, const Consts& c, const Tabs& tb, double*
     mark(0);
     if (w.Nr > 0)
         k_cn<MIXED, R><<<nblk(w.Nr, w.blk_cn), w.blk_cn, 0, st>>>(w, c, tb.rcpair, tb.exptab, tb.cnref, tb.cnref2,
-                                                                  tb.dcr, tb.nref, (const T*)tb.c6);
+                                                                  tb.dcr, tb.nref, (const T*)tb.c6, tb.k1rc, tb.exptab64);
     mark(1);  // the weights (Eq. 3) are formed inside the CN pass
     mark(2);
-    if (MIXED && w.cl_mode && !w_atom) {
-        const cudaError_t e = launch_disp_cl(w, c, tb.pair, e_atom != nullptr, st);
+    if (w.cl_mode && !w_atom) {
+        const cudaError_t e = MIXED ? launch_disp_cl(w, c, tb.pair, e_atom != nullptr, st)
+                                    : launch_disp_cl64(w, c, (const dbl4*)tb.pair, e_atom != nullptr, st);
         if (e != cudaSuccess) return e;
     } else if (w.Nr > 0) {
         const int TB = w.blk_disp;
