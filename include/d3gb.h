@@ -242,8 +242,8 @@ d3_status d3_compute_batch_host(d3_handle *h, int32_t B, const int64_t *offsets,
  *   dLdpos     device double[N][3] = dL/dx (per A), input order
  * The force term needs the Hessian-vector product H*(dL/dF); it is formed by
  * forward-mode differentiation of the whole force evaluation along dL/dF
- * (coordination numbers recomputed, no per-pair storage).  A D3_FP64 handle
- * differentiates in FP64 dual numbers; a D3_MIXED handle forms the values with
+ * (coordination numbers recomputed).  A D3_FP64 handle
+ * carries values and tangents in FP64; a D3_MIXED handle forms the values with
  * the mixed forward's arithmetic (double-single Eq. 4 terms, float-float Eq. 3
  * exponents, FP32 pair math on split positions, compensated sums) and the
  * tangents in FP32, several times faster with the mixed forward's relative

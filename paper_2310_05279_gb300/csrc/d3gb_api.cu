@@ -30,9 +30,9 @@ cudaError_t launch_plan_ids(const StructGeo* geo, const int64_t* offsets, int B,
                             int* sid_in, int* clu_sid, int* fin_sid, cudaStream_t st);
 cudaError_t launch_backward(const Work& w, const Consts& c, const double* c6d, const dbl4* paird,
                             const double* cnref, const int* nref, const Tabs& tbm, const double* dLdE,
-                            const double* dLdF, double* dLdp, double* dLdx, double* scratch, int B, bool mixed,
-                            cudaStream_t st);
-int64_t backward_scratch_doubles(const Work& w, int B);
+                            const double* dLdF, double* dLdp, double* dLdx, double* scratch, int64_t list_cn, int B,
+                            bool mixed, cudaStream_t st);
+int64_t backward_scratch_doubles(const Work& w, int B, int64_t list_cn, bool mixed);
 }  // namespace d3gb
 
 using namespace d3gb;
@@ -1418,7 +1418,8 @@ d3_status d3_backward(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     Plan& P = h->plan;
     if (!built) s = enqueue_build(h, P, pos, types, st, kFullLists);
     if (s != D3_OK) return s;
-    const size_t need = (size_t)backward_scratch_doubles(P.w, B) * sizeof(double);
+    const bool mixed = h->prm.precision == D3_MIXED;
+    const size_t need = (size_t)backward_scratch_doubles(P.w, B, P.list_cn, mixed) * sizeof(double);
     if (need > P.bwd.cap) {  // (otherwise kept: a captured call must not lose the memory it refers to)
         const cudaError_t e = P.bwd.reserve(need);
         if (e != cudaSuccess) return cuda_fail(h, e, "backward scratch");
@@ -1431,8 +1432,10 @@ d3_status d3_backward(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     tbm.exptab = h->d_exptab;
     tbm.cnref2 = h->d_cnref2;
     tbm.dcr = h->d_dcr;
+    tbm.k1rc = h->d_k1rc;
+    tbm.exptab64 = h->d_exptab64;
     cudaError_t e = launch_backward(P.w, c, h->d_c6d, h->d_pairb, h->d_cnref, h->d_nref, tbm, dLdE, dLdF, dLdparams,
-                                    dLdpos, reinterpret_cast<double*>(P.bwd.base), B, h->prm.precision == D3_MIXED, st);
+                                    dLdpos, reinterpret_cast<double*>(P.bwd.base), P.list_cn, B, mixed, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "backward launch");
     return D3_OK;
 }

@@ -1,6 +1,5 @@
 // d3gb_backward.cu -- hand-written backward of (E, F) for damping refits.
-// The handle's precision selects the form of the backward: FP64 dual numbers
-// throughout, or (mixed form) the forward's mixed arithmetic for the values --
+// The handle's precision selects the form of the backward: FP64 throughout, or (mixed form) the forward's mixed arithmetic for the values --
 // the double-single Eq. 4 term and chain coefficient, float-float Eq. 3
 // exponents, FP32 pair math on split positions -- with FP32 tangents.  GB300
 // runs FP64 at 1/64 of the FP32 rate, so the FP64 passes bound the mixed form's
@@ -14,9 +13,10 @@
 // Both second-order terms are directional derivatives along u = gF.  They are
 // obtained by running the whole evaluation (Eq. 4 coordination numbers, Eq. 3
 // weights, Eq. 2 pair terms with their analytic derivatives in s6, s8, a1, a2,
-// and the coordination-number chain rule) once in dual numbers (value,
-// derivative along u), in FP64.  The coordination numbers are recomputed and
-// nothing is stored per pair.
+// and the coordination-number chain rule) once with every quantity's derivative
+// along u beside its value.  The coordination numbers are recomputed; the FP64
+// form keeps the Eq. 4 coefficient and its tangent per CN-list entry, the mixed
+// form stores nothing per pair.
 #include "d3gb_pair.cuh"
 
 namespace d3gb {
@@ -27,9 +27,7 @@ struct Dual {
     double v, t;
 };
 __device__ __forceinline__ Dual dd(double v, double t = 0.0) { return Dual{v, t}; }
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return Dual{a.v + b.v, a.t + b.t}; }
 __device__ __forceinline__ Dual operator-(Dual a, Dual b) { return Dual{a.v - b.v, a.t - b.t}; }
-__device__ __forceinline__ Dual operator-(Dual a) { return Dual{-a.v, -a.t}; }
 __device__ __forceinline__ Dual operator*(Dual a, Dual b) { return Dual{a.v * b.v, a.v * b.t + a.t * b.v}; }
 __device__ __forceinline__ Dual operator*(double s, Dual a) { return Dual{s * a.v, s * a.t}; }
 __device__ __forceinline__ Dual operator+(Dual a, double s) { return Dual{a.v + s, a.t}; }
@@ -46,11 +44,6 @@ __device__ __forceinline__ Dual dexp(Dual a) {
     const double e = exp(a.v);
     return Dual{e, a.t * e};
 }
-__device__ __forceinline__ Dual dsqrt(Dual a) {
-    const double s = sqrt(a.v);
-    return Dual{s, 0.5 * a.t / s};
-}
-
 // per-atom dual arrays carved from one scratch block
 struct BW {
     Dual* n;      // [Nr]
@@ -60,7 +53,8 @@ struct BW {
     Dual* dEdn;   // [Nr]
     Dual* F;      // [Nr][3]
     Dual* th;     // [Nr][4] dE_i/d(s6, s8, a1, a2), half pair sums
-    double* xd;   // [(Nr + ghost_cap) * 3] tangent positions (bohr)
+    dbl4* xd;     // [Nr + ghost_cap] tangent positions (bohr)
+    double2* cc;  // FP64 form: per CN-list entry, f'(r)/r and its tangent (0 outside R_cn)
     double* sth;  // [B][8] per-structure dE/dtheta (value, tangent)
     // mixed form of the dispersion pass
     float* vf;    // [Nr][T][2 * RP]: R values of v padded to RP, then R tangents padded to RP
@@ -69,8 +63,13 @@ struct BW {
     int RP;
 };
 
-__host__ __device__ inline BW carve(double* s, int64_t Nr, int64_t Ng, int T, int R, int B) {
+// (s on a 32-byte boundary, as the 32-byte records at its start need)
+__host__ __device__ inline BW carve(double* s, int64_t Nr, int64_t Ng, int64_t list_cn, int T, int R, int B) {
     BW b;
+    b.xd = reinterpret_cast<dbl4*>(s);
+    s += 4 * (Nr + Ng);
+    b.cc = reinterpret_cast<double2*>(s);
+    s += 2 * list_cn;
     Dual* d = reinterpret_cast<Dual*>(s);
     b.n = d;
     d += Nr;
@@ -87,8 +86,6 @@ __host__ __device__ inline BW carve(double* s, int64_t Nr, int64_t Ng, int T, in
     b.th = d;
     d += 4 * Nr;
     double* x = reinterpret_cast<double*>(d);
-    b.xd = x;
-    x += 3 * (Nr + Ng);
     b.sth = x;
     x += 8 * (int64_t)B;
     b.RP = R <= 4 ? 4 : 8;
@@ -107,7 +104,8 @@ struct BConsts {
 };
 
 // tangent positions: x(t) = x + t * gF / bohr for real atoms, images follow their source
-__global__ void kb_xdot(Work w, BW b, const double* __restrict__ gF, int64_t nt) {
+// (FP32 for the mixed form, else FP64)
+__global__ void kb_xdot(Work w, BW b, const double* __restrict__ gF, int64_t nt, bool mixed) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= nt || q >= w.Nr + w.start_ghost[w.ncells]) return;
     const int src = rec_tsrc(w, q) >> 4;
@@ -116,37 +114,68 @@ __global__ void kb_xdot(Work w, BW b, const double* __restrict__ gF, int64_t nt)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         t[a] = gF[3 * (int64_t)i + a] * (1.0 / kBohrA);
-        b.xd[3 * q + a] = t[a];
     }
-    b.xdf[q] = make_float4((float)t[0], (float)t[1], (float)t[2], 0.0f);
+    if (mixed) b.xdf[q] = make_float4((float)t[0], (float)t[1], (float)t[2], 0.0f);
+    else b.xd[q] = dbl4_make(t[0], t[1], t[2], 0.0);
 }
 
-__device__ __forceinline__ void ddist(const Work& w, const BW& b, int64_t p, int64_t q, Dual (&d)[3], Dual& r2) {
-    const dbl4 x = w.pos64[p], y = w.pos64[q];
-    d[0] = Dual{y.x - x.x, b.xd[3 * q] - b.xd[3 * p]};
-    d[1] = Dual{y.y - x.y, b.xd[3 * q + 1] - b.xd[3 * p + 1]};
-    d[2] = Dual{y.z - x.z, b.xd[3 * q + 2] - b.xd[3 * p + 2]};
-    r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+// FP64 form of the CN, dispersion and chain passes.  The FP64 pipe bounds them (one warp
+// instruction takes about 80 issue slots), so the tangents come from closed forms: every
+// pair function depends on r^2 alone, its tangent is its derivative times
+// d(r^2)/dt = 2 d.u (u the tangent of the pair vector d), and where values and tangents
+// only meet in one result they are combined before they are summed (dual-number
+// arithmetic took 372 instructions per ordered pair in the dispersion pass, this 102:
+// 4.53 ms and 1.34 ms on 6.2 M ordered pairs; CN pass 288 us and 93, chain 415 and 51).
+// kLanes lanes share an atom's list, entry k going to lane k mod kLanes, and add up their
+// sums in a fixed order: with one thread per atom a batch of some 20,000 atoms leaves
+// the chip two thirds idle.
+constexpr int kLanes = 8;
+
+__device__ __forceinline__ double lanes_sum(double x) {
+#pragma unroll
+    for (int o = 1; o < kLanes; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
 }
 
-__global__ void kb_cn(Work w, BW b, BConsts c) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= w.Nr) return;
+// n and dn/dt = sum_q f'(r)/r (d.u); per entry the coefficient c = f'(r)/r and its tangent
+// c (d.u) (-k1 rc (1 - 2 f)/r - 3)/r^2.  (The threads past the last atom repeat it.)
+__global__ void __launch_bounds__(128) kb_cn(Work w, BW b, BConsts c, const double* __restrict__ k1rc,
+                                            const double* __restrict__ exptab64) {
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = (int)(id % kLanes);
+    const bool live = id / kLanes < w.Nr;
+    const int64_t p = live ? id / kLanes : w.Nr - 1;
     const StructGeo& G = w.geo[w.sid[p]];
-    const ListView LV{w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn)};
+    const int64_t base = list_row(G.list_base_cn, p - G.atom_base, G.cap_cn);
     const int cnt = w.cnt_cn[p];
-    const double rki = w.pos64[p].w;
-    Dual n = dd(0.0);
-    LV.for_each(0, cnt, [&](int q) {
-        Dual d[3], r2;
-        ddist(w, b, p, q, d, r2);
-        if (!(r2.v < c.rc_cn2)) return;
-        const Dual rinv = inv(dsqrt(r2));
-        const double rc = rki + w.pos64[q].w;
-        const Dual t = dexp(-c.k1 * (rc * rinv + (-1.0)));
-        n += inv(t + 1.0);
-    });
-    b.n[p] = n;
+    const dbl4 x = w.pos64[p], ux = b.xd[p];
+    const double* krow = k1rc + (rec_tsrc(w, p) & 15) * c.T;
+    double n = 0.0, nt = 0.0;
+    for (int k = lane; k < cnt; k += kLanes) {
+        const int q = __ldg(w.nbr_cn + base + list_off(k));
+        const dbl4 y = w.pos64[q];
+        const double dx = y.x - x.x, dy = y.y - x.y, dz = y.z - x.z;
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        double2 o = make_double2(0.0, 0.0);
+        if (r2 < c.rc_cn2) {
+            const dbl4 uq = b.xd[q];
+            const double du = fma(dx, uq.x - ux.x, fma(dy, uq.y - ux.y, dz * (uq.z - ux.z)));
+            const double rinv = __double2hiint(r2) > 0x00100000 ? rsqrt64(r2) : 1.0 / sqrt(r2);
+            const double a = krow[rec_tsrc(w, q) & 15];
+            const double t = exp64(fma(-a, rinv, c.k1), exptab64);
+            const double f = rcp64(1.0 + t);
+            const double ri2 = rinv * rinv, ar = a * rinv;
+            o.x = -(ar * ri2) * (t * f * f);
+            const double s = o.x * du;
+            o.y = s * (ri2 * fma(fma(2.0, f, -1.0), ar, -3.0));
+            n += f;
+            nt += s;
+        }
+        if (live) b.cc[base + list_off(k)] = o;
+    }
+    n = lanes_sum(n);
+    nt = lanes_sum(nt);
+    if (live && lane == 0) b.n[p] = Dual{n, nt};
 }
 
 template <int R>
@@ -195,58 +224,115 @@ __global__ void kb_weights(Work w, BW b, BConsts c, const double* __restrict__ c
     }
 }
 
+// Dispersion pass.  With i6 = 1/(r^6 + R^6), i8 = 1/(r^8 + R^8) and x = r^2 (derivatives by x):
+//   g    = s6 i6 + s8 R0^2 i8                       g'   = -fc0/2
+//   fc0  = 6 s6 r^4 i6^2 + 8 s8 R0^2 r^6 i8^2       fc0' = 12 s6 r^2 i6^2 (3 R^6 i6 - 2)
+//                                                          + 24 s8 R0^2 r^4 i8^2 ((8 R^8 i8 - 5)/3)
+//   i6'  = -3 r^4 i6^2                              i8'  = -4 r^6 i8^2
+//   h    = 6 s6 R^5 i6^2 + 8 s8 R0^2 R^7 i8^2       (-dg/dR), h' = 12 s6 R^5 i6 i6' + 16 s8 R0^2 R^7 i8 i8'
+// An ordered pair adds -g dC6/dn to dE/dn, fc0 C6 d to the force and C6 (-i6, -R0^2 i8, R0 h, h)
+// to dE/d(s6, s8, a1, a2) (halved at the end).  Of the last two only gE times the value minus the
+// tangent is needed: the force's negative (F slot of b, its v part) and th's t part.
 // pairb[ti*T + tj] = (R0, R, R0^2, 0) in bohr
+constexpr int kBTab = 12;
 template <int R>
-__global__ void kb_disp(Work w, BW b, BConsts c, const dbl4* __restrict__ pairb) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= w.Nr) return;
+__global__ void __launch_bounds__(128) kb_disp(Work w, BW b, BConsts c, const dbl4* __restrict__ pairb,
+                                              const double* __restrict__ gE) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* tab = reinterpret_cast<double*>(smem_raw);
+    for (int k = threadIdx.x; k < c.T * c.T; k += blockDim.x) {
+        const dbl4 pb = pairb[k];
+        const double Rd = pb.y, R2 = Rd * Rd, R4 = R2 * R2, R6 = R4 * R2, R8 = R4 * R4, y = c.s8 * pb.z;
+        double* t = tab + kBTab * k;
+        t[0] = R6; t[1] = R8; t[2] = c.s6; t[3] = y;
+        t[4] = 6.0 * c.s6; t[5] = 8.0 * y;
+        t[6] = 6.0 * c.s6 * R4 * Rd; t[7] = 8.0 * y * R6 * Rd;
+        t[8] = 3.0 * R6; t[9] = 8.0 / 3.0 * R8;
+        t[10] = pb.x; t[11] = pb.z;
+    }
+    __syncthreads();
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = (int)(id % kLanes);
+    const bool live = id / kLanes < w.Nr;
+    const int64_t p = live ? id / kLanes : w.Nr - 1;
     const int ti = rec_tsrc(w, p) & 15;
+    const int s = w.sid[p];
+    const StructGeo& G = w.geo[s];
+    const int* row = w.nbr_disp + list_row(G.list_base_disp, p - G.atom_base, G.cap_disp);
+    const int cnt = w.cnt_disp[p];
+    const dbl4 x = w.pos64[p], ux = b.xd[p];
+    const double ge = gE[s];
     Dual Wi[R], dWi[R];
 #pragma unroll
     for (int a = 0; a < R; ++a) {
         Wi[a] = b.W[p * R + a];
         dWi[a] = b.dW[p * R + a];
     }
-    const StructGeo& G = w.geo[w.sid[p]];
-    const ListView LV{w.nbr_disp + list_row(G.list_base_disp, p - G.atom_base, G.cap_disp)};
-    const int cnt = w.cnt_disp[p];
-    Dual dn = dd(0.0), F[3] = {dd(0.0), dd(0.0), dd(0.0)}, th[4] = {dd(0.0), dd(0.0), dd(0.0), dd(0.0)};
-    LV.for_each(0, cnt, [&](int q) {
-        Dual d[3], r2;
-        ddist(w, b, p, q, d, r2);
-        if (!(r2.v < c.rc_disp2)) return;
+    const double* trow = tab + kBTab * ti * c.T;
+    const Dual* vb = b.v + (int64_t)ti * R;
+    const int vstride = c.T * R;
+    double dn = 0, dnt = 0, Gx = 0, Gy = 0, Gz = 0, t6 = 0, t6t = 0, t8 = 0, tR = 0, ta = 0;
+    for (int k = lane; k < cnt; k += kLanes) {
+        const int q = __ldg(row + list_off(k));
+        const dbl4 y = w.pos64[q];
+        const double dx = y.x - x.x, dy = y.y - x.y, dz = y.z - x.z;
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        if (!(r2 < c.rc_disp2)) continue;
         const int tsq = rec_tsrc(w, q);
-        const int src = tsq >> 4;
-        const dbl4 pb = pairb[ti * c.T + (tsq & 15)];
-        const double R0 = pb.x, Rd = pb.y, R0sq = pb.z;
-        const double R2 = Rd * Rd, R4 = R2 * R2, R6 = R4 * R2, R8 = R4 * R4;
-        Dual C6 = dd(0.0), dC6 = dd(0.0);
+        const dbl4 uq = b.xd[q];
+        const double vx = uq.x - ux.x, vy = uq.y - ux.y, vz = uq.z - ux.z;
+        const double du = fma(dx, vx, fma(dy, vy, dz * vz));  // d(r^2)/dt / 2
+        const double* t = trow + kBTab * (tsq & 15);
+        const Dual* vq = vb + (int64_t)(tsq >> 4) * vstride;
+        double C = 0, Ct = 0, D = 0, Dt = 0;
 #pragma unroll
         for (int a = 0; a < R; ++a) {
-            const Dual vq = b.v[((int64_t)src * c.T + ti) * R + a];
-            C6 += Wi[a] * vq;
-            dC6 += dWi[a] * vq;
+            const Dual v = vq[a];
+            C = fma(Wi[a].v, v.v, C);
+            Ct = fma(Wi[a].v, v.t, fma(Wi[a].t, v.v, Ct));
+            D = fma(dWi[a].v, v.v, D);
+            Dt = fma(dWi[a].v, v.t, fma(dWi[a].t, v.v, Dt));
         }
-        const Dual r4 = r2 * r2, r6 = r4 * r2, r8 = r4 * r4;
-        const Dual i6 = inv(r6 + R6), i8 = inv(r8 + R8);
-        const Dual t6 = c.s6 * i6, t8 = (c.s8 * R0sq) * i8;
-        const Dual g = t6 + t8;
-        dn += -(g * dC6);
-        const Dual fc = C6 * (6.0 * (r4 * (t6 * i6)) + 8.0 * (r6 * (t8 * i8)));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) F[a] += fc * d[a];
-        // derivatives of this ordered instance's energy -C6 g (halved at the end)
-        th[0] += -(C6 * i6);
-        th[1] += -(R0sq * (C6 * i8));
-        const Dual dR = C6 * ((c.s6 * 6.0 * R4 * Rd) * (i6 * i6) + (c.s8 * R0sq * 8.0 * R6 * Rd) * (i8 * i8));
-        th[2] += R0 * dR;
-        th[3] += dR;
-    });
-    b.dEdn[p] = dn;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) b.F[3 * p + a] = F[a];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) b.th[4 * p + m] = 0.5 * th[m];
+        const double r4 = r2 * r2, r6 = r4 * r2;
+        const double d6 = r6 + t[0], d8 = fma(r4, r4, t[1]);
+        const double pinv = rcp64(d6 * d8);
+        const double i6 = d8 * pinv, i8 = d6 * pinv;
+        const double g = fma(t[3], i8, t[2] * i6);
+        const double a6 = r2 * i6, A6 = a6 * a6, e8 = i8 * i8, B8 = r6 * e8;  // r^4 i6^2, r^6 i8^2
+        const double fc0 = fma(t[5], B8, t[4] * A6);
+        const double P6 = i6 * a6 * fma(t[8], i6, -2.0), P8 = r4 * e8 * fma(t[9], i8, -5.0 / 3.0);
+        const double fc1 = fma(3.0 * t[5], P8, 2.0 * t[4] * P6);
+        const double h = fma(t[7], e8, t[6] * (i6 * i6));
+        const double h1 = fma(4.0 * t[7], i8 * B8, 3.0 * t[6] * (i6 * A6));  // -h'/2
+        dn = fma(-g, D, dn);
+        dnt = fma(-g, Dt, dnt);
+        dnt = fma(fc0 * du, D, dnt);
+        // gE (value) - (tangent): Cv of C6, Cd of the 2 d.u that multiplies derivatives
+        const double Cv = fma(ge, C, -Ct), Cd = 2.0 * du * C;
+        const double fc = C * fc0;
+        const double A = -fma(Cv, fc0, -Cd * fc1);  // tangent - gE (value) of the force coefficient
+        Gx = fma(A, dx, fma(fc, vx, Gx));
+        Gy = fma(A, dy, fma(fc, vy, Gy));
+        Gz = fma(A, dz, fma(fc, vz, Gz));
+        t6 = fma(i6, Cv, t6);
+        t6t = fma(A6, Cd, t6t);
+        t8 = fma(t[11], fma(i8, Cv, 4.0 * B8 * Cd), t8);
+        const double z = fma(h, Cv, 2.0 * h1 * Cd);
+        ta = fma(t[10], z, ta);
+        tR += z;
+    }
+    dn = lanes_sum(dn); dnt = lanes_sum(dnt);
+    Gx = lanes_sum(Gx); Gy = lanes_sum(Gy); Gz = lanes_sum(Gz);
+    t6 = lanes_sum(fma(3.0, t6t, t6)); t8 = lanes_sum(t8); ta = lanes_sum(ta); tR = lanes_sum(tR);
+    if (!live || lane != 0) return;
+    b.dEdn[p] = Dual{dn, dnt};
+    b.F[3 * p] = Dual{Gx, 0.0};
+    b.F[3 * p + 1] = Dual{Gy, 0.0};
+    b.F[3 * p + 2] = Dual{Gz, 0.0};
+    b.th[4 * p] = Dual{0.0, 0.5 * t6};
+    b.th[4 * p + 1] = Dual{0.0, 0.5 * t8};
+    b.th[4 * p + 2] = Dual{0.0, -0.5 * ta};
+    b.th[4 * p + 3] = Dual{0.0, -0.5 * tR};
 }
 
 // ---- mixed form of the dispersion pass of the backward: the same dual-number
@@ -390,37 +476,40 @@ __global__ void __launch_bounds__(128) kb_disp_mixed(Work w, BW b, BConsts c, co
     for (int m = 0; m < 4; ++m) b.th[4 * p + m] = Dual{0.5 * thv[m].value(), 0.5 * tht[m].value()};
 }
 
-__global__ void kb_chain(Work w, BW b, BConsts c, const double* __restrict__ gE, double* __restrict__ dLdx) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= w.Nr) return;
+// Chain rule: dLdx = -gE F + dF/dt, both from the stored coefficients and tangents.
+__global__ void __launch_bounds__(128) kb_chain(Work w, BW b, BConsts c, const double* __restrict__ gE,
+                                               double* __restrict__ dLdx) {
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = (int)(id % kLanes);
+    const bool live = id / kLanes < w.Nr;
+    const int64_t p = live ? id / kLanes : w.Nr - 1;
     const int s = w.sid[p];
     const StructGeo& G = w.geo[s];
-    const ListView LV{w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn)};
+    const int64_t base = list_row(G.list_base_cn, p - G.atom_base, G.cap_cn);
     const int cnt = w.cnt_cn[p];
-    const double rki = w.pos64[p].w;
+    const dbl4 x = w.pos64[p], ux = b.xd[p];
     const Dual dni = b.dEdn[p];
-    Dual F[3] = {b.F[3 * p], b.F[3 * p + 1], b.F[3 * p + 2]};
-    LV.for_each(0, cnt, [&](int q) {
-        Dual d[3], r2;
-        ddist(w, b, p, q, d, r2);
-        if (!(r2.v < c.rc_cn2)) return;
-        const int src = rec_tsrc(w, q) >> 4;
-        const Dual rinv = inv(dsqrt(r2));
-        const double rc = rki + w.pos64[q].w;
-        const Dual t = dexp(-c.k1 * (rc * rinv + (-1.0)));
-        const Dual f = inv(t + 1.0);
-        const Dual dfdr = (-c.k1 * rc) * (rinv * rinv * t * f * f);
-        const Dual coef = (dni + b.dEdn[src]) * dfdr * rinv;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) F[a] += coef * d[a];
-    });
-    if (dLdx) {
-        const double u = kHartreeEV / kBohrA;
-        const double ge = gE[s];
-        const int i = w.perm[p];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) dLdx[3 * (int64_t)i + a] = (-ge * F[a].v + F[a].t) * u;
+    const double ge = gE[s];
+    double Gx = 0, Gy = 0, Gz = 0;
+    for (int k = lane; k < cnt; k += kLanes) {
+        const double2 cc = b.cc[base + list_off(k)];
+        if (__double_as_longlong(cc.x) == 0) continue;  // outside R_cn
+        const int q = __ldg(w.nbr_cn + base + list_off(k));
+        const dbl4 y = w.pos64[q], uq = b.xd[q];
+        const Dual dq = b.dEdn[rec_tsrc(w, q) >> 4];
+        const double S = dni.v + dq.v, cv = S * cc.x;
+        const double A = fma(dni.t + dq.t, cc.x, fma(S, cc.y, -ge * cv));
+        Gx = fma(A, y.x - x.x, fma(cv, uq.x - ux.x, Gx));
+        Gy = fma(A, y.y - x.y, fma(cv, uq.y - ux.y, Gy));
+        Gz = fma(A, y.z - x.z, fma(cv, uq.z - ux.z, Gz));
     }
+    Gx = lanes_sum(Gx); Gy = lanes_sum(Gy); Gz = lanes_sum(Gz);
+    if (!live || lane != 0) return;
+    const double u = kHartreeEV / kBohrA;
+    double* o = dLdx + 3 * (int64_t)w.perm[p];
+    o[0] = (b.F[3 * p].v + Gx) * u;
+    o[1] = (b.F[3 * p + 1].v + Gy) * u;
+    o[2] = (b.F[3 * p + 2].v + Gz) * u;
 }
 
 // ---- mixed form of the CN, weight and chain passes of the backward
@@ -649,13 +738,13 @@ inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 template <int R>
 cudaError_t backward_impl(const Work& w, const Consts& cc, const double* c6d, const dbl4* pairb, const double* cnref,
                           const int* nref, const Tabs& tbm, const double* gE, const double* gF, double* dLdp,
-                          double* dLdx, double* scratch, int B, bool mixed, cudaStream_t st) {
-    BW b = carve(scratch, w.Nr, w.ghost_cap, w.T, R, B);
+                          double* dLdx, double* scratch, int64_t list_cn, int B, bool mixed, cudaStream_t st) {
+    BW b = carve(scratch, w.Nr, w.ghost_cap, mixed ? 0 : list_cn, w.T, R, B);
     BConsts c{cc.rc_disp2, cc.rc_cn2, cc.k1, cc.k3, cc.s6, cc.s8, cc.T, R};
     const int TB = 128;
     if (w.Nr > 0) {
         // tangent positions for real atoms and every image actually built
-        kb_xdot<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w, b, gF, w.Nr + w.ghost_cap);
+        kb_xdot<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w, b, gF, w.Nr + w.ghost_cap, mixed);
         if (mixed) {
             kb_cn_mixed<<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, cc, tbm.rcpair, tbm.exptab);
             kb_weights_mixed<R><<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, cc, tbm.cnref2, tbm.dcr, tbm.nref,
@@ -663,10 +752,11 @@ cudaError_t backward_impl(const Work& w, const Consts& cc, const double* c6d, co
             kb_disp_mixed<R><<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, c, pairb);
             kb_chain_mixed<<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, cc, tbm.rcpair, tbm.exptab, gE, dLdx);
         } else {
-            kb_cn<<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, c);
+            const unsigned nl = nblk(w.Nr * kLanes, TB);
+            kb_cn<<<nl, TB, 0, st>>>(w, b, c, tbm.k1rc, tbm.exptab64);
             kb_weights<R><<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, c, cnref, nref, c6d);
-            kb_disp<R><<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, c, pairb);
-            kb_chain<<<nblk(w.Nr, TB), TB, 0, st>>>(w, b, c, gE, dLdx);
+            kb_disp<R><<<nl, TB, (size_t)c.T * c.T * kBTab * sizeof(double), st>>>(w, b, c, pairb, gE);
+            if (dLdx) kb_chain<<<nl, TB, 0, st>>>(w, b, c, gE, dLdx);
         }
     }
     kb_struct_sum<<<B, 256, 0, st>>>(w, b);
@@ -676,20 +766,21 @@ cudaError_t backward_impl(const Work& w, const Consts& cc, const double* c6d, co
 
 }  // namespace
 
-int64_t backward_scratch_doubles(const Work& w, int B) {
+int64_t backward_scratch_doubles(const Work& w, int B, int64_t list_cn, bool mixed) {
     const int64_t Nr = w.Nr, Ng = w.ghost_cap;
     const int64_t duals = Nr * (1 + 2 * (int64_t)w.R + (int64_t)w.T * w.R + 1 + 3 + 4);
     const int64_t rp = w.R <= 4 ? 4 : 8;
-    // duals, tangent positions, per-structure sums, FP32 v rows and tangents (+ alignment)
-    return 2 * duals + 3 * (Nr + Ng) + 8 * (int64_t)B + Nr * (int64_t)w.T * rp + 2 * (Nr + Ng) + Nr + 64;
+    // tangent positions, CN coefficients (FP64 form), duals, per-structure sums, FP32 v rows and tangents (+ alignment)
+    return 4 * (Nr + Ng) + (mixed ? 0 : 2 * list_cn) + 2 * duals + 8 * (int64_t)B + Nr * (int64_t)w.T * rp +
+           2 * (Nr + Ng) + Nr + 64;
 }
 
 cudaError_t launch_backward(const Work& w, const Consts& c, const double* c6d, const dbl4* pairb,
                             const double* cnref, const int* nref, const Tabs& tbm, const double* dLdE,
-                            const double* dLdF, double* dLdp, double* dLdx, double* scratch, int B, bool mixed,
-                            cudaStream_t st) {
+                            const double* dLdF, double* dLdp, double* dLdx, double* scratch, int64_t list_cn, int B,
+                            bool mixed, cudaStream_t st) {
 #define D3_BWD(RR) \
-    return backward_impl<RR>(w, c, c6d, pairb, cnref, nref, tbm, dLdE, dLdF, dLdp, dLdx, scratch, B, mixed, st)
+    return backward_impl<RR>(w, c, c6d, pairb, cnref, nref, tbm, dLdE, dLdF, dLdp, dLdx, scratch, list_cn, B, mixed, st)
     switch (c.R) {
         case 1: D3_BWD(1);
         case 2: D3_BWD(2);
