@@ -55,6 +55,8 @@ constexpr int kEvents = kStages + 3;  // kStages + 1 stage boundaries, 2 around 
 constexpr int32_t kDefaultShape[4] = {64, 128, 128, 16};
 constexpr int32_t kBlockCand[2] = {64, 128};
 constexpr int32_t kBuildCand[2] = {8, 16};
+constexpr int64_t kStructCells = 12000;  // cells that a block counts in shared memory (two blocks per SM)
+constexpr double kStructItems = 4500.0;  // build_by_struct
 constexpr int64_t kTuneMinAtoms = 16384;  // below this launch overhead decides, not the shape
 constexpr int kTuneReps = 3;
 
@@ -140,6 +142,8 @@ struct Plan {
     std::vector<double> cells;
     std::vector<int32_t> pbc;
     std::vector<StructGeo> geo;
+    int64_t max_ncell = 0;   // cells of the largest grid
+    std::vector<double> ghost_est;  // [B] estimated images
     std::vector<double> cap_est;  // [2 B] estimated CN and cluster list capacities
     int64_t Nr = 0, ncells = 0, list_disp = 0, list_cn = 0, list_cl = 0, ncl = 0;
     int ghost_cap = 0;
@@ -404,6 +408,7 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
     P.geo.assign(B, StructGeo{});
     ghost_est.assign(B, 0.0);
     P.cap_est.assign(2 * (size_t)B, 0.0);
+    P.max_ncell = 0;
     // structures streamed through one handle are alike: start from the ratios of the earlier ones, so
     // that the sizing pass rarely has to regrow and build again (up to a size where memory matters)
     const bool learn = offsets[B] <= ((int64_t)1 << 18);
@@ -480,7 +485,8 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
             G.ext_hif[k] = (float)G.ext_hi[k];
         }
         G.cell_base = cell_base;
-        cell_base += nc_total;
+        cell_base += nc_total + 1;  // and the end of the last cell
+        P.max_ncell = std::max<int64_t>(P.max_ncell, nc_total);
         G.atom_base = offsets[s];
         G.natoms = (int32_t)n;
         const double vol = std::fabs(det);  // bohr^3
@@ -553,6 +559,7 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     w.blk_chain = h->shape[2];
     w.build_per_sm = h->shape[3];
     w.max_natoms = maxn;
+    w.max_ncell = (int)std::min<int64_t>(P.max_ncell, 1 << 26);
     w.n_fin = nfin;
     // Lists longer than this are split over a block (k_disp_cl_split) where clusters are few: 64
     // entries (one chunk) when every warp of the chip could take a part, up to 1024 while a single
@@ -777,7 +784,7 @@ d3_status enqueue_build(d3_handle* h, Plan& P, const double* pos, const int32_t*
     }
     e = launch_build_impl(w, pos, types, h->d_rk, P.bsum, st, lmarks);
     if (e != cudaSuccess) return cuda_fail(h, e, "neighbour build launch");
-    if (P.Nr > 0) h->launches += kBuildLaunches;
+    if (P.Nr > 0) h->launches += P.w.by_struct ? kStructBuildLaunches : kBuildLaunches;
     return D3_OK;
 }
 
@@ -836,7 +843,7 @@ d3_status tune_shapes(d3_handle* h, Plan& P, const double* pos, const int32_t* t
             if (e == cudaSuccess) e = launch_forward(w, c, mixed, tb, E, F, W, nullptr, nullptr, nullptr, P.B, st,
                                                      ev.data() + 1);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            h->launches += kBuildLaunches + kForwardLaunches + c.atm + w.cl_mode;
+            h->launches += (w.by_struct ? kStructBuildLaunches : kBuildLaunches) + kForwardLaunches + c.atm + w.cl_mode;
             const int from[4] = {0, 1, 3, 5};
             for (int m = 0; m < 4 && e == cudaSuccess; ++m) {
                 float ms = 0.f;
@@ -865,6 +872,20 @@ d3_status tune_shapes(d3_handle* h, Plan& P, const double* pos, const int32_t* t
     return D3_OK;
 }
 
+// Whether one block per structure builds the batch (k_build_struct): it costs about 10 ns
+// per atom or image of the largest structure (and of an SM's share of the batch) and saves
+// seven kernels, some 50 us, so the line lies at 4,500 of them; the images of a structure are
+// its share, by the estimates, of those counted.  Not with list reuse, where most calls only
+// refill the positions.
+int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
+    if (h->prm.skin_A > 0 || P.max_ncell > kStructCells) return 0;
+    double est = 0.0, most = 0.0;
+    for (double x : P.ghost_est) est += x;
+    const double share = est > 0 ? gcount / est : 0.0;
+    for (int s = 0; s < P.B; ++s) most = std::max(most, P.geo[s].natoms + share * P.ghost_est[s]);
+    return most <= kStructItems && (double)P.Nr + gcount <= kStructItems * P.w.num_sms ? 1 : 0;
+}
+
 // Make the plan match the geometry; on a new geometry run the build once
 // synchronously and grow image and list capacities until nothing overflows.
 // *built: the sizing pass left the lists of these positions (the caller need not build again).
@@ -882,11 +903,10 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         P.cells.assign(cells, cells + 9 * (size_t)B);
         P.pbc.assign(pbc, pbc + 3 * (size_t)B);
         P.Nr = offsets[B];
-        std::vector<double> gest;
-        d3_status s = plan_geometry(h, P, B, offsets, cells, pbc, gest);
+        d3_status s = plan_geometry(h, P, B, offsets, cells, pbc, P.ghost_est);
         if (s != D3_OK) return s;
         double g = 64.0;
-        for (double x : gest) g += 1.15 * x + 8.0;
+        for (double x : P.ghost_est) g += 1.15 * x + 8.0;
         if (g > 2.0e9) return fail(h, D3_ERR_ARG, "too many periodic images");
         P.ghost_cap = (int)g;
         s = plan_alloc(h, P, st);
@@ -934,6 +954,7 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
             // image rows of v and dv are copies of their source's when that is cheap
             // (few images, or few types); otherwise the pass resolves each image's source
             P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
+            P.w.by_struct = build_by_struct(h, P, gcount);
             if (mode == kClusterLists) {
                 P.split_on = 0;
                 // (with more clusters the long lists hide behind the others, and leaving them out costs 2%)
@@ -1552,9 +1573,8 @@ d3_status d3_list_stats(d3_handle* h, int64_t* stats) {
     };
     stats[0] = P.Nr;
     int ng = 0;
-    if (e == cudaSuccess && P.ncells > 0)
-        e = cudaMemcpy(&ng, P.w.start_ghost + P.ncells, sizeof(int), cudaMemcpyDeviceToHost);
-    stats[1] = ng;
+    if (e == cudaSuccess && P.Nr > 0) e = cudaMemcpy(&ng, P.w.ghost_count, sizeof(int), cudaMemcpyDeviceToHost);
+    stats[1] = std::min(ng, P.ghost_cap);
     stats[2] = P.ncl;
     const bool cl = P.last_mode == kClusterLists;
     if (cl) sum_ints(P.w.cnt_cl, P.ncl, &stats[3]);

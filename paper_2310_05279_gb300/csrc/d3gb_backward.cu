@@ -107,7 +107,7 @@ struct BConsts {
 // (FP32 for the mixed form, else FP64)
 __global__ void kb_xdot(Work w, BW b, const double* __restrict__ gF, int64_t nt, bool mixed) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nt || q >= w.Nr + w.start_ghost[w.ncells]) return;
+    if (q >= nt || q >= w.Nr + min(*w.ghost_count, w.ghost_cap)) return;
     const int src = rec_tsrc(w, q) >> 4;
     const int i = w.perm[src];
     double t[3];

@@ -76,16 +76,12 @@ __device__ __forceinline__ void add_lattice(double (&x)[3], const StructGeo& G, 
     }
 }
 
-// Wrap into the cell, bin, and record each structure's occupied fractional
-// range per periodic axis (as float bits: the fractions are >= 0).  The
-// lattice translation that wraps an atom is chosen from its FP32 fractional
-// coordinates; the wrapped position is x - sum_k n_k H_k in FP64 (x itself
-// when the atom is inside the cell).
-__global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__ pos, const int32_t* __restrict__ types) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= w.Nr || skip_build(w)) return;
-    const int s = w.sid_in[i];
-    const StructGeo& G = w.geo[s];
+// Wrap atom i into the cell and bin it: fills f (fractional coordinates), stores the
+// wrapped position, cell and in-cell key, returns the cell.  The lattice translation that
+// wraps an atom is chosen from its FP32 fractional coordinates; the wrapped position is
+// x - sum_k n_k H_k in FP64 (x itself when the atom is inside the cell).
+__device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int64_t i, const double* __restrict__ pos,
+                                         const int32_t* __restrict__ types, float (&f)[3]) {
     double xb[3];
     bool fin = true;
 #pragma unroll
@@ -100,7 +96,6 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
     const int t = types[i];
     if (t < 0 || t >= w.T) atomicOr(w.status, ST_TYPE);
     const float xf[3] = {(float)xb[0], (float)xb[1], (float)xb[2]};
-    float f[3];
     int n[3] = {0, 0, 0};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -139,6 +134,18 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
     const int cid = cell_id(G, f, &key);
     w.cell_of[i] = cid;
     w.skey[i] = key;
+    return cid;
+}
+
+// The same for every atom of the batch, with each structure's occupied fractional range
+// per periodic axis (as float bits: the fractions are >= 0).
+__global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__ pos, const int32_t* __restrict__ types) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= w.Nr || skip_build(w)) return;
+    const int s = w.sid_in[i];
+    const StructGeo& G = w.geo[s];
+    float f[3];
+    const int cid = wrap_atom(w, G, i, pos, types, f);
     w.slot_of[i] = atomicAdd(&w.cnt_real[cid], 1);
     // occupied range: one atomic per group of lanes in the same structure
     const unsigned grp = __match_any_sync(__activemask(), s);
@@ -157,42 +164,73 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
 
 // Periodic images that can be within the list radius of a real atom: along a
 // periodic axis an image is kept when its fraction lies within delta (list
-// radius / plane spacing) of the structure's occupied range.  Slots are
-// reserved once per block (each thread counts, the block scans, one atomic).
-__global__ void __launch_bounds__(256) k_images(Work w) {
-    if (skip_build(w)) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = i < w.Nr;
-    const int s = live ? w.sid_in[i] : 0;
-    const StructGeo& G = w.geo[s];
-    float f[3] = {0, 0, 0};
+// radius / plane spacing) of the structure's occupied range [omin, omax] (float bits).
+struct ImageRange {
     int nlo[3] = {0, 0, 0}, nhi[3] = {0, 0, 0};
     float u0[3] = {0, 0, 0};
-    if (live) {
+    int count = 0;
+    __device__ ImageRange() {}
+    __device__ ImageRange(const Work& w, const StructGeo& G, int64_t i, const int* omin_bits, const int* omax_bits) {
+        float f[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             f[k] = w.fw[3 * i + k];
             u0[k] = (f[k] - G.lof[k]) * G.fscalef[k];
             if (G.img[k] > 0) {
                 const float delta = G.ext_hif[k] - 1.0f;
-                const float omin = __int_as_float(w.frange[3 * s + k]);
-                const float omax = __int_as_float(w.frange[3 * (w.B + s) + k]);
+                const float omin = __int_as_float(omin_bits[k]);
+                const float omax = __int_as_float(omax_bits[k]);
                 nlo[k] = max(-G.img[k], (int)ceilf(fmaxf(G.ext_lof[k], omin - delta) - f[k]));
                 nhi[k] = min(G.img[k], min((int)ceilf(G.ext_hif[k] - f[k]) - 1, (int)floorf(omax + delta - f[k])));
             }
         }
+        if (nhi[0] >= nlo[0] && nhi[1] >= nlo[1] && nhi[2] >= nlo[2])
+            // the identity is always inside the range; it is the atom itself
+            count = (nhi[0] - nlo[0] + 1) * (nhi[1] - nlo[1] + 1) * (nhi[2] - nlo[2] + 1) - 1;
     }
-    int mine = 0;
-    if (live && nhi[0] >= nlo[0] && nhi[1] >= nlo[1] && nhi[2] >= nlo[2]) {
-        mine = (nhi[0] - nlo[0] + 1) * (nhi[1] - nlo[1] + 1) * (nhi[2] - nlo[2] + 1);
-        // the identity is always inside the range; it is the atom itself
-        mine -= 1;
+    // the image records of atom i of structure s from slot on, counted per cell in cnt[cell - c0]
+    __device__ void emit(const Work& w, const StructGeo& G, int64_t i, int s, int slot, int* cnt, int c0) const {
+        auto cell_of_axis = [&](int k, int n) {
+            const int c = (int)floorf(u0[k] + (float)n * G.fscalef[k]);
+            return min(max(c, 0), G.ncell[k] - 1);
+        };
+        for (int n0 = nlo[0]; n0 <= nhi[0]; ++n0) {
+            const int cx = cell_of_axis(0, n0);
+            for (int n1 = nlo[1]; n1 <= nhi[1]; ++n1) {
+                const int cy = cell_of_axis(1, n1);
+                for (int n2 = nlo[2]; n2 <= nhi[2]; ++n2) {
+                    if (n0 == 0 && n1 == 0 && n2 == 0) continue;
+                    if (slot >= w.ghost_cap) {
+                        atomicOr(w.status, ST_GHOST_CAP);
+                        return;
+                    }
+                    const int cz = cell_of_axis(2, n2);
+                    const int gc = (int)cell_index(G, cx, cy, cz);
+                    w.ghost_src[slot] = (int)i;
+                    w.ghost_shift[slot] = pack_shift(n0, n1, n2);
+                    w.ghost_cell[slot] = gc;
+                    w.ghost_slot[slot] = atomicAdd(&cnt[gc - c0], 1);
+                    w.ghost_sid[slot] = s;
+                    ++slot;
+                }
+            }
+        }
     }
+};
+
+// Slots are reserved once per block (each thread counts, the block scans, one atomic).
+__global__ void __launch_bounds__(256) k_images(Work w) {
+    if (skip_build(w)) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = i < w.Nr;
+    const int s = live ? w.sid_in[i] : 0;
+    const StructGeo& G = w.geo[s];
+    const ImageRange img = live ? ImageRange(w, G, i, w.frange + 3 * s, w.frange + 3 * (w.B + s)) : ImageRange();
     // block scan of the counts
     __shared__ int wsum[8];
     __shared__ int base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int x = mine;
+    int x = img.count;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, o);
@@ -210,37 +248,11 @@ __global__ void __launch_bounds__(256) k_images(Work w) {
         base = acc > 0 ? atomicAdd(w.ghost_count, acc) : 0;
     }
     __syncthreads();
-    if (live) {  // the atom's image records are consecutive from here
-        w.gfirst[i] = base + wsum[wid] + x - mine;
-        w.gcnt[i] = mine > 0 ? mine : 0;
-    }
-    if (!live || mine <= 0) return;
-    int slot = base + wsum[wid] + x - mine;
-    auto cell_of_axis = [&](int k, int n) {
-        const int c = (int)floorf(u0[k] + (float)n * G.fscalef[k]);
-        return min(max(c, 0), G.ncell[k] - 1);
-    };
-    for (int n0 = nlo[0]; n0 <= nhi[0]; ++n0) {
-        const int cx = cell_of_axis(0, n0);
-        for (int n1 = nlo[1]; n1 <= nhi[1]; ++n1) {
-            const int cy = cell_of_axis(1, n1);
-            for (int n2 = nlo[2]; n2 <= nhi[2]; ++n2) {
-                if (n0 == 0 && n1 == 0 && n2 == 0) continue;
-                if (slot >= w.ghost_cap) {
-                    atomicOr(w.status, ST_GHOST_CAP);
-                    return;
-                }
-                const int cz = cell_of_axis(2, n2);
-                const int gc = (int)cell_index(G, cx, cy, cz);
-                w.ghost_src[slot] = (int)i;
-                w.ghost_shift[slot] = pack_shift(n0, n1, n2);
-                w.ghost_cell[slot] = gc;
-                w.ghost_slot[slot] = atomicAdd(&w.cnt_ghost[gc], 1);
-                w.ghost_sid[slot] = s;
-                ++slot;
-            }
-        }
-    }
+    if (!live) return;
+    const int slot = base + wsum[wid] + x - img.count;  // the atom's image records are consecutive from here
+    w.gfirst[i] = slot;
+    w.gcnt[i] = img.count;
+    if (img.count > 0) img.emit(w, G, i, s, slot, w.cnt_ghost, 0);
 }
 
 // ---- exclusive scan of int counts (n entries) into start[0..n], start[n] = total
@@ -354,34 +366,6 @@ __global__ void k_scatter(Work w) {
     w.ukey[k] = image_key(w, (int)g);
 }
 
-// Each slot's final place in its cell is the number of smaller keys in the cell
-// (one thread per slot; the threads of a cell read the same keys).  Writes the
-// sorted order and, for real atoms, its inverse (slot_of[i] = sorted slot of
-// input atom i; until here slot_of held the atoms' places in their cells).
-__global__ void __launch_bounds__(256) k_rank(Work w) {
-    if (skip_build(w)) return;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool real = t < w.Nr;
-    const int ng = min(*w.ghost_count, w.ghost_cap);
-    if (!real && t - w.Nr >= ng) return;
-    const int u = w.usrc[t];
-    const int c = real ? w.cell_of[u] : w.ghost_cell[u];
-    const int* start = real ? w.start_real : w.start_ghost;
-    const int64_t off = real ? 0 : w.Nr;
-    const int b = start[c], e = start[c + 1];
-    const long long mine = w.ukey[t];
-    const long long* key = w.ukey + off;
-    int rank = 0;
-    for (int m = b; m < e; ++m) rank += key[m] < mine ? 1 : 0;
-    if (real) {
-        w.sorted_src[b + rank] = u;
-        w.slot_of[u] = b + rank;
-    } else {
-        w.gsorted[b + rank] = u;
-        w.ginv[u] = b + rank;
-    }
-}
-
 // Zero the counters of a build (and count the build).
 __global__ void k_reset(Work w) {
     if (skip_build(w)) return;
@@ -464,57 +448,267 @@ __device__ inline void store_pos(Work& w, int64_t q, const double x[3], double r
     store_ipos(w, q, x, tsrc);
 }
 
-// Sorted positions: threads [0, Nr) fill the real atoms' slots, the next ones the
-// images'.  An image's FP64 position is its source's plus the lattice
-// translation; its split is the source's split plus the translation's (grid
-// parts add exactly), moved back to the nearest grid point (|lo| <= 2^-11) by
-// whole grid steps.
-__global__ void k_fill(Work w, const int32_t* __restrict__ types, const double* __restrict__ rk_tab) {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < w.Nr) {
-        const int i = w.sorted_src[p];
-        int t = types[i];
-        if (t < 0 || t >= w.T) t = 0;
-        w.perm[p] = i;
-        w.sid[p] = w.sid_in[i];
-        w.cell_sorted[p] = w.cell_of[i];
-        const double x[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
-        store_pos(w, p, x, rk_tab[t], t | ((int)p << 4));
-        return;
-    }
-    const int64_t q = p - w.Nr;
-    const int ng = w.start_ghost[w.ncells];
-    if (q >= ng) return;
-    const int g = w.gsorted[q];
+// Sorted slot p of real atom i.
+__device__ __forceinline__ void fill_real(Work& w, int64_t p, int i, int s, const int32_t* __restrict__ types,
+                                          const double* __restrict__ rk_tab) {
+    int t = types[i];
+    if (t < 0 || t >= w.T) t = 0;
+    w.perm[p] = i;
+    w.sid[p] = s;
+    w.cell_sorted[p] = w.cell_of[i];
+    const double x[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
+    store_pos(w, p, x, rk_tab[t], t | ((int)p << 4));
+}
+// Sorted image slot q of image record g.  An image's FP64 position is its source's plus
+// the lattice translation; its split is the source's (read from the source's record: forming
+// it again took 12 of 18 FP64 instructions an image, which bound the fill) plus the
+// translation's (grid parts add exactly), moved back to the nearest grid point (|lo| <=
+// 2^-11) by whole grid steps.
+__device__ __forceinline__ void fill_image(Work& w, int64_t q, int g, const StructGeo& G) {
     const int i = w.ghost_src[g];
     int n0, n1, n2;
     unpack_shift(w.ghost_shift[g], n0, n1, n2);
-    const StructGeo& G = w.geo[w.ghost_sid[g]];
-    int t = types[i];
-    if (t < 0 || t >= w.T) t = 0;
     const int ps = w.slot_of[i];  // the source's sorted slot (inverse permutation of the sort)
-    const double rk = rk_tab[t];
-    const double xs[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
-    double x[3] = {xs[0], xs[1], xs[2]};
+    const dbl4 xs = w.pos64[ps];
+    const float4 sh = w.rec[2 * (int64_t)ps], sl = w.rec[2 * (int64_t)ps + 1];
+    double x[3] = {xs.x, xs.y, xs.z};
     add_lattice(x, G, n0, n1, n2);
-    w.pos64[w.Nr + q] = dbl4_make(x[0], x[1], x[2], rk);
-    float sh[3], sl[3];  // the source's split, as its own slot holds it
-    split_pos(xs, sh, sl);
+    w.pos64[w.Nr + q] = dbl4_make(x[0], x[1], x[2], xs.w);
+    const float shv[3] = {sh.x, sh.y, sh.z}, slv[3] = {sl.x, sl.y, sl.z};
     const float f0 = (float)n0, f1 = (float)n1, f2 = (float)n2;
     float h[3], l[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        h[a] = sh[a] + (f0 * G.Hh[a] + f1 * G.Hh[3 + a] + f2 * G.Hh[6 + a]);
-        l[a] = sl[a] + (f0 * G.Hl[a] + f1 * G.Hl[3 + a] + f2 * G.Hl[6 + a]);
+        h[a] = shv[a] + (f0 * G.Hh[a] + f1 * G.Hh[3 + a] + f2 * G.Hh[6 + a]);
+        l[a] = slv[a] + (f0 * G.Hl[a] + f1 * G.Hl[3 + a] + f2 * G.Hl[6 + a]);
         const float m = rintf(l[a] * 1024.0f);
         h[a] += m * (1.0f / 1024.0f);
         l[a] -= m * (1.0f / 1024.0f);
     }
-    const int tsrc = t | (ps << 4);
+    const int tsrc = __float_as_int(sh.w);  // the source's type and slot
     w.rec[2 * (w.Nr + q)] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
-    w.rec[2 * (w.Nr + q) + 1] = make_float4(l[0], l[1], l[2], (float)rk);
+    w.rec[2 * (w.Nr + q) + 1] = make_float4(l[0], l[1], l[2], sl.w);
     w.hi[w.Nr + q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
     store_ipos(w, w.Nr + q, x, tsrc);
+}
+
+// Each slot's final place in its cell is the number of smaller keys in the cell
+// (one thread per slot; the threads of a cell read the same keys).  Writes the
+// sorted order and, for real atoms, its inverse (slot_of[i] = sorted slot of
+// input atom i; until here slot_of held the atoms' places in their cells) and the
+// atom's position records (with the lists kept, those alone).
+__global__ void __launch_bounds__(256) k_rank(Work w, const int32_t* __restrict__ types,
+                                              const double* __restrict__ rk_tab) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool real = t < w.Nr;
+    if (skip_build(w)) {
+        if (real) fill_real(w, t, w.sorted_src[t], w.sid[t], types, rk_tab);
+        return;
+    }
+    const int ng = min(*w.ghost_count, w.ghost_cap);
+    if (!real && t - w.Nr >= ng) return;
+    const int u = w.usrc[t];
+    const int c = real ? w.cell_of[u] : w.ghost_cell[u];
+    const int* start = real ? w.start_real : w.start_ghost;
+    const int64_t off = real ? 0 : w.Nr;
+    const int b = start[c], e = start[c + 1];
+    const long long mine = w.ukey[t];
+    const long long* key = w.ukey + off;
+    int rank = 0;
+    for (int m = b; m < e; ++m) rank += key[m] < mine ? 1 : 0;
+    if (real) {
+        w.sorted_src[b + rank] = u;
+        w.slot_of[u] = b + rank;
+        fill_real(w, b + rank, u, w.sid_in[u], types, rk_tab);
+    } else {
+        w.gsorted[b + rank] = u;
+        w.ginv[u] = b + rank;
+    }
+}
+
+// Position records of the images.
+__global__ void __launch_bounds__(256) k_fill(Work w) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= min(*w.ghost_count, w.ghost_cap)) return;
+    const int g = w.gsorted[q];
+    fill_image(w, q, g, w.geo[w.ghost_sid[g]]);
+}
+
+// ---- the steps above in one kernel, for batches of small structures
+// One block per structure: binning, occupied range, images, the scan of the cell counts
+// (in shared memory), the rank sort and the fill, with block barriers instead of kernel
+// boundaries.  Each structure takes a segment of the image slots (one atomic), so image
+// numbers depend on the order of the blocks; nothing else does: lists are walked by cell,
+// and the order inside a cell is by key.  Bound by latency (some ten
+// phases of a few dependent loads each, and FP64 conversions on one SM's pipe), so it pays
+// where launches count: 9 kernels of the steps above take 88 us on 128 x 1440 atoms and
+// 49 on 64 atoms, this 44 and 25; with 815 atoms and 3,970 images per structure and 256
+// structures 164 and 220.
+
+// exclusive scan of a[0, n) in place (all kStructThreads threads of the block)
+template <int kStructThreads>
+__device__ inline void block_scan_array(int* a, int n) {
+    __shared__ int wsum[kStructThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int per = (n + kStructThreads - 1) / kStructThreads;
+    const int b = min(n, (int)threadIdx.x * per), e = min(n, b + per);
+    int v = 0;
+    for (int k = b; k < e; ++k) v += a[k];
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        int t = lane < kStructThreads / 32 ? wsum[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < kStructThreads / 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        if (lane < kStructThreads / 32) wsum[lane] = t;
+    }
+    __syncthreads();
+    int run = x - v + (wid > 0 ? wsum[wid - 1] : 0);
+    for (int k = b; k < e; ++k) {
+        const int t = a[k];
+        a[k] = run;
+        run += t;
+    }
+    __syncthreads();
+}
+
+template <int kStructThreads>
+__global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build_struct(Work w, const double* __restrict__ pos,
+                                                                    const int32_t* __restrict__ types,
+                                                                    const double* __restrict__ rk_tab) {
+    extern __shared__ int counts[];  // [2][ncell + 1]: atoms and images per cell, then their starts
+    __shared__ int fr[6], seg[2], wsum[kStructThreads / 32];
+    const int s = blockIdx.x, tid = threadIdx.x;
+    const StructGeo& G = w.geo[s];
+    const int n = G.natoms;
+    const int64_t a0 = G.atom_base;
+    const int nc = G.ncell[0] * G.ncell[1] * G.ncell[2], c0 = (int)G.cell_base;
+    int* cr = counts;
+    int* cg = counts + nc + 1;
+    for (int k = tid; k < 2 * (nc + 1); k += kStructThreads) counts[k] = 0;
+    if (tid < 3) {  // minima start at a huge float, maxima at +0
+        fr[tid] = 0x7f7f7f7f;
+        fr[3 + tid] = 0;
+        w.maxcnt[3 * s + tid] = 0;
+    }
+    __syncthreads();
+    for (int k0 = 0; k0 < n; k0 += kStructThreads) {
+        const int k = k0 + tid;
+        const bool live = k < n;
+        float f[3] = {0.f, 0.f, 0.f};
+        if (live) {
+            const int64_t i = a0 + k;
+            const int cid = wrap_atom(w, G, i, pos, types, f);
+            w.slot_of[i] = atomicAdd(&cr[cid - c0], 1);
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if (!G.pbc[m]) continue;
+            const int lo = __reduce_min_sync(0xffffffffu, live ? __float_as_int(f[m]) : 0x7f7f7f7f);
+            const int hi = __reduce_max_sync(0xffffffffu, live ? __float_as_int(f[m]) : 0);
+            if ((tid & 31) == 0) {
+                atomicMin(&fr[m], lo);
+                atomicMax(&fr[3 + m], hi);
+            }
+        }
+    }
+    __syncthreads();
+    // images: the block's total first (one segment of slots), then the records
+    int mine = 0;
+    for (int k = tid; k < n; k += kStructThreads) mine += ImageRange(w, G, a0 + k, fr, fr + 3).count;
+    int x = mine;
+    const int lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (tid == 0) {
+        int acc = 0;
+        for (int k = 0; k < kStructThreads / 32; ++k) {
+            const int v = wsum[k];
+            wsum[k] = acc;
+            acc += v;
+        }
+        seg[0] = acc > 0 ? atomicAdd(w.ghost_count, acc) : 0;
+        seg[1] = max(0, min(acc, w.ghost_cap - seg[0]));
+    }
+    __syncthreads();
+    const int g0 = seg[0], ng = seg[1];
+    {
+        int slot = g0 + wsum[wid] + x - mine;  // a thread's atoms one after the other
+        for (int k = tid; k < n; k += kStructThreads) {
+            const ImageRange img(w, G, a0 + k, fr, fr + 3);
+            w.gfirst[a0 + k] = slot;
+            w.gcnt[a0 + k] = img.count;
+            if (img.count > 0) img.emit(w, G, a0 + k, s, slot, cg, c0);
+            slot += img.count;
+        }
+    }
+    __syncthreads();
+    block_scan_array<kStructThreads>(cr, nc + 1);
+    block_scan_array<kStructThreads>(cg, nc + 1);
+    for (int k = tid; k <= nc; k += kStructThreads) {
+        w.start_real[c0 + k] = (int)a0 + cr[k];
+        w.start_ghost[c0 + k] = g0 + cg[k];
+    }
+    // cell order (any order inside a cell) with the keys, then each slot's rank in its cell
+    for (int k = tid; k < n; k += kStructThreads) {
+        const int i = (int)a0 + k;
+        const int64_t d = a0 + cr[w.cell_of[i] - c0] + w.slot_of[i];
+        w.usrc[d] = i;
+        w.ukey[d] = real_key(w, i);
+    }
+    for (int k = tid; k < ng; k += kStructThreads) {
+        const int g = g0 + k;
+        const int64_t d = w.Nr + g0 + cg[w.ghost_cell[g] - c0] + w.ghost_slot[g];
+        w.usrc[d] = g;
+        w.ukey[d] = image_key(w, g);
+    }
+    __syncthreads();
+    for (int k = tid; k < n; k += kStructThreads) {
+        const int u = w.usrc[a0 + k];
+        const int c = w.cell_of[u] - c0, b = cr[c], e = cr[c + 1];
+        const long long key = w.ukey[a0 + k];
+        int rank = 0;
+        for (int m = b; m < e; ++m) rank += w.ukey[a0 + m] < key ? 1 : 0;
+        const int64_t p = a0 + b + rank;
+        w.sorted_src[p] = u;
+        w.slot_of[u] = (int)p;
+        fill_real(w, p, u, s, types, rk_tab);
+    }
+    __syncthreads();  // (the images read their sources' sorted slots)
+    for (int k = tid; k < ng; k += kStructThreads) {
+        const int u = w.usrc[w.Nr + g0 + k];
+        const int c = w.ghost_cell[u] - c0, b = cg[c], e = cg[c + 1];
+        const long long key = w.ukey[w.Nr + g0 + k];
+        int rank = 0;
+        for (int m = b; m < e; ++m) rank += w.ukey[w.Nr + g0 + m] < key ? 1 : 0;
+        const int q = g0 + b + rank;
+        w.gsorted[q] = u;
+        w.ginv[u] = q;
+        fill_image(w, q, u, G);
+    }
+}
+
+// Zero the batch's own counters of a build by structure (and count the build).
+__global__ void k_reset_struct(Work w) {
+    *w.ghost_count = 0;
+    w.work_ctr[0] = 0;
+    w.work_ctr[1] = 0;
+    w.work_ctr[2] = 0;
+    atomicAdd(w.nbuild, 1ull);
 }
 
 // ---- per-atom lists within the two list radii ------------------------------
@@ -528,6 +722,9 @@ __device__ __forceinline__ int64_t next_chunk(const Work& w, int lane, int ctr) 
     if (lane == 0) chunk = atomicAdd(w.work_ctr + ctr, 1);
     return (int64_t)__shfl_sync(0xffffffffu, chunk, 0);
 }
+// The clusters from both ends alternately: those of sparse rows at the edges of the
+// occupied cells span the row and take longest, and most of them come first or last.
+__device__ __forceinline__ int64_t from_both_ends(int64_t k, int64_t n) { return (k & 1) ? n - 1 - (k >> 1) : k >> 1; }
 
 // One warp takes 8 consecutive sorted atoms (as the cluster lists below) and walks the
 // union of their cell windows once: the rows of cells (real and image atoms of each row)
@@ -556,8 +753,9 @@ __global__ void __launch_bounds__(128) k_build_lists(Work w) {
     float4* ch = sh_ch[threadIdx.x >> 5];
     int* cq = sh_cq[threadIdx.x >> 5];
     for (;;) {
-        const int64_t I = next_chunk(w, lane, 0);
-        if (I >= w.ncl) return;
+        const int64_t next = next_chunk(w, lane, 0);
+        if (next >= w.ncl) return;
+        const int64_t I = from_both_ends(next, w.ncl);
         const int s = w.clu_sid[I];
         const StructGeo& G = w.geo[s];
         const int64_t p0 = G.atom_base + (I - G.clu_base) * kClusterAtoms;
@@ -759,8 +957,9 @@ __global__ void __launch_bounds__(128) k_build_clist(Work w) {
     float4* ch = sh_ch[threadIdx.x >> 5];
     int* cq = sh_cq[threadIdx.x >> 5];
     for (;;) {
-        const int64_t I = next_chunk(w, lane, 1);
-        if (I >= w.ncl) return;
+        const int64_t next = next_chunk(w, lane, 1);
+        if (next >= w.ncl) return;
+        const int64_t I = from_both_ends(next, w.ncl);
         const int s = w.clu_sid[I];
         const StructGeo& G = w.geo[s];
         const int64_t p0 = G.atom_base + (I - G.clu_base) * kClusterAtoms;
@@ -971,16 +1170,27 @@ cudaError_t launch_build_impl(const Work& w, const double* pos, const int32_t* t
                               int* bsum, cudaStream_t st, cudaEvent_t* lmarks) {
     if (w.Nr == 0) return cudaGetLastError();
     const int TB = 256;
-    const int64_t nreset = std::max<int64_t>(w.ncells + 1, 3 * (int64_t)w.B);
-    k_reset<<<nblk(nreset, TB), TB, 0, st>>>(w);
-    k_wrap<<<nblk(w.Nr, TB), TB, 0, st>>>(w, pos, types);
-    k_images<<<nblk(w.Nr, TB), TB, 0, st>>>(w);
-    const ScanPair sp{{w.cnt_real, w.cnt_ghost}, {w.start_real, w.start_ghost}};
-    const cudaError_t e = scan2(sp, bsum, w.ncells, w.gate, st);
-    if (e != cudaSuccess) return e;
-    k_scatter<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w);
-    k_rank<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w);
-    k_fill<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w, types, rk_tab);
+    if (w.by_struct) {
+        const size_t sm = 2 * sizeof(int) * ((size_t)w.max_ncell + 1);
+        const bool wide = w.B <= w.num_sms;  // a structure to itself on an SM takes twice the threads
+        const cudaError_t e = cudaFuncSetAttribute(wide ? k_build_struct<1024> : k_build_struct<512>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        k_reset_struct<<<1, 1, 0, st>>>(w);
+        if (wide) k_build_struct<1024><<<(unsigned)w.B, 1024, sm, st>>>(w, pos, types, rk_tab);
+        else k_build_struct<512><<<(unsigned)w.B, 512, sm, st>>>(w, pos, types, rk_tab);
+    } else {
+        const int64_t nreset = std::max<int64_t>(w.ncells + 1, 3 * (int64_t)w.B);
+        k_reset<<<nblk(nreset, TB), TB, 0, st>>>(w);
+        k_wrap<<<nblk(w.Nr, TB), TB, 0, st>>>(w, pos, types);
+        k_images<<<nblk(w.Nr, TB), TB, 0, st>>>(w);
+        const ScanPair sp{{w.cnt_real, w.cnt_ghost}, {w.start_real, w.start_ghost}};
+        const cudaError_t e = scan2(sp, bsum, w.ncells, w.gate, st);
+        if (e != cudaSuccess) return e;
+        k_scatter<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w);
+        k_rank<<<nblk(w.Nr + w.ghost_cap, TB), TB, 0, st>>>(w, types, rk_tab);
+        k_fill<<<nblk(w.ghost_cap, TB), TB, 0, st>>>(w);
+    }
     {
         // persistent warps: w.build_per_sm blocks per SM, work handed out per cluster
         const int bcl = (int)std::min<int64_t>((w.ncl + 3) / 4, (int64_t)w.num_sms * w.build_per_sm);

@@ -64,7 +64,7 @@ struct StructGeo {
     int win_cn[3];    // window half-width (cells) covering the CN list radius
     int img[3];       // image range, 0 along open axes
     int pbc[3];
-    int64_t cell_base;
+    int64_t cell_base;  // (one entry more than cells: the end of the last cell)
     int64_t atom_base;
     int32_t natoms;
     int32_t cap_disp, cap_cn;
@@ -132,6 +132,8 @@ struct Work {
     int* ghost_slot;         // [ghost_cap]
     int* ghost_sid;          // [ghost_cap] structure of the image
     int* ghost_count;        // [1]
+    int by_struct;           // build: 1 = one block per structure (k_build_struct), 0 = kernels over the batch
+    int max_ncell;           // cells of the largest grid
     int* sorted_src;         // [Nr] sorted -> input index
     int* gsorted;            // [ghost_cap] sorted image slot -> raw image record
     int* ginv;               // [ghost_cap] raw image record -> sorted image slot
@@ -368,4 +370,5 @@ constexpr int kForwardLaunches = 5;  // kernels per forward pass (B > 0, N > 0):
 constexpr int kBuildLaunches = 10;   // kernels per neighbour build (N > 0): reset, wrap, images, 3 scan (both
                                      // count arrays), scatter, rank (in-cell sort), fill, lists (per-atom or
                                      // cluster lists)
+constexpr int kStructBuildLaunches = 3;  // by structure: reset, build, lists
 }  // namespace d3gb
