@@ -115,10 +115,9 @@ void d3_destroy(d3_handle *h);
  * Takes effect for work enqueued afterwards on the handle's last stream. */
 d3_status d3_set_damping(d3_handle *h, double s6, double s8, double a1, double a2_bohr);
 
-/* Graph replay (default on): from the second call in a row for a geometry and
- * parameter set on, a compute call whose pointers match the captured one's is replayed as one
- * CUDA graph (captured once on an internal stream, launched on the caller's
- * stream), which removes the per-kernel launch overhead.  Calls made while
+/* Graph replay (default on): a compute call that repeats the previous one's
+ * geometry, pointers and parameters is replayed as one CUDA graph (captured
+ * once on an internal stream, launched on the caller's stream), which removes the per-kernel launch overhead.  Calls made while
  * profiling (d3_profile_enable) or while the caller's stream is being captured
  * enqueue their kernels directly.  on = 0 always enqueues directly.  Results
  * are identical either way. */

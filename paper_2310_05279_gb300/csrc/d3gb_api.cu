@@ -230,7 +230,7 @@ struct d3_handle {
     int64_t glaunches = 0;         // kernels in the captured call
     const void* gkey[10] = {};     // pointers and generations the graph was captured with
     int64_t plan_gen = 0, param_gen = 0;
-    int64_t last_gen[2] = {-1, -1};  // plan_gen and param_gen of the previous call
+    const void* lkey[10] = {};       // key of the previous call
     // list capacities the sizing passes settled on, over plan_geometry's estimates (largest ratio seen)
     double cap_ratio_cn = 1.0, cap_ratio_cl = 1.0;
     // launch shapes (d3_launch_shapes): chosen per size class by the autotuner unless fixed
@@ -788,6 +788,15 @@ d3_status enqueue_build(d3_handle* h, Plan& P, const double* pos, const int32_t*
     return D3_OK;
 }
 
+// Kernels of one forward pass over at least one atom: CN, dispersion (in cluster mode also its
+// finish, and the long lists where they are split off), chain, the per-structure sums, and the
+// three-body term.
+int forward_launches(const d3_handle* h, const Work& w, const Consts& c, int mode) {
+    int n = 3 + (w.max_natoms <= kFinChunk ? 1 : 2) + c.atm;
+    if (mode == kClusterLists) n += 1 + (h->prm.precision == D3_MIXED ? w.split_on : 0);
+    return n;
+}
+
 // The autotuner: once per size class, right after a new geometry is sized,
 // run the build and the forward passes kTuneReps times with each candidate
 // shape (alternating) and keep, per kernel, the candidate with the shortest
@@ -843,7 +852,7 @@ d3_status tune_shapes(d3_handle* h, Plan& P, const double* pos, const int32_t* t
             if (e == cudaSuccess) e = launch_forward(w, c, mixed, tb, E, F, W, nullptr, nullptr, nullptr, P.B, st,
                                                      ev.data() + 1);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            h->launches += (w.by_struct ? kStructBuildLaunches : kBuildLaunches) + kForwardLaunches + c.atm + w.cl_mode;
+            h->launches += (w.by_struct ? kStructBuildLaunches : kBuildLaunches) + forward_launches(h, w, c, mode);
             const int from[4] = {0, 1, 3, 5};
             for (int m = 0; m < 4 && e == cudaSuccess; ++m) {
                 float ms = 0.f;
@@ -884,6 +893,21 @@ int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
     const double share = est > 0 ? gcount / est : 0.0;
     for (int s = 0; s < P.B; ++s) most = std::max(most, P.geo[s].natoms + share * P.ghost_est[s]);
     return most <= kStructItems && (double)P.Nr + gcount <= kStructItems * P.w.num_sms ? 1 : 0;
+}
+
+// Whether the mixed form's CN pass (bit 0) and chain pass (bit 1) take 8 lanes per atom.
+// For few atoms one thread per atom is a chain of 0.55 us per list entry (64 atoms: CN pass
+// 37 us and 13 with 8 lanes, chain pass 18 and 12; 6,912 atoms: 36 and 15, 20 and 15). In
+// batches of different structures of several elements lists differ so much in length that
+// the lanes of a warp wait for one another, and the CN pass gains up to some 250,000 atoms
+// (64 structures, 63,709 atoms: 74 and 47 us; 256, 208,635 atoms: 150 and 128; 512, 497,680
+// atoms: 245 and 274); the chain pass does not (76 and 146 us on 208,635 atoms). With even
+// lists one thread per atom is the faster from some 50,000 atoms on (55,296 atoms in a box:
+// 43 and 48 us, 128 bilayers of 1440 atoms: 94 and 143).
+int wide_passes(const d3_handle* h, const Plan& P) {
+    if (h->prm.precision != D3_MIXED || P.Nr == 0) return 0;
+    if (P.Nr <= 32768) return 3;
+    return P.Nr <= 262144 && P.B >= 16 && h->T > 1 ? 1 : 0;
 }
 
 // Make the plan match the geometry; on a new geometry run the build once
@@ -955,6 +979,7 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
             // (few images, or few types); otherwise the pass resolves each image's source
             P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;
             P.w.by_struct = build_by_struct(h, P, gcount);
+            P.w.wide = wide_passes(h, P);
             if (mode == kClusterLists) {
                 P.split_on = 0;
                 // (with more clusters the long lists hide behind the others, and leaving them out costs 2%)
@@ -1014,20 +1039,19 @@ d3_status enqueue_forward(d3_handle* h, const double* pos, const int32_t* types,
     cudaError_t e = launch_forward(P.w, c, mixed, tb, E, F, W, e_atom, cn, w_atom, P.B, st,
                                    ev.size() == kEvents ? ev.data() + 1 : nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "forward launch");
-    h->launches += (P.Nr > 0 ? kForwardLaunches + c.atm + (mode == kClusterLists ? 1 : 0) : 1);
+    h->launches += P.Nr > 0 ? forward_launches(h, P.w, c, mode) : 1;
     if (ev.size() == kEvents) h->ev_pending.push_back(ev);
     else for (cudaEvent_t x : ev) h->ev_pool.push_back(x);
     return D3_OK;
 }
 
 // A call on a sized plan is the same sequence of kernels and memsets every time for
-// the same pointers and parameters, so it is captured once as a CUDA graph on an
-// internal stream and then replayed on the caller's stream with one launch.  The
-// first call of a geometry, or of a parameter set, enqueues its kernels directly:
-// capturing and instantiating a graph takes about 100 us of host time and pays only
-// when calls follow one another (a run whose cell changes in every call never gets
-// there).  Calls made while profiling, or while the caller's stream is itself being
-// captured, enqueue directly.
+// the same pointers and parameters.  When a call repeats the previous one's, that
+// sequence is captured once as a CUDA graph on an internal stream and then replayed
+// on the caller's stream with one launch.  A call that does not (other buffers, a new
+// geometry, new parameters) enqueues its kernels directly: capturing and instantiating
+// a graph takes about 100 us of host time and pays only when it is replayed.  Calls made
+// while profiling, or while the caller's stream is itself being captured, enqueue directly.
 bool same_key(const void* const (&a)[10], const void* const (&b)[10]) {
     for (int i = 0; i < 10; ++i)
         if (a[i] != b[i]) return false;
@@ -1057,9 +1081,8 @@ d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const d
         return direct();
     const void* key[10] = {pos, types, E, F, W, e_atom, cn, w_atom, (const void*)(intptr_t)h->plan_gen,
                            (const void*)(intptr_t)(h->param_gen * 2 + (h->accumulate ? 1 : 0))};
-    const bool again = h->last_gen[0] == h->plan_gen && h->last_gen[1] == h->param_gen;  // as in the previous call
-    h->last_gen[0] = h->plan_gen;
-    h->last_gen[1] = h->param_gen;
+    const bool again = same_key(key, h->lkey);  // as in the previous call
+    for (int i = 0; i < 10; ++i) h->lkey[i] = key[i];
     // (the last build was in the other list mode: rebuild once directly, a
     // replayed graph would take the list-reuse decision on stale lists)
     const bool captured_before = h->gexec && same_key(key, h->gkey);

@@ -190,6 +190,7 @@ struct Work {
     double skin_half2;       // (skin / 2)^2, bohr^2
     unsigned long long* nbuild;  // [1] builds executed
     int num_sms;
+    int wide;                // mixed form: 8 lanes per atom in the CN (1) and chain (2) pass
     // launch shapes (read on the host when enqueueing; every choice gives the same results)
     int blk_cn, blk_disp, blk_chain;  // threads per block of the CN, dispersion and chain passes
     int build_per_sm;                 // list-builder blocks per SM
@@ -364,9 +365,6 @@ cudaError_t launch_disp_cl64(const Work& w, const Consts& c, const dbl4* pair_ta
 cudaError_t launch_atm(const Work& w, const Consts& c, bool mixed, const void* rtab, cudaStream_t st);
 // Eq. 8 per atom: J_i = W_i . v_i (device arrays).
 cudaError_t launch_heat(int64_t n, const double* w_atom, const double* vel, double* J, cudaStream_t st);
-constexpr int kForwardLaunches = 5;  // kernels per forward pass (B > 0, N > 0): CN, dispersion, chain, 2 sums
-                                     // (one more with the three-body term; in cluster mode one more,
-                                     // the fixed-point finish)
 constexpr int kBuildLaunches = 10;   // kernels per neighbour build (N > 0): reset, wrap, images, 3 scan (both
                                      // count arrays), scatter, rank (in-cell sort), fill, lists (per-atom or
                                      // cluster lists)

@@ -84,16 +84,20 @@ __device__ __forceinline__ long long fix_value(double v, int e, int bits) {
 // W and dW/dn rows of atom p and its projections v_p^(u)_a = sum_b C6ref[u][t][a][b] W_b
 // (and, for the cluster-list dispersion pass, the same rows next to
 // dv_p^(u)_a = sum_b C6ref[u][t][a][b] dW_b in w.vd)
+// (u0, us: the partner types u0, u0 + us, ... are this thread's; u0 = 0 stores the rest)
 template <class T, int R>
 __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, const T* __restrict__ c6, int64_t p, int t,
-                                              const T (&L)[R], const T (&Wr)[8], const T (&dWr)[8]) {
-    store_row<T>((T*)w.W + p * c.RP, Wr, c.RP);
-    store_row<T>((T*)w.dW + p * c.RP, dWr, c.RP);
+                                              const T (&L)[R], const T (&Wr)[8], const T (&dWr)[8], int u0 = 0,
+                                              int us = 1) {
+    if (u0 == 0) {
+        store_row<T>((T*)w.W + p * c.RP, Wr, c.RP);
+        store_row<T>((T*)w.dW + p * c.RP, dWr, c.RP);
+    }
     T* vp = (T*)w.v + p * c.T * c.RP;
     T* dvp = (sizeof(T) == 4 && w.vd) ? (T*)w.vd + p * c.T * 2 * c.RP : nullptr;  // [T][2][RP] per atom
     constexpr int S64 = row64_len(R);
     int edmax = -1022;  // FP64 form: |dv| < 2^edmax over all rows
-    for (int u = 0; u < c.T; ++u) {
+    for (int u = u0; u < c.T; u += us) {
         const T* cu = c6 + ((size_t)(u * c.T + t) * R) * R;  // C6ref[u][t][a][b]
         T vr[8], dvr[8];
 #pragma unroll
@@ -142,6 +146,7 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
             w.kd[p] = min(900, 61 - (edmax + c.fx_eG + fix_log2_pairs(w, c, w.sid[p])));
         }
     }
+    if (u0 != 0) return;
     if (p == 0 && w.npairs) *w.npairs = 0ull;  // pair count of this call's dispersion pass
     if (w.acc) {  // clear the atom's fixed-point sums of the cluster-list dispersion pass
         constexpr int n = sizeof(T) == 8 ? 8 : 4;
@@ -214,7 +219,7 @@ template <int R>
 __device__ __forceinline__ void weights_atom_mixed(const Work& w, const Consts& c, const float2* __restrict__ cnref2,
                                                    const float* __restrict__ dcr, const int* __restrict__ nref,
                                                    const float* __restrict__ c6, int64_t p, int t, float Nh,
-                                                   float Nl) {
+                                                   float Nl, int u0 = 0, int us = 1) {
     const int nr = nref[t];
     float xh[R], xl[R];
     float mh = -3.0e38f, ml = 0.0f;
@@ -262,7 +267,7 @@ __device__ __forceinline__ void weights_atom_mixed(const Work& w, const Consts& 
             Wr[a] = dWr[a] = 0.0f;
         }
     }
-    store_weights<float, R>(w, c, c6, p, t, L, Wr, dWr);
+    store_weights<float, R>(w, c, c6, p, t, L, Wr, dWr, u0, us);
 }
 
 // ------------------------------------------------------------------ Eq. 4
@@ -374,6 +379,73 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
         }
         w.cn[p] = (double)nh;
         weights_atom<MIXED, R>(w, c, cnref, nref, c6, p, S.tsrc() & 15, (double)nh);
+    }
+}
+
+// The CN pass of the mixed form with kWide lanes per atom, for batches that leave most of
+// the chip idle with one thread per atom (a list of 66 entries is then a chain of some
+// 35 us whatever the batch).  Entry k goes to lane k mod kWide; the terms are then added in
+// list order by every lane (shuffles), so the sums are those of k_cn, bit for bit.
+constexpr int kWide = 8;
+template <int R>
+__global__ void __launch_bounds__(128) k_cn_wide(Work w, Consts c, const float4* __restrict__ rcpair,
+                                                const float2* __restrict__ exptab, const float2* __restrict__ cnref2,
+                                                const float* __restrict__ dcr, const int* __restrict__ nref,
+                                                const float* __restrict__ c6) {
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = (int)(id % kWide), first = (threadIdx.x & 31) & ~(kWide - 1);
+    const bool live = id / kWide < w.Nr;
+    const int64_t p = live ? id / kWide : w.Nr - 1;  // (threads past the last atom repeat it and store nothing)
+    const Site<true> S(w, p);
+    const StructGeo& G = w.geo[w.sid[p]];
+    const int* row = w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn);
+    float* grow = w.gcn + (row - w.nbr_cn);
+    const int cnt = w.cnt_cn[p];
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    const float4* rrow = rcpair + (S.tsrc() & 15) * c.T;
+    float nh = 0.f, nl = 0.f;
+    int nint = 0;
+    int qn = l < cnt ? __ldg(row + list_off(l)) : (int)p;  // the next round's entry
+    for (int k0 = 0; k0 < most; k0 += kWide) {
+        const int k = k0 + l, q = qn;
+        qn = k + kWide < cnt ? __ldg(row + list_off(k + kWide)) : (int)p;
+        float v1 = 0.f, v2 = 0.f, g = 0.f;
+        bool one = false;
+        if (k < cnt) {
+            float D[3], r2, ah, al, rch, rcl, r2l, y;
+            int tq;
+            if (cn_pair_precise(S, q, rrow, c.k1f, c.rc_cn2f, c.rc_cn2, D, r2, ah, al, rch, tq, &rcl, &r2l, &y)) {
+                const CnDS z = cn_ds(ah, al, exptab);
+                one = z.th < 1.0f;
+                v1 = one ? -z.ch : z.fh;
+                v2 = one ? -z.cl : z.fl;
+                g = chain_coef(z, y, r2, r2l, rch, rcl, c.k1f);
+            }
+        }
+        if (live && k < ((cnt + 3) & ~3)) grow[list_off(k)] = g;  // (0 up to the end of the last group of four)
+        nint += __popc((__ballot_sync(0xffffffffu, one) >> first) & ((1u << kWide) - 1u));
+#pragma unroll
+        for (int j = 0; j < kWide; ++j) {
+            acc_add(nh, nl, __shfl_sync(0xffffffffu, v1, first + j));
+            nl += __shfl_sync(0xffffffffu, v2, first + j);
+        }
+    }
+    if (!live) return;
+    float Nh, Nl;
+    two_sum((float)nint, nh, Nh, Nl);
+    Nl += nl;
+    if (l == 0) w.cn[p] = (double)Nh + (double)Nl;
+    weights_atom_mixed<R>(w, c, cnref2, dcr, nref, c6, p, S.tsrc() & 15, Nh, Nl, l, kWide);
+    if (w.vd_images) {  // copies of the atom's v/dv rows for its image atoms, each lane those of its types
+        const int rows4 = c.T * 2 * c.RP / 4, per = 2 * c.RP / 4;
+        const int i = w.perm[p];
+        const int g0 = w.gfirst[i], ng = w.gcnt[i];
+        const float4* from = reinterpret_cast<const float4*>(w.vd) + p * rows4;
+        for (int k = 0; k < ng && g0 + k < w.ghost_cap; ++k) {
+            float4* to = reinterpret_cast<float4*>(w.vd) + (w.Nr + w.ginv[g0 + k]) * (int64_t)rows4;
+            for (int u = l; u < c.T; u += kWide)
+                for (int m = u * per; m < (u + 1) * per; ++m) to[m] = from[m];
+        }
     }
 }
 
@@ -617,6 +689,78 @@ __global__ void __launch_bounds__(128) k_chain(Work w, Consts c, const float4* _
     if (cn_out) cn_out[i] = w.cn[p];
 }
 
+// The chain pass of the mixed form with kWide lanes per atom (as k_cn_wide): the lanes load
+// and form their entries' terms, every lane adds them in list order.
+__global__ void __launch_bounds__(128) k_chain_wide(Work w, Consts c, double* __restrict__ F, double* __restrict__ e_atom,
+                                                   double* __restrict__ cn_out) {
+    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = (int)(id % kWide), first = (threadIdx.x & 31) & ~(kWide - 1);
+    const bool live = id / kWide < w.Nr;
+    const int64_t p = live ? id / kWide : w.Nr - 1;
+    const Site<true> S(w, p);
+    const float* dEdn = (const float*)w.dEdn;
+    const float dni = dEdn[p];
+    const StructGeo& G = w.geo[w.sid[p]];
+    const int* row = w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn);
+    const float* grow = w.gcn + (row - w.nbr_cn);
+    const int cnt = w.cnt_cn[p];
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    float fx = 0, fy = 0, fz = 0;
+    float s[6] = {0, 0, 0, 0, 0, 0};
+    double Sv[6] = {0, 0, 0, 0, 0, 0};
+    auto promote = [&]() {
+#pragma unroll
+        for (int m = 0; m < 6; ++m) {
+            Sv[m] += (double)s[m];
+            s[m] = 0.f;
+        }
+    };
+    int qn = l < cnt ? __ldg(row + list_off(l)) : 0;
+    float gn = l < cnt ? __ldg(grow + list_off(l)) : 0.f;
+    for (int k0 = 0; k0 < most; k0 += kWide) {
+        const int k = k0 + l, q = qn;
+        const float g = gn;
+        const bool more = k + kWide < cnt;
+        qn = more ? __ldg(row + list_off(k + kWide)) : 0;
+        gn = more ? __ldg(grow + list_off(k + kWide)) : 0.f;
+        float D[3], er[3];
+        int tq;
+        S.dist_exact(g != 0.0f ? q : (int)p, D, er, tq);  // (an entry with g = 0 adds nothing)
+        const float coef = (dni + dEdn[tq >> 4]) * g;
+#pragma unroll
+        for (int j = 0; j < kWide; ++j) {
+            const int from = first + j;
+            const float cj = __shfl_sync(0xffffffffu, coef, from), gj = __shfl_sync(0xffffffffu, g, from);
+            const float dx = __shfl_sync(0xffffffffu, D[0], from), dy = __shfl_sync(0xffffffffu, D[1], from),
+                        dz = __shfl_sync(0xffffffffu, D[2], from);
+            fx += cj * dx; fy += cj * dy; fz += cj * dz;
+            const float gx = gj * dx, gy = gj * dy, gz = gj * dz;
+            s[0] = fmaf(gx, dx, s[0]); s[1] = fmaf(gy, dy, s[1]); s[2] = fmaf(gz, dz, s[2]);
+            s[3] = fmaf(gx, dy, s[3]); s[4] = fmaf(gx, dz, s[4]); s[5] = fmaf(gy, dz, s[5]);
+        }
+        if (((k0 + kWide) & (kChunk - 1)) == 0) promote();  // every kChunk entries, as k_chain
+    }
+    promote();
+    if (!live || l != 0) return;
+    const float4 fd = ((const float4*)w.Fd)[p];
+    const double u = kHartreeEV / kBohrA;
+    const int i = w.perm[p];
+    const double f0 = ((double)fd.x + (double)fx) * u, f1 = ((double)fd.y + (double)fy) * u,
+                 f2 = ((double)fd.z + (double)fz) * u;
+    double* Fi = F + 3 * (int64_t)i;
+    if (c.accumulate) {
+        Fi[0] += f0; Fi[1] += f1; Fi[2] += f2;
+    } else {
+        Fi[0] = f0; Fi[1] = f1; Fi[2] = f2;
+    }
+    double* wv = w.wv + 6 * p;
+    const double dn = (double)dni;
+#pragma unroll
+    for (int m = 0; m < 6; ++m) wv[m] -= dn * Sv[m];
+    if (e_atom) e_atom[i] = w.eat[p] * kHartreeEV;
+    if (cn_out) cn_out[i] = w.cn[p];
+}
+
 // ------------------------------------------------------------------ per-structure sums
 // Two fixed-order levels: block (s, c) sums atoms [c*kFinChunk, (c+1)*kFinChunk)
 // of structure s into part[fin_base_s + c][7]; then warp s adds its structure's
@@ -679,6 +823,35 @@ __global__ void __launch_bounds__(128) k_fin_struct(Work w, const double* __rest
     }
 }
 
+// Both levels in one kernel where no structure has more than one chunk.
+__global__ void __launch_bounds__(256) k_fin_one(Work w, double* __restrict__ E, double* __restrict__ Wout, int accumulate) {
+    const int s = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const StructGeo& G = w.geo[s];
+    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+    for (int k = threadIdx.x; k < G.natoms; k += 256) {
+        const int64_t p = G.atom_base + k;
+        acc[0] += w.eat[p];
+        const double2* v = reinterpret_cast<const double2*>(w.wv + 6 * p);
+        const double2 v0 = v[0], v1 = v[1], v2 = v[2];
+        acc[1] += v0.x; acc[2] += v0.y; acc[3] += v1.x; acc[4] += v1.y; acc[5] += v2.x; acc[6] += v2.y;
+    }
+    __shared__ double red[8][7];
+#pragma unroll
+    for (int m = 0; m < 7; ++m) {
+        for (int o = 16; o > 0; o >>= 1) acc[m] += __shfl_xor_sync(0xffffffffu, acc[m], o);
+        if (lane == 0) red[wid][m] = acc[m];
+    }
+    __syncthreads();
+    if (threadIdx.x >= 10) return;
+    const int from[10] = {0, 1, 4, 5, 4, 2, 6, 5, 6, 3};  // E, then W row by row of xx yy zz xy xz yz
+    double x = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x += red[k][from[threadIdx.x]];
+    x *= kHartreeEV;
+    double* out = threadIdx.x == 0 ? E + s : Wout + 9 * (int64_t)s + threadIdx.x - 1;
+    *out = accumulate ? *out + x : x;
+}
+
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <bool MIXED, int R>
@@ -691,7 +864,10 @@ cudaError_t forward_impl(const Work& w, const Consts& c, const Tabs& tb, double*
         if (marks) cudaEventRecord(marks[k], st);
     };
     mark(0);
-    if (w.Nr > 0)
+    if (MIXED && (w.wide & 1))
+        k_cn_wide<R><<<nblk(w.Nr * kWide, 128), 128, 0, st>>>(w, c, tb.rcpair, tb.exptab, tb.cnref2, tb.dcr, tb.nref,
+                                                              (const float*)tb.c6);
+    else if (w.Nr > 0)
         k_cn<MIXED, R><<<nblk(w.Nr, w.blk_cn), w.blk_cn, 0, st>>>(w, c, tb.rcpair, tb.exptab, tb.cnref, tb.cnref2,
                                                                   tb.dcr, tb.nref, (const T*)tb.c6, tb.k1rc, tb.exptab64);
     mark(1);  // the weights (Eq. 3) are formed inside the CN pass
@@ -715,13 +891,17 @@ cudaError_t forward_impl(const Work& w, const Consts& c, const Tabs& tb, double*
     mark(4);
     if (w.Nr > 0) {
         const int TB = w.blk_chain;
-        if (w_atom)
+        if (MIXED && (w.wide & 2) && !w_atom)
+            k_chain_wide<<<nblk(w.Nr * kWide, 128), 128, 0, st>>>(w, c, F, e_atom, cn_out);
+        else if (w_atom)
             k_chain<MIXED, true><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, tb.rcpair, tb.exptab, F, e_atom, cn_out, w_atom);
         else
             k_chain<MIXED, false><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, tb.rcpair, tb.exptab, F, e_atom, cn_out, nullptr);
     }
     mark(5);
-    if (B > 0) {
+    if (B > 0 && w.max_natoms <= kFinChunk) {
+        k_fin_one<<<B, 256, 0, st>>>(w, E, W, c.accumulate);
+    } else if (B > 0) {
         if (w.n_fin > 0) k_fin_chunks<<<(unsigned)w.n_fin, 256, 0, st>>>(w, w.fin_part);
         k_fin_struct<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(w, w.fin_part, E, W, c.accumulate);
     }
