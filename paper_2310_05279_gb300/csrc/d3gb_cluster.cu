@@ -64,24 +64,65 @@ __device__ __forceinline__ void red_add_if(bool p, unsigned long long* a, unsign
                  :: "l"(a), "l"(x), "r"((unsigned)p) : "memory");
 }
 
-// Data of one list entry for the lane's step: the neighbour's split position and
-// its rows v^(t_i), dv^(t_i) (its own, or its source atom's); q = -1 past the end
-// of the list.
+// Pairs of floats in one 64-bit register pair and the FP32 pipe's operations on both
+// halves at once (each half rounds as the scalar operation does).
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float low2(f2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return lo;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Data of one list entry for the lane's step: the neighbour's split position (x and y
+// packed) and its row of (v_a, dv_a) pairs for partner type t_i (its own, or its source
+// atom's); q = -1 past the end of the list.
 template <int R>
 struct JData {
-    float4 h, l;
-    float v[R], dv[R];
-    int q;
+    f2 hxy, lxy;
+    float hz, lz;
+    int ts, q;
+    f2 vd[R];
 };
 
 template <int R>
 __device__ __forceinline__ void load_j(const Work& w, const float* __restrict__ vdb, int rows, int q, int src,
                                        JData<R>& J) {
     J.q = q;
-    rec_load(w, q >= 0 ? q : 0, J.h, J.l);
+    f2 hz, lz;
+    asm("ld.global.nc.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(J.hxy), "=l"(hz), "=l"(J.lxy), "=l"(lz)
+        : "l"(w.rec + 2 * (int64_t)(q >= 0 ? q : 0)));
+    float ts, rk;
+    unpack2(hz, J.hz, ts);
+    J.ts = __float_as_int(ts);
+    unpack2(lz, J.lz, rk);
     const float* r = vdb + (int64_t)(src >= 0 ? src : 0) * rows;
-    load_vec<R>(r, J.v);
-    load_vec<R>(r + (R <= 4 ? 4 : 8), J.dv);
+    f2 t[8];
+    asm("ld.global.nc.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(t[0]), "=l"(t[1]), "=l"(t[2]), "=l"(t[3]) : "l"(r));
+    if constexpr (R == 5) {
+        asm("ld.global.nc.b64 %0, [%1];" : "=l"(t[4]) : "l"(r + 8));
+    } else if constexpr (R > 5) {
+        asm("ld.global.nc.v4.b64 {%0,%1,%2,%3}, [%4];" : "=l"(t[4]), "=l"(t[5]), "=l"(t[6]), "=l"(t[7]) : "l"(r + 8));
+    }
+#pragma unroll
+    for (int a = 0; a < R; ++a) J.vd[a] = t[a];
 }
 
 // Split form: the steps of one chunk (16) of the force terms on i, and the chunk's
@@ -97,7 +138,9 @@ constexpr int kSplitFloats = kSplitForce + 8 * 32;  // per warp
 template <int R, bool SITE, bool SPLIT>
 struct ClusterPass {
     Site<true> S;
-    float Wi[R], dWi[R];
+    f2 nhxy, nlxy;        // minus the atom's split position, x and y
+    f2 Wi2[R];            // W_ia in both halves
+    float dWi[R];
     const float4* trow;
     int pthr;             // a pair is used when q > pthr: later clusters, images, own cluster after i
     float rc2, band;
@@ -108,30 +151,49 @@ struct ClusterPass {
     unsigned npairs = 0;  // used pairs of the warp (warp-uniform)
     float* fbuf = nullptr;  // SPLIT: the lane's slots of the chunk
     // running sums of the lane's i
-    float fx = 0.f, fy = 0.f, fz = 0.f;
+    f2 gxy = 0;           // minus the force on i (SPLIT: the lane's component in gz)
+    float gz = 0.f;
     float dnc = 0.f, dnh = 0.f, dnl = 0.f;            // dE/dn_i: chunk partial and compensated sum
     float ec = 0.f, Eh = 0.f, El = 0.f;               // energy (half pair energies for SITE, else whole)
-    float sv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};     // virial chunk partials (of -fc d (x) d)
+    f2 svd = 0;                                       // virial chunk partials (of -fc d (x) d): xx, yy
+    float sv[4] = {0.f, 0.f, 0.f, 0.f};               // zz, xy, xz, yz
     float Vh[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, Vl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 
-    __device__ ClusterPass(const Work& w, int64_t p) : S(w, p) {}
+    __device__ ClusterPass(const Work& w, int64_t p) : S(w, p) {
+        nhxy = pack2(-S.h.x, -S.h.y);
+        nlxy = pack2(-S.l.x, -S.l.y);
+    }
+    // the weights of atom p
+    __device__ __forceinline__ void load_weights(const Work& w, const Consts& c, int64_t p) {
+        float W[R];
+        load_vec<R>((const float*)w.W + p * c.RP, W);
+        load_vec<R>((const float*)w.dW + p * c.RP, dWi);
+#pragma unroll
+        for (int a = 0; a < R; ++a) Wi2[a] = pack2(W[a], W[a]);
+    }
 
     __device__ __forceinline__ void chunk() {
         acc_add(dnh, dnl, dnc);
         acc_add(Eh, El, ec);
+        float xx, yy;
+        unpack2(svd, xx, yy);
+        acc_add(Vh[0], Vl[0], xx);
+        acc_add(Vh[1], Vl[1], yy);
+        svd = 0;
 #pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            acc_add(Vh[m], Vl[m], sv[m]);
+        for (int m = 0; m < 4; ++m) {
+            acc_add(Vh[2 + m], Vl[2 + m], sv[m]);
             sv[m] = 0.f;
         }
         dnc = ec = 0.f;
     }
 
-    __device__ __forceinline__ void pair_vec(const JData<R>& J, float& dx, float& dy, float& dz, float& r2,
-                                             bool& use, bool& near) const {
-        dx = (J.h.x - S.h.x) + (J.l.x - S.l.x);
-        dy = (J.h.y - S.h.y) + (J.l.y - S.l.y);
-        dz = (J.h.z - S.h.z) + (J.l.z - S.l.z);
+    __device__ __forceinline__ void pair_vec(const JData<R>& J, f2& dxy, float& dz, float& r2, bool& use,
+                                             bool& near) const {
+        dxy = add2(add2(J.hxy, nhxy), add2(J.lxy, nlxy));
+        dz = (J.hz - S.h.z) + (J.lz - S.l.z);
+        float dx, dy;
+        unpack2(dxy, dx, dy);
         r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
         const bool listed = J.q > pthr;
         near = listed && fabsf(r2 - rc2) <= band;
@@ -140,16 +202,19 @@ struct ClusterPass {
 
     // pair terms of a used pair (zero weight otherwise) and the i-side sums; returns
     // the j-side values: force on j (nt), dE/dn_j, energy share
-    __device__ __forceinline__ void pair(const JData<R>& J, int step, float dx, float dy, float dz, float r2, bool use,
+    __device__ __forceinline__ void pair(const JData<R>& J, int step, f2 dxy, float dz, float r2, bool use,
                                          float& ntx, float& nty, float& ntz, float& dnj, float& e) {
-        const float4 tb = trow[__float_as_int(J.h.w) & 15];
-        float C6 = 0.f, dC6i = 0.f, dC6j = 0.f;
+        const float4 tb = trow[J.ts & 15];
+        f2 c = 0;  // C6, dC6/dn_j
+        float dC6i = 0.f;
 #pragma unroll
         for (int a = 0; a < R; ++a) {
-            C6 = fmaf(Wi[a], J.v[a], C6);
-            dC6i = fmaf(dWi[a], J.v[a], dC6i);
-            dC6j = fmaf(Wi[a], J.dv[a], dC6j);
+            c = fma2(Wi2[a], J.vd[a], c);
+            dC6i = fmaf(dWi[a], low2(J.vd[a]), dC6i);
         }
+        float C6, dC6j, dx, dy;
+        unpack2(c, C6, dC6j);
+        unpack2(dxy, dx, dy);
         const float r4 = r2 * r2, r6 = r4 * r2, r8 = r4 * r4;
         const float d6 = r6 + tb.x, d8 = r8 + tb.y;
         const float pinv = rcp_approx(d6 * d8);
@@ -160,16 +225,19 @@ struct ClusterPass {
         // F_i = -(de/dr) d/r = -nfc d, nfc = -C6 (6 r^4 t6 i6 + 8 r^6 t8 i8); the force on j is nfc d
         const float nfc = use ? -C6 * fmaf(6.0f * r4, t6 * i6, 8.0f * r6 * (t8 * i8)) : 0.f;
         ntx = nfc * dx; nty = nfc * dy; ntz = nfc * dz;
+        const f2 nxy = pack2(ntx, nty);
         if constexpr (SPLIT) {
             float* f = fbuf + step * 96;
             f[0] = ntx; f[32] = nty; f[64] = ntz;
         } else {
-            fx -= ntx; fy -= nty; fz -= ntz;
+            gxy = add2(gxy, nxy);
+            gz += ntz;
         }
         dnc = fmaf(mg, dC6i, dnc);
         ec += e;
-        sv[0] = fmaf(ntx, dx, sv[0]); sv[1] = fmaf(nty, dy, sv[1]); sv[2] = fmaf(ntz, dz, sv[2]);
-        sv[3] = fmaf(ntx, dy, sv[3]); sv[4] = fmaf(ntx, dz, sv[4]); sv[5] = fmaf(nty, dz, sv[5]);
+        svd = fma2(nxy, dxy, svd);
+        sv[0] = fmaf(ntz, dz, sv[0]); sv[1] = fmaf(ntx, dy, sv[1]);
+        sv[2] = fmaf(ntx, dz, sv[2]); sv[3] = fmaf(nty, dz, sv[3]);
         dnj = mg * dC6j;
     }
 
@@ -214,10 +282,11 @@ struct ClusterPass {
 
     // (step: place of A in its chunk, used by SPLIT)
     __device__ __forceinline__ void step2(const JData<R>& A, const JData<R>& B, int step) {
-        float ax, ay, az, ar2, bx, by, bz, br2;
+        f2 axy, bxy;
+        float az, ar2, bz, br2;
         bool ause, anear, buse, bnear;
-        pair_vec(A, ax, ay, az, ar2, ause, anear);
-        pair_vec(B, bx, by, bz, br2, buse, bnear);
+        pair_vec(A, axy, az, ar2, ause, anear);
+        pair_vec(B, bxy, bz, br2, buse, bnear);
         if (__any_sync(0xffffffffu, anear || bnear)) {  // a pair within the FP32 error band of R_pot
             if (anear) ause = S.inside(A.q, ar2, rc2, rc2d);
             if (bnear) buse = S.inside(B.q, br2, rc2, rc2d);
@@ -232,14 +301,14 @@ struct ClusterPass {
         }
         npairs += __popc(uma) + __popc(umb);
         float atx, aty, atz, adn, ae, btx, bty, btz, bdn, be;
-        pair(A, step, ax, ay, az, ar2, ause, atx, aty, atz, adn, ae);
-        pair(B, step + 1, bx, by, bz, br2, buse, btx, bty, btz, bdn, be);
+        pair(A, step, axy, az, ar2, ause, atx, aty, atz, adn, ae);
+        pair(B, step + 1, bxy, bz, br2, buse, btx, bty, btz, bdn, be);
         if constexpr (SITE) {
-            flush_j(__float_as_int(A.h.w), uma, atx, aty, atz, adn, ae);
-            flush_j(__float_as_int(B.h.w), umb, btx, bty, btz, bdn, be);
+            flush_j(A.ts, uma, atx, aty, atz, adn, ae);
+            flush_j(B.ts, umb, btx, bty, btz, bdn, be);
         } else {
             const float pa = part_j(atx, aty, atz, adn), pb = part_j(btx, bty, btz, bdn);
-            flush_j2(__float_as_int(A.h.w), uma, pa, __float_as_int(B.h.w), umb, pb);
+            flush_j2(A.ts, uma, pa, B.ts, umb, pb);
         }
     }
 };
@@ -270,8 +339,7 @@ template <int R, bool SITE, bool SPLIT>
 __device__ __forceinline__ void cluster_setup(ClusterPass<R, SITE, SPLIT>& P, const Work& w, const Consts& c,
                                               const ClusterRow& C, const float4* tab, int lane) {
     const int ti = P.S.tsrc() & 15;
-    load_vec<R>((const float*)w.W + C.p * c.RP, P.Wi);
-    load_vec<R>((const float*)w.dW + C.p * c.RP, P.dWi);
+    P.load_weights(w, c, C.p);
     P.trow = tab + ti * c.T;
     P.pthr = C.ilive ? (int)C.p : 0x7fffffff;
     P.rc2 = c.rc_disp2f;
@@ -347,7 +415,10 @@ template <int R, bool SITE, bool SPLIT>
 __device__ __forceinline__ void cluster_finish(ClusterPass<R, SITE, SPLIT>& P, const Work& w, const ClusterRow& C,
                                                int lane) {
     const int il = lane & 7, js = lane >> 3;
-    float fx = P.fx, fy = P.fy, fz = P.fz, dnh = P.dnh, dnl = P.dnl, Eh = P.Eh, El = P.El;
+    float fx, fy, fz = -P.gz, dnh = P.dnh, dnl = P.dnl, Eh = P.Eh, El = P.El;
+    unpack2(P.gxy, fx, fy);
+    fx = -fx;
+    fy = -fy;
 #pragma unroll
     for (int o = 8; o < 32; o <<= 1) {
         fx += __shfl_xor_sync(0xffffffffu, fx, o);
@@ -396,13 +467,20 @@ __device__ __forceinline__ void cluster_finish(ClusterPass<R, SITE, SPLIT>& P, c
 
 // IMGSRC: image atoms have no rows of their own; each list entry's source atom is
 // resolved once per block of 32 entries (from the image's compact record).
-// The bound (128, 3) holds every instantiation to 168 registers, so that three
-// 128-thread blocks (12 warps) stay resident per SM whatever R is.
+// 57% of issue slots and 67% of the L1 data path's wavefronts (broadcast loads, shuffles,
+// reductions): both are shared out over more warps by holding two steps' neighbour data at
+// a time instead of four, for 128 registers and four 128-thread blocks (16 warps) per SM.
+// Packed pairs of floats carry C6 with dC6/dn_j, and x with y of the pair vectors, forces
+// and virial. Measured on 128 x 1440 atoms, a 1,048,576-atom box and 512 uneven structures:
+// 320, 3030 and 1600 us with scalar arithmetic, 12 warps and the next two steps' loads
+// ahead; 314, 2958 and 1549 with 16 warps; 309, 2711 and 1481 with both (packed with 12
+// warps 335, 2950 and 1661; 20 warps spill; rows loaded only for steps that have a pair
+// 350, 3045 and 1611).
 // BESIDE: clusters with more than w.split_min entries are left to k_disp_cl_split, which
 // runs at the same time: this kernel is launched without waiting for it and waits before
 // it ends, so that what follows sees both.
 template <int R, bool SITE, bool IMGSRC, bool BESIDE>
-__global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const float4* __restrict__ pair_tab) {
+__global__ void __launch_bounds__(128, 4) k_disp_cl(Work w, Consts c, const float4* __restrict__ pair_tab) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4* tab = reinterpret_cast<float4*>(smem_raw);
     for (int k = threadIdx.x; k < c.T * c.T; k += blockDim.x) tab[k] = pair_tab[k];
@@ -419,8 +497,7 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
     const int64_t p = p0 + (ilive ? il : 0);  // lanes past the cluster's end mirror its first atom, unused
     ClusterPass<R, SITE, false> P(w, p);
     const int ti = P.S.tsrc() & 15;
-    load_vec<R>((const float*)w.W + p * c.RP, P.Wi);
-    load_vec<R>((const float*)w.dW + p * c.RP, P.dWi);
+    P.load_weights(w, c, p);
     P.trow = tab + ti * c.T;
     P.pthr = ilive ? (int)p : 0x7fffffff;
     P.rc2 = c.rc_disp2f;
@@ -444,7 +521,6 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
     // list entries of steps 8b..8b+7 (block b) come from one coalesced load, lane k
     // holding entry 32b + k, together with the entry's source atom (itself for a real
     // atom; with IMGSRC, an image's source from its compact record), a block ahead.
-    // The neighbour data of the next two steps is loaded while two steps compute.
     // Whole blocks are processed: entries past the end of the list are -1 (unused).
     const int nr = (int)w.Nr;
     auto src_of = [&](int q) { return IMGSRC && q >= nr ? (__float_as_int(__ldg(&w.hi[q].w)) >> 4) : q; };
@@ -458,35 +534,29 @@ __global__ void __launch_bounds__(128, 3) k_disp_cl(Work w, Consts c, const floa
         const int src = IMGSRC ? __shfl_sync(0xffffffffu, sa, from) : q;
         load_j<R>(w, vdb, rows, q, src, J);
     };
-    JData<R> A, B, C, D;
-    load(0, A);
-    load(1, B);
+    JData<R> A, B;
     const int nblocks = (nsteps + 7) >> 3;
     for (int b = 0; b < nblocks; ++b) {
-        load(2, C);
-        load(3, D);
-        P.step2(A, B, 0);
-        load(4, A);
-        load(5, B);
-        P.step2(C, D, 0);
-        load(6, C);
-        load(7, D);
-        P.step2(A, B, 0);
-        // next block: its entries become current, the one after is loaded
+#pragma unroll
+        for (int st = 0; st < 8; st += 2) {
+            load(st, A);
+            load(st + 1, B);
+            P.step2(A, B, 0);
+        }
         qa = qb;
         sa = sb;
         const int k = 32 * (b + 2) + lane;
         qb = k < cnt ? __ldg(row + k) : -1;
         sb = src_of(qb);
-        load(0, A);
-        load(1, B);
-        P.step2(C, D, 0);
         if (b & 1) P.chunk();  // every 16 steps
     }
     P.chunk();
     if (lane == 0 && w.npairs) atomicAdd(w.npairs, (unsigned long long)P.npairs);
     // i side: sum the 4 lanes of each i (fixed order) and add to the accumulators
-    float fx = P.fx, fy = P.fy, fz = P.fz, dnh = P.dnh, dnl = P.dnl, Eh = P.Eh, El = P.El;
+    float fx, fy, fz = -P.gz, dnh = P.dnh, dnl = P.dnl, Eh = P.Eh, El = P.El;
+    unpack2(P.gxy, fx, fy);
+    fx = -fx;
+    fy = -fy;
 #pragma unroll
     for (int o = 8; o < 32; o <<= 1) {
         fx += __shfl_xor_sync(0xffffffffu, fx, o);
@@ -570,8 +640,9 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
             if (ch < nchunks) {
                 P.fbuf = mine;
                 P.dnc = P.ec = 0.f;
+                P.svd = 0;
 #pragma unroll
-                for (int m = 0; m < 6; ++m) P.sv[m] = 0.f;
+                for (int m = 0; m < 4; ++m) P.sv[m] = 0.f;
                 const int b1 = min(nblocks, 2 * ch + 2);
                 cluster_blocks<R, SITE, IMGSRC, true>(P, w, c, C, lane, 2 * ch, b1);
                 if (b1 == 2 * ch + 1)  // the last chunk has 8 steps
@@ -580,8 +651,9 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
                 float* q = mine + kSplitForce;
                 q[0] = P.dnc;
                 q[32] = P.ec;
+                unpack2(P.svd, q[64], q[96]);
 #pragma unroll
-                for (int m = 0; m < 6; ++m) q[64 + 32 * m] = P.sv[m];
+                for (int m = 0; m < 4; ++m) q[128 + 32 * m] = P.sv[m];
             }
             __syncthreads();
             // warp t = 0, 1, 2 adds force component t and some of the other sums, chunk by chunk
@@ -589,10 +661,8 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
                 const int n = min(nw, nchunks - c0);
                 for (int r = 0; r < n; ++r) {
                     const float* f = buf + r * kSplitFloats + 32 * wid + lane;
-                    float x = P.fx;
 #pragma unroll
-                    for (int s = 0; s < kChunkSteps; ++s) x = __fsub_rn(x, f[s * 96]);
-                    P.fx = x;
+                    for (int s = 0; s < kChunkSteps; ++s) P.gz = __fadd_rn(P.gz, f[s * 96]);
                     const float* q = buf + r * kSplitFloats + kSplitForce + lane;
                     if (wid == 0) {
                         acc_add(P.dnh, P.dnl, q[0]);
@@ -609,7 +679,7 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
         // everything to warp 0
         if (wid == 1 || wid == 2) {
             float* o = buf + wid * kSplitFloats + lane;
-            o[0] = P.fx;
+            o[0] = P.gz;
 #pragma unroll
             for (int m = 0; m < 3; ++m) {
                 o[32 + 64 * m] = P.Vh[m];
@@ -619,8 +689,8 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
         __syncthreads();
         if (wid == 0) {
             const float *o1 = buf + kSplitFloats + lane, *o2 = buf + 2 * kSplitFloats + lane;
-            P.fy = o1[0];
-            P.fz = o2[0];
+            P.gxy = pack2(P.gz, o1[0]);
+            P.gz = o2[0];
 #pragma unroll
             for (int m = 0; m < 3; ++m) {
                 P.Vh[m] = o1[32 + 64 * m];

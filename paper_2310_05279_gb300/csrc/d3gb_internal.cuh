@@ -177,7 +177,7 @@ struct Work {
     double* gcnd;            // FP64 form: per CN-list entry, the chain coefficient f'(r)/r (as gcn)
     float* gcn;              // mixed form: per CN-list entry, the chain coefficient f'(r)/r of Eq. 4
                              // (written by the CN pass, 0 outside R_cn; read by the chain pass)
-    float* vd;               // [Nr (+ ghost_cap)][T][2][RP] per atom q and partner type t: v_q^(t) and
+    float* vd;               // [Nr (+ ghost_cap)][T][RP][2] per atom q and partner type t: pairs of v_q^(t)_a and
                              // dv_q^(t)_a = sum_b C6ref[t][tq][a][b] dW_qb
     int vd_images;           // 1: image atoms have rows (copies of their source's, written by the CN pass),
                              // 0: the dispersion pass reads their source's

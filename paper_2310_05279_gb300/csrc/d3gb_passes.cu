@@ -82,7 +82,7 @@ __device__ __forceinline__ long long fix_value(double v, int e, int bits) {
 }
 
 // W and dW/dn rows of atom p and its projections v_p^(u)_a = sum_b C6ref[u][t][a][b] W_b
-// (and, for the cluster-list dispersion pass, the same rows next to
+// (and, for the cluster-list dispersion pass, the same values beside those of
 // dv_p^(u)_a = sum_b C6ref[u][t][a][b] dW_b in w.vd)
 // (u0, us: the partner types u0, u0 + us, ... are this thread's; u0 = 0 stores the rest)
 template <class T, int R>
@@ -94,7 +94,7 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
         store_row<T>((T*)w.dW + p * c.RP, dWr, c.RP);
     }
     T* vp = (T*)w.v + p * c.T * c.RP;
-    T* dvp = (sizeof(T) == 4 && w.vd) ? (T*)w.vd + p * c.T * 2 * c.RP : nullptr;  // [T][2][RP] per atom
+    T* dvp = (sizeof(T) == 4 && w.vd) ? (T*)w.vd + p * c.T * 2 * c.RP : nullptr;  // [T][RP][2] per atom
     constexpr int S64 = row64_len(R);
     int edmax = -1022;  // FP64 form: |dv| < 2^edmax over all rows
     for (int u = u0; u < c.T; u += us) {
@@ -128,8 +128,10 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
             }
         }
         if (dvp) {
-            store_row<T>(dvp + 2 * u * c.RP, vr, c.RP);
-            store_row<T>(dvp + (2 * u + 1) * c.RP, dvr, c.RP);
+            float4* d = reinterpret_cast<float4*>(dvp + 2 * u * c.RP);  // (v_a, dv_a) pairs
+#pragma unroll
+            for (int a = 0; a < 8; a += 2)
+                if (a < c.RP) d[a / 2] = make_float4((float)vr[a], (float)dvr[a], (float)vr[a + 1], (float)dvr[a + 1]);
         }
     }
     if constexpr (sizeof(T) == 8) {
