@@ -403,9 +403,28 @@ __global__ void __launch_bounds__(128) kb_disp_mixed(Work w, BW b, BConsts c, co
     for (int k0 = 0; k0 < cnt; k0 += kChunk) {
         const int k1e = min(cnt, k0 + kChunk);
         float dt = 0.0f, fv[3] = {0, 0, 0}, ft[3] = {0, 0, 0}, hv[4] = {0, 0, 0, 0}, ht[4] = {0, 0, 0, 0};
-        LV.for_each(k0, k1e, [&](int q) {
-            float4 hq, lq;
-            rec_load(w, q, hq, lq);
+        // an entry's position record and tangent, then its v row for type t_i (R values, then R
+        // tangents, each padded to RP: vector loads); two entries' loads are issued before their
+        // arithmetic (the pass waits for them: 27% of the issue slots were used with one; 57.4 M
+        // ordered pairs 1.61 ms and 1.40; the next two's records ahead as well: slower, 168 registers)
+        struct Entry {
+            float4 h, l, u;
+            float vv[R], vt[R];
+            int q;
+        };
+        auto fetch = [&](int q, Entry& x) {
+            x.q = q;
+            rec_load(w, q, x.h, x.l);
+            x.u = __ldg(b.xdf + q);
+        };
+        auto fetch_row = [&](Entry& x) {
+            const float* vq = b.vf + (int64_t)(__float_as_int(x.h.w) >> 4) * stride + ti * 2 * RP;
+            load_vec<R>(vq, x.vv);
+            load_vec<R>(vq + RP, x.vt);
+        };
+        auto add = [&](const Entry& x) {
+            const float4 hq = x.h, lq = x.l;
+            const int q = x.q;
             const float dx = (hq.x - hp.x) + (lq.x - lp.x), dy = (hq.y - hp.y) + (lq.y - lp.y),
                         dz = (hq.z - hp.z) + (lq.z - lp.z);
             const float r2v = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -419,19 +438,14 @@ __global__ void __launch_bounds__(128) kb_disp_mixed(Work w, BW b, BConsts c, co
             }
             if (!in) return;
             const int tsq = __float_as_int(hq.w);
-            const float4 tq = b.xdf[q];
+            const float4 tq = x.u;
             const float ux = tq.x - tp.x, uy = tq.y - tp.y, uz = tq.z - tp.z;
             const DF r2 = DF{r2v, 2.0f * fmaf(dx, ux, fmaf(dy, uy, dz * uz))};
             const float* tb = tab[ti * c.T + (tsq & 15)];
-            // the v row of q for type t_i: R values, then R tangents, each padded to RP (vector loads)
-            const float* vq = b.vf + (int64_t)(tsq >> 4) * stride + ti * 2 * RP;
-            float vv[R], vt[R];
-            load_vec<R>(vq, vv);
-            load_vec<R>(vq + RP, vt);
             DF C6 = DF{0.0f, 0.0f}, dC6 = DF{0.0f, 0.0f};
 #pragma unroll
             for (int a = 0; a < R; ++a) {
-                const DF v = DF{vv[a], vt[a]};
+                const DF v = DF{x.vv[a], x.vt[a]};
                 C6 = C6 + Wi[a] * v;
                 dC6 = dC6 + dWi[a] * v;
             }
@@ -455,7 +469,21 @@ __global__ void __launch_bounds__(128) kb_disp_mixed(Work w, BW b, BConsts c, co
             const DF dR = C6 * (tb[4] * (i6 * i6) + tb[5] * (i8 * i8));
             hv[2] = fmaf(tb[3], dR.v, hv[2]); ht[2] = fmaf(tb[3], dR.t, ht[2]);
             hv[3] += dR.v; ht[3] += dR.t;
-        });
+        };
+        auto add_two = [&](int qa, int qb, bool two) {
+            Entry x, y;
+            fetch(qa, x);
+            fetch(two ? qb : (int)p, y);
+            fetch_row(x);
+            fetch_row(y);
+            add(x);
+            if (two) add(y);
+        };
+        for (int k = k0; k < k1e; k += 4) {
+            const int4 q4 = __ldg(reinterpret_cast<const int4*>(LV.p + list_off(k)));
+            add_two(q4.x, q4.y, k + 1 < k1e);
+            if (k + 2 < k1e) add_two(q4.z, q4.w, k + 3 < k1e);
+        }
         dnt.add(dt);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -529,10 +557,11 @@ __global__ void __launch_bounds__(128) kb_cn_mixed(Work w, BW b, Consts c, const
     const float4 tp = b.xdf[p];
     float nh = 0.f, nl = 0.f, th = 0.f, tl = 0.f;
     int nint = 0;
-    LV.for_each(0, cnt, [&](int q) {
+    auto add = [&](int q, const float4* rec, const float4& uq) {
         float D[3], r2, ah, al, rch;
         int tq;
-        if (!cn_pair_precise(S, q, rrow, k1, rc2, c.rc_cn2, D, r2, ah, al, rch, tq)) return;
+        if (!cn_pair_precise(S, q, rrow, k1, rc2, c.rc_cn2, D, r2, ah, al, rch, tq, nullptr, nullptr, nullptr, rec))
+            return;
         const CnDS z = cn_ds(ah, al, exptab);
         if (z.th < 1.0f) {
             ++nint;
@@ -542,11 +571,23 @@ __global__ void __launch_bounds__(128) kb_cn_mixed(Work w, BW b, Consts c, const
             acc_add(nh, nl, z.fh);
             nl += z.fl;
         }
-        const float4 uq = b.xdf[q];
         const float du = fmaf(D[0], uq.x - tp.x, fmaf(D[1], uq.y - tp.y, D[2] * (uq.z - tp.z)));
         const float ri = rsqrt_nr(r2);
         acc_add(th, tl, -k1 * rch * z.fh * z.ch * (ri * ri * ri) * du);
-    });
+    };
+    for (int k = 0; k < cnt; k += 4) {  // four entries' loads before their arithmetic
+        const int4 q4 = __ldg(reinterpret_cast<const int4*>(LV.p + list_off(k)));
+        const int q[4] = {q4.x, k + 1 < cnt ? q4.y : (int)p, k + 2 < cnt ? q4.z : (int)p, k + 3 < cnt ? q4.w : (int)p};
+        float4 rec[4][2], u[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            rec_load(w, q[e], rec[e][0], rec[e][1]);
+            u[e] = __ldg(b.xdf + q[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (k + e < cnt) add(q[e], rec[e], u[e]);
+    }
     b.n[p] = Dual{(double)nint + (double)nh + (double)nl, (double)th + (double)tl};
 }
 
@@ -651,15 +692,13 @@ __global__ void __launch_bounds__(128) kb_chain_mixed(Work w, BW b, Consts c, co
     const float dni = dnd.x, dnit = dnd.y;
     const float4 tp = b.xdf[p];
     float fv[3] = {0.f, 0.f, 0.f}, ft[3] = {0.f, 0.f, 0.f};
-    LV.for_each(0, cnt, [&](int q) {
+    auto add = [&](int q, const float4* rec, const float4& uq, const float2& dqd) {
         float D[3], r2, ah, al, rch, rcl, r2l;
         int tq;
-        if (!cn_pair_precise(S, q, rrow, k1, rc2, c.rc_cn2, D, r2, ah, al, rch, tq, &rcl, &r2l)) return;
+        if (!cn_pair_precise(S, q, rrow, k1, rc2, c.rc_cn2, D, r2, ah, al, rch, tq, &rcl, &r2l, nullptr, rec)) return;
         const CnDS z = cn_ds(ah, al, exptab);
         const float g = chain_coef(z, r2, r2l, rch, rcl, k1);
-        const float2 dqd = b.dEdnf[tq >> 4];
         const float dnq = dqd.x, dnqt = dqd.y;
-        const float4 uq = b.xdf[q];
         const float u[3] = {uq.x - tp.x, uq.y - tp.y, uq.z - tp.z};
         const float du = fmaf(D[0], u[0], fmaf(D[1], u[1], D[2] * u[2]));
         const float ri = rsqrt_nr(r2), ri2 = ri * ri;
@@ -674,7 +713,23 @@ __global__ void __launch_bounds__(128) kb_chain_mixed(Work w, BW b, Consts c, co
             fv[a] = fmaf(cv, D[a], fv[a]);
             ft[a] = fmaf(ct, D[a], fmaf(cv, u[a], ft[a]));
         }
-    });
+    };
+    for (int k = 0; k < cnt; k += 4) {  // four entries' loads before their arithmetic
+        const int4 q4 = __ldg(reinterpret_cast<const int4*>(LV.p + list_off(k)));
+        const int q[4] = {q4.x, k + 1 < cnt ? q4.y : (int)p, k + 2 < cnt ? q4.z : (int)p, k + 3 < cnt ? q4.w : (int)p};
+        float4 rec[4][2], uu[4];
+        float2 dq[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            rec_load(w, q[e], rec[e][0], rec[e][1]);
+            uu[e] = __ldg(b.xdf + q[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dq[e] = b.dEdnf[__float_as_int(rec[e][0].w) >> 4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (k + e < cnt) add(q[e], rec[e], uu[e], dq[e]);
+    }
     if (dLdx) {
         const double uc = kHartreeEV / kBohrA;
         const double ge = gE[s];
