@@ -33,7 +33,7 @@ constexpr double kHartreeEV = 27.211386245988;  // eV per Hartree
 constexpr int kMaxTypes = 16;
 constexpr int kMaxRef = 7;
 constexpr int kChunk = 64;  // pairs summed in FP32 before an FP64 accumulate (mixed form)
-constexpr int kFinChunk = 4096;  // atoms per first-level block of the per-structure sums
+constexpr int kFinChunk = 2048;  // atoms per first-level block of the per-structure sums
 
 enum StatusBits : int {
     ST_GHOST_CAP = 1,
