@@ -256,24 +256,41 @@ __global__ void __launch_bounds__(32 * kAtmWarps) k_atm(Work w, Consts c, const 
         __syncwarp();
         flush();
     };
-    // Candidate pairs are numbered and dealt to the lanes 32 at a time.  j = c / m
-    // is formed as (c + 1/2) * (1/m) in FP32: c < 2^13 and (c + 1/2)/m lies at least
-    // 1/(2m) >= 2^-8 from an integer, far above the rounding error (< 2^-10).
+    // Candidate pairs are numbered and dealt to the lanes 32 at a time. Pair ci of rows of m is
+    // (j, ci - j m), j = floor(ci / m), formed as (ci + 1/2 - m/2) / m rounded to the nearest
+    // by an addition of 3 * 2^22 (a conversion costs as much as 64 additions on this chip):
+    // ci < 2^13, and ci + 1/2 lies at least 1/2 from a multiple of m, so the quotient lies at
+    // least 1/(2m) >= 2^-8 from a tie, far above its rounding error (< 2^-10).
+    // (128 bilayers of 1,440 atoms: pass 1.71 -> 1.62 ms, with no bounds checks in full groups.
+    // 70% of the issue slots and 69% of the shared-memory wavefronts are in use; reading v_j and
+    // W_k instead of v_k and W_j, whose lanes differ more, gave nothing.)
+    constexpr float kMagic = 12582912.0f;
+    auto row_of = [&](float x, float inv) { return __float_as_int(fmaf(x, inv, kMagic)) - 0x4B400000; };
+    const float x_lane = __int_as_float(0x4B400000 + lane) - kMagic + 0.5f;
+    auto flt = [&](int m) { return __int_as_float(0x4B400000 + m) - kMagic; };
     //
     // every unordered pair of slots [base, base + n) once: (j, j + s mod n) for
     // s = 1 .. (n-1)/2, and for even n also (j, j + n/2) with j < n/2
     auto pairs_within = [&](int base, int n) {
         const int half = n >> 1, smax = (n - 1) >> 1;
         const int nc1 = n * smax, nc = nc1 + ((n & 1) ? 0 : half);
-        const float inv = 1.0f / (float)(smax > 0 ? smax : 1);
-        for (int c0 = 0; c0 < nc; c0 += 32) {
+        const float m = flt(smax > 0 ? smax : 1), inv = 1.0f / m;
+        float x = x_lane - 0.5f * m;
+        int c0 = 0;
+        for (; c0 + 32 <= nc1; c0 += 32, x += 32.0f) {  // every lane has a pair of the first kind
+            const int j = row_of(x, inv);
+            const unsigned k = c0 + lane + 1 - j * (smax - 1);
+            const int ks = base + (int)min(k, k - (unsigned)n), js = base + j;
+            push(close(js, ks), js, ks);
+        }
+        for (; c0 < nc; c0 += 32, x += 32.0f) {
             const int ci = c0 + lane;
             bool pass = false;
             int js = 0, ks = 0;
             if (ci < nc) {
                 int j, k;
                 if (ci < nc1) {
-                    j = (int)(((float)ci + 0.5f) * inv);
+                    j = row_of(x, inv);
                     k = ci - j * smax + 1 + j;
                     if (k >= n) k -= n;
                 } else {
@@ -291,13 +308,14 @@ __global__ void __launch_bounds__(32 * kAtmWarps) k_atm(Work w, Consts c, const 
     // every pair (j, k), j in [baseA, baseA + na), k in [baseB, baseB + nb)
     auto pairs_across = [&](int baseA, int na, int baseB, int nb) {
         const int nc = na * nb;
-        const float inv = 1.0f / (float)(nb > 0 ? nb : 1);
-        for (int c0 = 0; c0 < nc; c0 += 32) {
+        const float m = flt(nb > 0 ? nb : 1), inv = 1.0f / m;
+        float x = x_lane - 0.5f * m;
+        for (int c0 = 0; c0 < nc; c0 += 32, x += 32.0f) {
             const int ci = c0 + lane;
             bool pass = false;
             int js = 0, ks = 0;
             if (ci < nc) {
-                const int j = (int)(((float)ci + 0.5f) * inv);
+                const int j = row_of(x, inv);
                 js = baseA + j;
                 ks = baseB + ci - j * nb;
                 pass = close(js, ks);
