@@ -309,14 +309,12 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
             if (!cn_pair_precise(S, q, rrow, k1, rc2, c.rc_cn2, D, r2, ah, al, rch, tq, &rcl, &r2l, &y, rec_q))
                 return 0.0f;
             const CnDS z = cn_ds(ah, al, exptab);
-            if (z.th < 1.0f) {
-                ++nint;
-                acc_add(nh, nl, -z.ch);
-                nl -= z.cl;
-            } else {
-                acc_add(nh, nl, z.fh);
-                nl += z.fl;
-            }
+            // (one sum with its term selected: 184,320 atoms 94.7 -> 90.7 us, the two branches
+            // each with a sum diverged)
+            const bool near = z.th < 1.0f;
+            nint += near;
+            acc_add(nh, nl, near ? -z.ch : z.fh);
+            nl += near ? -z.cl : z.fl;
             return chain_coef(z, y, r2, r2l, rch, rcl, k1);
         };
         for (int k = 0; k < cnt; k += 4) {
