@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(128) kb_cn(Work w, BW b, BConsts c, const doub
             const double du = fma(dx, uq.x - ux.x, fma(dy, uq.y - ux.y, dz * (uq.z - ux.z)));
             const double rinv = __double2hiint(r2) > 0x00100000 ? rsqrt64(r2) : 1.0 / sqrt(r2);
             const double a = krow[rec_tsrc(w, q) & 15];
-            const double t = exp64(fma(-a, rinv, c.k1), exptab64);
+            const double t = exp64_int(fix53(fma(-a, rinv, c.k1)), exptab64);
             const double f = rcp64(1.0 + t);
             const double ri2 = rinv * rinv, ar = a * rinv;
             o.x = -(ar * ri2) * (t * f * f);

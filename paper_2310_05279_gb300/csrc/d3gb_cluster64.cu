@@ -136,18 +136,9 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
         }
         const int ev = (int)rv[2 * R], ed = (int)(rv[2 * R] >> 32);
         const int kDj = __ldg(w.kd + src);
-        // pair vector, and r^2 = r2u 2^(-36 - 2 sh) from it normalised by its largest component
         long long dx = ya.x - xa.x, dy = ya.y - xa.y, dz = yb.x - xb.x;
-        const unsigned long long o = (unsigned long long)((dx ^ (dx >> 63)) | (dy ^ (dy >> 63)) | (dz ^ (dz >> 63)));
-        const int sh = __clzll((long long)o) - 1;
-        const long long nx = dx << sh, ny = dy << sh, nz = dz << sh;
-        const unsigned long long r2u = (unsigned long long)(__mul64hi(nx, nx) + __mul64hi(ny, ny)) +
-                                       (unsigned long long)__mul64hi(nz, nz);
-        const int lz = __clzll((long long)r2u);
-        const unsigned long long mant = r2u << lz;
-        const unsigned long long bits = ((unsigned long long)(unsigned)(1049 - 2 * sh - lz) << 52) + (mant >> 11) +
-                                        ((mant >> 10) & 1);  // (the leading bit adds one to the exponent)
-        const double r2 = r2u ? __longlong_as_double((long long)bits) : 0.0;
+        unsigned long long mant;
+        const double r2 = ipos_r2(dx, dy, dz, mant);
         const double* t = trow + kDamp * (tsq & 15);
         // damping: g = -de/dC6 = s6/(r^6 + R^6) + s8 R0^2/(r^8 + R^8), fc0 = (de/dr)/(C6 r)
         const double r4 = r2 * r2, r6 = r4 * r2;
