@@ -514,7 +514,7 @@ def rooflines(fwd, fp64, batch, peaks, rates, sm_count, fmax, pairs):
                                         "k_build_clist")
     if fp64 is not None:
         r["fp64_roofline"] = alu_roofline(
-            "k_disp<FP64> (per-atom full lists: each pair evaluated from both atoms)", ops * pairs,
+            "k_disp_cl64 (cluster half lists; all but the damping function on the integer pipe: can exceed 1)", ops * pairs,
             fp64["stage_ms"]["disp"], rates["fp64_lane_ops_per_s"], "T FP64 lane-instructions/s",
             f"{ops:.1f} lane instructions per unique pair (DFMA = 1) x {pairs:,} pairs",
             {"peak_source": "measured DFMA lane rate (d3_peak_rates: independent FMA chains, 8 blocks of 256 "

@@ -467,9 +467,10 @@ __device__ __forceinline__ void cluster_finish(ClusterPass<R, SITE, SPLIT>& P, c
 
 // IMGSRC: image atoms have no rows of their own; each list entry's source atom is
 // resolved once per block of 32 entries (from the image's compact record).
-// 57% of issue slots and 67% of the L1 data path's wavefronts (broadcast loads, shuffles,
-// reductions): both are shared out over more warps by holding two steps' neighbour data at
-// a time instead of four, for 128 registers and four 128-thread blocks (16 warps) per SM.
+// Bound by issue and latency: 61% of issue slots on the scan below, no pipe above 39%, 44% of
+// the L1 data path's wavefronts (broadcast loads, shuffles, reductions), and waits for the
+// neighbours' rows. More warps share that out: two steps' neighbour data are held at a time
+// instead of four, for 128 registers and four 128-thread blocks (16 warps) per SM.
 // Packed pairs of floats carry C6 with dC6/dn_j, and x with y of the pair vectors, forces
 // and virial. Measured on 128 x 1440 atoms, a 1,048,576-atom box and 512 uneven structures:
 // 320, 3030 and 1600 us with scalar arithmetic, 12 warps and the next two steps' loads
