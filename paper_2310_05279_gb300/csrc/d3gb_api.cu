@@ -903,7 +903,7 @@ int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
 // (64 structures, 63,709 atoms: 74 and 47 us; 256, 208,635 atoms: 150 and 128; 512, 497,680
 // atoms: 245 and 274); the chain pass does not (76 and 146 us on 208,635 atoms). With even
 // lists one thread per atom is the faster from some 50,000 atoms on (55,296 atoms in a box:
-// 43 and 48 us, 128 bilayers of 1440 atoms: 94 and 143).
+// 43 and 48 us, 128 bilayers of 1440 atoms: 91 and 143).
 int wide_passes(const d3_handle* h, const Plan& P) {
     if (h->prm.precision != D3_MIXED || P.Nr == 0) return 0;
     if (P.Nr <= 32768) return 3;
