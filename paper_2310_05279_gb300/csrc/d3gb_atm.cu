@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(32 * kAtmWarps) k_atm(Work w, Consts c, const 
     // ci < 2^13, and ci + 1/2 lies at least 1/2 from a multiple of m, so the quotient lies at
     // least 1/(2m) >= 2^-8 from a tie, far above its rounding error (< 2^-10).
     // (128 bilayers of 1,440 atoms: pass 1.71 -> 1.62 ms, with no bounds checks in full groups.
-    // 70% of the issue slots and 69% of the shared-memory wavefronts are in use; reading v_j and
+    // 69% of the issue slots and 65% of the shared-memory wavefronts are in use; reading v_j and
     // W_k instead of v_k and W_j, whose lanes differ more, gave nothing.)
     constexpr float kMagic = 12582912.0f;
     auto row_of = [&](float x, float inv) { return __float_as_int(fmaf(x, inv, kMagic)) - 0x4B400000; };
