@@ -198,10 +198,10 @@ struct d3_handle {
     double* d_rk = nullptr;
     double* d_k1rc = nullptr;    // k1 k2 (Rcov_i + Rcov_j)
     double* d_exptab64 = nullptr;  // 2^(j/64), j = 0..63
-    // bounds of the FP64 form over cluster lists (Consts::fx_*); fx_ok: finite and positive
+    float4* d_bound = nullptr;   // FP64 form: bounds of a pair's terms (Tabs::bound)
+    // FP64 form over cluster lists: whether the bounds can be formed, and their constants (Consts)
     bool fx_ok = false;
-    int fx_e[5] = {}, fx_dsh = 0;
-    float fx_ratio = 1.0f;
+    float fx_s6 = 0.0f, fx_r2min = 0.0f;
     int* d_status = nullptr;
     int* h_status = nullptr;                 // pinned host word for the status read of the host-buffer path
     unsigned long long* d_nbuild = nullptr;  // builds executed on the device
@@ -263,62 +263,59 @@ double det3(const double* H) {
     return H[0] * (H[4] * H[8] - H[5] * H[7]) - H[1] * (H[3] * H[8] - H[5] * H[6]) + H[2] * (H[3] * H[7] - H[4] * H[6]);
 }
 
-// Bounds on one pair's terms over all element pairs and distances (FP64 form over
-// cluster lists): with C the largest |C6 reference| of the pair, x = |s6|, y = |s8| R0^2,
-//   de/dC6          x / R^6 + y / R^8                               (at r = 0)
-//   |C6 de/dC6|     C times that
-//   |de/dr|         C (1.56 x / R^7 + 2.03 y / R^9)                  (6 u^5/(1 + u^6)^2 <= 1.56, 8 u^7/(1 + u^8)^2 <= 2.03)
-//   r |de/dr|       C (1.5 x / R^6 + 2 y / R^8)                      (at r = R)
-//   |de/dr| / r     C (1.69 x / R^8 + 2.14 y / R^10)                 (6 u^4/(1 + u^6)^2, 8 u^6/(1 + u^8)^2)
-// and fx_ratio the largest ratio of a pair's terms at r >= R_cn to these bounds (every
-// term falls with r beyond R).  Exponents e with bound < 2^e.
-void fixed_point_bounds(d3_handle* h) {
+// Bounds of a pair's terms for the FP64 form over cluster lists (SumBound, RowBound in d3gb_passes.cu).
+// With x = |s6|, y = |s8| R0^2 and a C6 of 1, any distance gives
+//   de/dC6          at most x / R^6 + y / R^8                    (at r = 0)
+//   |de/dr|         1.56 x / R^7 + 2.03 y / R^9                  (6 u^5/(1 + u^6)^2 <= 1.56, 8 u^7/(1 + u^8)^2 <= 2.03)
+//   r |de/dr|       1.5 x / R^6 + 2 y / R^8                      (at r = R)
+// and every term falls with r beyond R.  The device forms an atom's bounds in FP32: the pass is used where
+// the largest of these lie well within its range, R within 1e-3 to 1e4 bohr, and R_cn is at least 4 A, so that
+// the partners beyond it, counted but not measured, don't set the units of sums that nearer ones make.
+// tab: Tabs::bound.
+void fixed_point_bounds(d3_handle* h, std::vector<float4>& tab) {
     const int T = h->T, R = h->R;
-    double mx[5] = {}, far[4] = {};
+    tab.assign(2 * (size_t)T * T, make_float4(0.f, 0.f, 0.f, 0.f));
+    double mx[4] = {}, rmin = 1e300;
     bool ok = true;
     const double rcn = h->prm.rc_cn_A / kBohrA;
+    const double x = std::fabs(h->prm.s6);
     for (int a = 0; a < T; ++a)
         for (int b = 0; b < T; ++b) {
             double C = 0.0;
             for (int k = 0; k < R * R; ++k) C = std::max(C, std::fabs(h->c6[((size_t)a * T + b) * R * R + k]));
             const double q = 3.0 * h->sqrtq[a] * h->sqrtq[b], Rd = std::fabs(h->prm.a1 * std::sqrt(q) + h->prm.a2_bohr);
-            const double x = std::fabs(h->prm.s6), y = std::fabs(h->prm.s8) * q;
+            const double y = std::fabs(h->prm.s8) * q;
             const double R2 = Rd * Rd, R6 = R2 * R2 * R2, R8 = R6 * R2;
-            const double r = std::max(rcn, Rd), r2 = r * r, r6 = r2 * r2 * r2, r8 = r6 * r2;
-            const double d6 = r6 + R6, d8 = r8 + R8, n6 = rcn * rcn * rcn * rcn * rcn * rcn;
-            const double v[4] = {C * (1.56 * x / (R6 * Rd) + 2.03 * y / (R8 * Rd)), C * (x / R6 + y / R8),
-                                 C * (1.5 * x / R6 + 2.0 * y / R8), x / R6 + y / R8};
-            const double g = x / (n6 + R6) + y / (n6 * rcn * rcn + R8);
-            const double f = 6.0 * x * r6 / r / (d6 * d6) + 8.0 * y * r8 / r / (d8 * d8);
-            const double u[4] = {C * f, C * g, C * f * r, g};
+            double f = 1.56 * x / (R6 * Rd) + 2.03 * y / (R8 * Rd), v = 1.5 * x / R6 + 2.0 * y / R8, g = x / R6 + y / R8;
+            const double top[4] = {C * f, C * v, C * g, g};
             for (int k = 0; k < 4; ++k) {
-                ok = ok && std::isfinite(v[k]) && std::isfinite(u[k]);
-                mx[k] = std::max(mx[k], v[k]);
-                far[k] = std::max(far[k], u[k]);
+                ok = ok && std::isfinite(top[k]);
+                mx[k] = std::max(mx[k], top[k]);
             }
-            mx[4] = std::max(mx[4], C * (1.69 * x / R8 + 2.14 * y / (R8 * R2)));
-            ok = ok && R8 > 1e-200;
+            const double r2 = rcn * rcn, r6 = r2 * r2 * r2, r8 = r6 * r2, d6 = r6 + R6, d8 = r8 + R8;
+            g = x / d6 + y / d8;
+            if (rcn >= Rd) {
+                v = 6.0 * x * (r6 / d6) / d6 + 8.0 * y * (r8 / d8) / d8;
+                f = v / rcn;
+            }
+            ok = ok && C < 1e30 && x < 1e30 && y < 1e30 && std::isfinite(f + v + g) && Rd >= 1e-3 && Rd <= 1e4;
+            rmin = std::min(rmin, Rd);
+            tab[(size_t)a * T + b] = make_float4((float)C, (float)R6, (float)R8, (float)y);
+            tab[(size_t)T * T + a * T + b] = make_float4((float)f, (float)v, (float)g, 0.f);
         }
-    double ratio = 0.0;
-    for (int k = 0; k < 5; ++k) {
-        ok = ok && mx[k] > 1e-100 && mx[k] < 1e100;
-        if (!ok) continue;
-        h->fx_e[k] = std::ilogb(mx[k]) + 1;
-        if (k < 4) ratio = std::max(ratio, far[k] / mx[k]);
-    }
-    // pair vectors (units of 2^-50 bohr, below 2^dexp bohr) are shifted left to at most 62 bits, and by no
-    // more than leaves a lane's virial sum, in units 2^(14 - dsh) of the force's, below 2^58
-    const int dexp = std::ilogb(h->prm.rc_disp_A / kBohrA) + 1;
-    h->fx_dsh = ok ? std::min(12 - dexp, 11 - (h->fx_e[2] - h->fx_e[0])) : 0;
-    ok = ok && h->fx_dsh >= 0;
-    h->fx_ok = ok;
-    h->fx_ratio = ok ? (float)std::min(1.0, 1.01 * ratio) : 1.0f;
+    for (int k = 0; k < 4; ++k) ok = ok && mx[k] > 1e-30 && mx[k] < 1e30;
+    // (and listed pair vectors, in units of 2^-50 bohr, stay below 2^62)
+    const double reach = std::max(h->prm.rc_disp_A, h->prm.rc_cn_A) + std::max(0.0, h->prm.skin_A);
+    h->fx_ok = ok && h->prm.rc_cn_A >= 4.0 && reach / kBohrA < 4000.0;
+    h->fx_s6 = (float)x;
+    h->fx_r2min = (float)(rmin * rmin / 16.0);
 }
 
 // Upload the damping table (R^6, R^8, s6, s8 R0^2 per element pair) in both precisions.
 d3_status upload_pair_table(d3_handle* h) {
     const int T = h->T;
-    fixed_point_bounds(h);
+    std::vector<float4> bnd;
+    fixed_point_bounds(h, bnd);
     std::vector<dbl4> pd(T * T), pb(T * T);
     std::vector<float4> pf(T * T);
     std::vector<double> rd(T * T);
@@ -339,6 +336,7 @@ d3_status upload_pair_table(d3_handle* h) {
     if (e == cudaSuccess) e = cudaMemcpy(h->d_rtabf, rf.data(), rf.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_pairf, pf.data(), pf.size() * sizeof(float4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_pairb, pb.data(), pb.size() * sizeof(dbl4), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_bound, bnd.data(), bnd.size() * sizeof(float4), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(h, e, "pair table upload");
     return D3_OK;
 }
@@ -379,13 +377,8 @@ Consts make_consts(const d3_handle* h) {
     c.alpha9f = (float)c.alpha9;
     c.alpha9_3f = (float)(c.alpha9 / 3.0);
     c.rc3_2f = (float)c.rc3_2;
-    c.fx_eF = h->fx_e[0];
-    c.fx_eE = h->fx_e[1];
-    c.fx_eV = h->fx_e[2];
-    c.fx_eG = h->fx_e[3];
-    c.fx_eM = h->fx_e[4];
-    c.fx_dsh = h->fx_dsh;
-    c.fx_ratio = h->fx_ratio;
+    c.fx_s6 = h->fx_s6;
+    c.fx_r2min = h->fx_r2min;
     return c;
 }
 
@@ -633,7 +626,8 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
             A(w.ipos, long long, 4 * Nt);
             A(w.row64, long long, Nr * h->T * row64_len(h->R));
             A(w.i64, long long, Nr * row64_len(h->R));
-            A(w.kd, int, Nr);
+            A(w.ks, int2, Nr);
+            A(w.tmask, int, B);
         }
         A(w.gate, int, 1);
         A(w.xref, double, 3 * Nr);
@@ -729,6 +723,7 @@ Tabs forward_tabs(const d3_handle* h) {
     tb.exptab = h->d_exptab;
     tb.k1rc = h->d_k1rc;
     tb.exptab64 = h->d_exptab64;
+    tb.bound = h->d_bound;
     tb.rtab = mixed ? (const void*)h->d_rtabf : (const void*)h->d_rtabd;
     return tb;
 }
@@ -1193,6 +1188,7 @@ d3_status d3_create(const d3_params* params, const d3_tables* tables, d3_handle*
     if (e == cudaSuccess) e = m.alloc(&h->d_rk, T);
     if (e == cudaSuccess) e = m.alloc(&h->d_k1rc, T * T);
     if (e == cudaSuccess) e = m.alloc(&h->d_exptab64, 64);
+    if (e == cudaSuccess) e = m.alloc(&h->d_bound, 2 * T * T);
     if (e == cudaSuccess) e = m.alloc(&h->d_status, 1);
     if (e == cudaSuccess) e = m.alloc(&h->d_nbuild, 1);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_nref, h->nref.data(), T * sizeof(int), cudaMemcpyHostToDevice);

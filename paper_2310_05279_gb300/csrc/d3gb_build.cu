@@ -393,6 +393,7 @@ __global__ void k_reset(Work w) {
         w.cnt_ghost[k] = 0;
     }
     if (k < 3 * (int64_t)w.B) w.maxcnt[k] = 0;
+    if (w.ipos && k < w.B) w.tmask[k] = 0;
     // occupied-range minima start at a huge float, maxima at +0
     if (k < 3 * (int64_t)w.B) {
         w.frange[k] = 0x7f7f7f7f;
@@ -473,6 +474,7 @@ __device__ __forceinline__ void fill_real(Work& w, int64_t p, int i, int s, cons
     if (t < 0 || t >= w.T) t = 0;
     w.perm[p] = i;
     w.sid[p] = s;
+    if (w.ipos && !((w.tmask[s] >> t) & 1)) atomicOr(&w.tmask[s], 1 << t);
     w.cell_sorted[p] = w.cell_of[i];
     const double x[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
     store_pos(w, p, x, rk_tab[t], t | ((int)p << 4));
@@ -617,6 +619,7 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
         fr[tid] = 0x7f7f7f7f;
         fr[3 + tid] = 0;
         w.maxcnt[3 * s + tid] = 0;
+        if (w.ipos) w.tmask[s] = 0;
     }
     __syncthreads();
     for (int k0 = 0; k0 < n; k0 += kStructThreads) {

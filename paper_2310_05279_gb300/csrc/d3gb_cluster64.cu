@@ -19,16 +19,18 @@
 //   * adds everything to per-atom 64-bit fixed-point sums, which associate, so the
 //     result does not depend on the order in which warps and splits of a list run.
 //
-// Scales.  A pair's terms are bounded (Becke-Johnson damping is finite at r = 0), and
-// terms beyond R_cn are smaller by fx_ratio; with the longest CN list and the fullest
-// cluster window of the structure that bounds every atom's sum within a factor of about
-// ten (fix_log2_pairs).  The scale leaves 61 bits to that bound: one unit is some 2^-57
-// of an atom's largest sum.  dE/dn has its own scale per atom, from its own dC6/dn.
-// Parameters whose bounds are not finite and positive keep the per-atom-list pass.
+// Units.  Each of an atom's sums (force, dE/dn, energy, virial) has its own unit, a power of
+// two that leaves 62 bits to a bound of the sum of its terms' sizes and 56 or 58 to one of its
+// largest term (SumBound, formed from the atom's own partners in the CN pass): below what
+// FP64 additions round.  A pair adds to i's sums in i's units and to j's in j's, which takes
+// nine 64-bit shifts a pair more than units for the whole batch.  (Units for
+// the whole batch, from the largest term of any element pair at r = 0, lost all digits at small
+// damping radii: at a1 = 0.05, a2 = 0.2 a C-C force at 5 A was off by 5e-5, at a2 = 0.003 by 1.)
+// Parameters beyond what the bounds hold in FP32 keep the per-atom-list pass.
 //
-// Measured on 128 x 1440 atoms (27.9 M pairs): 1.61 ms against 5.62 ms for the per-atom-list
-// pass, FP64 pipe 61% busy, 48% of issue slots used, 16 warps per SM (128 registers; at 142
-// registers and 12 warps 2.07 ms).
+// Measured on 128 x 1440 atoms (27.9 M pairs): 1.71 ms against 5.62 ms for the per-atom-list
+// pass, 16 warps per SM (128 registers; at 142 registers and 12 warps 2.07 ms); 1.61 ms with
+// units for the whole batch, 1.78 with 61 bits to every sum and shifts in both directions.
 #include "d3gb_pair.cuh"
 
 namespace d3gb {
@@ -44,6 +46,13 @@ __device__ __forceinline__ long long shr_rn(long long v, int s) {
     s = min(s, 62);
     return (v + (1LL << (s - 1))) >> s;
 }
+// the same for s >= 1 and several values
+struct Shift {
+    int s;
+    long long half;
+    __device__ __forceinline__ explicit Shift(int s1) : s(min(max(s1, 1), 62)), half(1LL << (s - 1)) {}
+    __device__ __forceinline__ long long operator()(long long v) const { return (v + half) >> s; }
+};
 // a normal double as m 2^(e - 1085), |m| in [2^62, 2^63)
 __device__ __forceinline__ long long mantissa(double v, int& e) {
     const long long b = __double_as_longlong(v);
@@ -55,17 +64,11 @@ __device__ __forceinline__ void red_add64(unsigned long long* a, long long x) {
     atomicAdd(a, (unsigned long long)x);  // result unused: a reduction, no return trip
 }
 
-// Scale exponents of a structure's force, energy and virial sums.
-struct FixScale {
-    int kF, kE, kV;  // kV: of a lane's sum; a cluster's has three bits less
-    int pv;          // bits that the virial's products take beyond the force sums'
-    __device__ FixScale(const Work& w, const Consts& c, int s) {
-        const int lg = fix_log2_pairs(w, c, s);
-        kF = min(61 - c.fx_eF - lg, 45 + c.fx_dsh - c.fx_eM);  // (the second: k_disp_cl64's sF stays above 0)
-        kE = 61 - c.fx_eE - lg;
-        pv = min(75 - c.fx_eV - lg - kF - c.fx_dsh, lg);  // (at least 3: fixed_point_bounds)
-        kV = kF + c.fx_dsh - 14 + pv;
-    }
+// The units of an atom's sums (Work::ks)
+struct Units {
+    int kF, kD, kE, kV;
+    __device__ __forceinline__ explicit Units(int2 k)
+        : kF((int)(short)k.x), kD(k.x >> 16), kE((int)(short)k.y), kV(k.y >> 16) {}
 };
 
 // Damping constants of an element pair in shared memory: R^6, R^8, s6, s8 R0^2, 6 s6, 8 s8 R0^2.
@@ -111,8 +114,7 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
     __syncwarp();
     const long long* wi = wsh + (int)(p - p0) * S64;
     const int eW = (int)wi[2 * R];
-    const int kDi = w.kd[p];
-    const FixScale K(w, c, s);
+    const Units K(w.ks[p]);
     const double* trow = tab + kDamp * ti * c.T;
     const long long* rbase = w.row64 + ti * S64;
     const int rstride = c.T * S64;
@@ -135,10 +137,11 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
             rv[a + 1] = t.y;
         }
         const int ev = (int)rv[2 * R], ed = (int)(rv[2 * R] >> 32);
-        const int kDj = __ldg(w.kd + src);
+        const Units J(__ldg(w.ks + src));
         long long dx = ya.x - xa.x, dy = ya.y - xa.y, dz = yb.x - xb.x;
         unsigned long long mant;
-        const double r2 = ipos_r2(dx, dy, dz, mant);
+        int sh;
+        const double r2 = ipos_r2(dx, dy, dz, sh, mant);
         const double* t = trow + kDamp * (tsq & 15);
         // damping: g = -de/dC6 = s6/(r^6 + R^6) + s8 R0^2/(r^8 + R^8), fc0 = (de/dr)/(C6 r)
         const double r4 = r2 * r2, r6 = r4 * r2;
@@ -157,39 +160,37 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
             dCi += __mul64hi(wi[R + a], rv[a]);   // 2^(eW + ev - 60)
             dCj += __mul64hi(W, rv[R + a]);       // 2^(ed - 61)
         }
-        C6 <<= 1;   // below 2^62 and a rounding error: the weights add up to 1
+        // |C6| is below 2^61 and a rounding error (the weights add up to 1): normalised to [2^61, 2^62)
+        const int sc = max(__clzll(C6 ^ (C6 >> 63)) - 2, 0), ec = ev - sc;
+        C6 <<= sc;  // units 2^(ec - 61)
         dCj <<= 1;
         int eg, ef;
         const long long mg = mantissa(g, eg), mf = mantissa(fc0, ef);
         // energy and dE/dn
-        const int sE = 1083 - eg - ev - K.kE + (SITE ? 1 : 0);  // SITE: half of it to each atom
-        const long long e = shr_rn(__mul64hi(mg, C6), sE);
-        aE += e;
-        aD += shr_rn(__mul64hi(mg, dCi), 1081 - eg - eW - ev - kDi);
+        // (terms of C6 lie in [2^59, 2^62) here, a virial's largest component in [2^57, 2^61): with the
+        // bits that the units leave to the bounds, every shift is at least 1)
+        const int sE = 1082 - eg - ec + (SITE ? 1 : 0);  // SITE: half of it to each atom
+        const long long e = __mul64hi(mg, C6);
+        aE += Shift(sE - K.kE)(e);
+        aD += shr_rn(__mul64hi(mg, dCi), 1081 - eg - eW - ev - K.kD);
         unsigned long long* aj = w.acc + 16 * src;
-        red_add64(aj + 3, shr_rn(__mul64hi(mg, dCj), 1083 - eg - ed - kDj));
-        if (SITE) red_add64(aj + 4, e);
-        // force, and the virial from it (rounded down: half a unit a pair is added at the end)
-        dx <<= c.fx_dsh; dy <<= c.fx_dsh; dz <<= c.fx_dsh;
-        const long long fC = __mul64hi(mf, C6) << 1;
-        // forces with pv bits more than their sums keep, for the virial
-        const int sF = min(1070 + c.fx_dsh - ef - ev - K.kF, 62) - K.pv;
-        const int dn = max(sF, 0), up = max(-sF, 0);
-        // (rounded: a half list's pair vectors do not cancel, so a bias would add up in the virial)
-        const long long h1 = (1LL << dn) >> 1, half = 1LL << (K.pv - 1);
-        const long long ux = (__mul64hi(fC, dx) + h1) >> dn << up, uy = (__mul64hi(fC, dy) + h1) >> dn << up,
-                        uz = (__mul64hi(fC, dz) + h1) >> dn << up;
-        const long long tx = (ux + half) >> K.pv, ty = (uy + half) >> K.pv, tz = (uz + half) >> K.pv;
-        aF[0] += tx; aF[1] += ty; aF[2] += tz;
-        red_add64(aj + 0, -tx);
-        red_add64(aj + 1, -ty);
-        red_add64(aj + 2, -tz);
-        aV[0] += __mul64hi(ux, dx);
-        aV[1] += __mul64hi(uy, dy);
-        aV[2] += __mul64hi(uz, dz);
-        aV[3] += __mul64hi(ux, dy);
-        aV[4] += __mul64hi(ux, dz);
-        aV[5] += __mul64hi(uy, dz);
+        red_add64(aj + 3, shr_rn(__mul64hi(mg, dCj), 1083 - eg - ed - J.kD));
+        if (SITE) red_add64(aj + 4, Shift(sE - J.kE)(e));
+        // force in units 2^-sF, and i's virial from it in units 2^-(sF + sh - 14)
+        const long long fC = __mul64hi(mf, C6) << 2;
+        const long long ux = __mul64hi(fC, dx), uy = __mul64hi(fC, dy), uz = __mul64hi(fC, dz);
+        const int sF = 1070 + sh - ef - ec;
+        const Shift fj(sF - J.kF), fi(sF - K.kF), vi(sF + sh - 14 - K.kV);
+        red_add64(aj + 0, -fj(ux));
+        red_add64(aj + 1, -fj(uy));
+        red_add64(aj + 2, -fj(uz));
+        aF[0] += fi(ux); aF[1] += fi(uy); aF[2] += fi(uz);
+        aV[0] += vi(__mul64hi(ux, dx));
+        aV[1] += vi(__mul64hi(uy, dy));
+        aV[2] += vi(__mul64hi(uz, dz));
+        aV[3] += vi(__mul64hi(ux, dy));
+        aV[4] += vi(__mul64hi(ux, dz));
+        aV[5] += vi(__mul64hi(uy, dz));
     };
     auto evaluate = [&]() {  // one pair per lane that has one
         if (n > 0) {
@@ -224,7 +225,6 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
     }
     while (__any_sync(0xffffffffu, n > 0)) evaluate();
 
-    const long long mine = npairs;  // the lane's pairs
     npairs = __reduce_add_sync(0xffffffffu, npairs);
     if (lane == 0 && w.npairs) atomicAdd(w.npairs, (unsigned long long)npairs);
     if (ilive) {
@@ -234,39 +234,25 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
         red_add64(ai + 2, aF[2]);
         red_add64(ai + 3, aD);
         red_add64(ai + 4, aE);
-        // the virial, in half units for the half that each pair's rounding lost on average: a
-        // cluster's sum of 32 lanes' (and splits') would need more bits than a word has, so the
-        // last four are added up on their own (13 bits each: at most 15 x 512)
-        unsigned long long* av = w.acc + 16 * p0 + 5;
-        unsigned long long rest[2] = {0, 0};
 #pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            const long long v = 2 * aV[m] + mine;
-            red_add64(av + m, v >> 4);
-            rest[m / 3] |= (unsigned long long)(v & 15) << (13 * (m % 3));
-        }
-        red_add64(av + 6, (long long)rest[0]);
-        red_add64(av + 7, (long long)rest[1]);
+        for (int m = 0; m < 6; ++m) red_add64(ai + 5 + m, aV[m]);
     }
 }
 
 // Per atom: the fixed-point totals into the arrays the chain pass, the per-structure
 // sums (and the optional three-body pass) read.
-__global__ void __launch_bounds__(256) k_disp_fin64(Work w, Consts c) {
+__global__ void __launch_bounds__(256) k_disp_fin64(Work w) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= w.Nr) return;
-    const FixScale K(w, c, w.sid[p]);
+    const Units K(w.ks[p]);
     const long long* a = reinterpret_cast<const long long*>(w.acc) + 16 * p;
     auto value = [](long long v, int k) { return ldexp((double)v, -k); };
     ((dbl4*)w.Fd)[p] = dbl4_make(value(a[0], K.kF), value(a[1], K.kF), value(a[2], K.kF), 0.0);
-    ((double*)w.dEdn)[p] = -value(a[3], w.kd[p]);
+    ((double*)w.dEdn)[p] = -value(a[3], K.kD);
     w.eat[p] = -value(a[4], K.kE);
     double* wv = w.wv + 6 * p;
 #pragma unroll
-    for (int m = 0; m < 6; ++m) {  // (zero but on a cluster's first atom)
-        const long long rest = (a[11 + m / 3] >> (13 * (m % 3))) & 8191;
-        wv[m] = a[5 + m] | rest ? -ldexp((double)a[5 + m] + 0.0625 * (double)rest, 3 - K.kV) : 0.0;
-    }
+    for (int m = 0; m < 6; ++m) wv[m] = -value(a[5 + m], K.kV);
 }
 
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -297,7 +283,7 @@ cudaError_t launch_disp_cl64(const Work& w, const Consts& c, const dbl4* pair_ta
         }
 #undef D3_CL
     }
-    k_disp_fin64<<<nblk(w.Nr, 256), 256, 0, st>>>(w, c);
+    k_disp_fin64<<<nblk(w.Nr, 256), 256, 0, st>>>(w);
     return cudaGetLastError();
 }
 

@@ -168,12 +168,13 @@ struct Work {
     int split_min;           // entries up to which one warp takes a cluster's whole list
     int split_on;            // some cluster of the plan has more
     unsigned long long* acc; // fixed-point sums of the dispersion pass: mixed [Nr][8] F (3), dE/dn, site energy;
-                             // FP64 [Nr][16] F (3), dE/dn, energy, and on a cluster's first atom its virial (6)
+                             // FP64 [Nr][16] F (3), dE/dn, energy, virial (6), in the atom's own units (ks)
     // FP64 form over cluster lists (d3gb_cluster64.cu): 64-bit integers scaled by powers of two
     long long* ipos;         // [Nr + ghost_cap][4] x, y, z in units of 2^-50 bohr, type | (source << 4)
     long long* row64;        // [Nr][T][row64_len(R)] rows v^(t), dv^(t) and their exponents
     long long* i64;          // [Nr][row64_len(R)] W, dW/dn and its exponent
-    int* kd;                 // [Nr] scale exponent of the atom's dE/dn sum
+    int2* ks;                // [Nr] units of the atom's sums, 2^-k: k of force, dE/dn (x) and energy, virial (y), 16 bits each
+    int* tmask;              // [B] the elements of each structure, one bit each
     double* gcnd;            // FP64 form: per CN-list entry, the chain coefficient f'(r)/r (as gcn)
     float* gcn;              // mixed form: per CN-list entry, the chain coefficient f'(r)/r of Eq. 4
                              // (written by the CN pass, 0 outside R_cn; read by the chain pass)
@@ -227,11 +228,9 @@ struct Consts {
     float s9f, alpha9f, alpha9_3f, rc3_2f;  // FP32 copies (alpha9_3f = alpha9 / 3) for the mixed form
     float k1f, rc_cn2f, k3f;   // FP32 copies for the mixed form
     float k3h, k3l;            // k3 as a float pair (k3h + k3l)
-    // FP64 form over cluster lists: binary exponents that bound one pair's force, energy and virial
-    // terms, de/dC6 and (de/dr)/r (Eq. 2), and the ratio of the bounds beyond R_cn to those at any distance
-    int fx_eF, fx_eE, fx_eV, fx_eG, fx_eM;
-    int fx_dsh;                // pair vectors: units of 2^-(50 + fx_dsh) bohr
-    float fx_ratio;
+    // FP64 form over cluster lists, for the bounds of a pair's terms (Tabs::bound): |s6|, and the r^2 below
+    // which a pair counts as one at that distance: (smallest damping radius / 4)^2
+    float fx_s6, fx_r2min;
 };
 
 // ---- neighbour lists: `cap` entries per atom (cap a multiple of 8).  The rows of
@@ -305,14 +304,6 @@ __host__ __device__ inline void unpack_shift(int s, int& a, int& b, int& c) {
     c = ((s >> 16) & 255) - 128;
 }
 
-// FP64 form over cluster lists: a bound on an atom's number of pairs of structure s,
-// weighted by the size their terms can have, as a binary logarithm (at least 5).  The
-// CN lists hold every partner within R_cn; beyond, terms are smaller by fx_ratio.
-__device__ __forceinline__ int fix_log2_pairs(const Work& w, const Consts& c, int s) {
-    const int n = w.maxcnt[3 * s + 1] + (int)(c.fx_ratio * (float)w.maxcnt[3 * s]) + 17;
-    return 32 - __clz(n);
-}
-
 // Structure of input atom i (binary search over offsets).
 __device__ inline int struct_of(const int64_t* off, int B, int64_t i) {
     int lo = 0, hi = B;  // off[lo] <= i < off[hi]
@@ -336,6 +327,8 @@ cudaError_t launch_check(const Work& w, const double* pos, cudaStream_t st);
 struct Tabs {
     const double* k1rc;    // [T][T] k1 k2 (Rcov_i + Rcov_j) (bohr), FP64 form
     const double* exptab64;  // [64] 2^(j/64), FP64 form
+    const float4* bound;   // FP64 form: [T][T] largest |C6 reference|, R^6, R^8, |s8| R0^2 of an element pair, then
+                           // [T][T] its largest force, virial and de/dC6 beyond R_cn, for a C6 of 1
     const void* c6;        // [T][T][R][R] real (float or double by precision)
     const void* pair;      // [T][T] real4: R^6, R^8, s6, s8 R0^2
     const double* cnref;   // [T][R]

@@ -91,19 +91,30 @@ __device__ __forceinline__ double exp64_int(long long X, const double* __restric
 
 // |d|^2 for integer pair vectors in units of 2^-50 bohr (Work::ipos), from the vector normalised
 // by its largest component: relative error a few 2^-58 before its rounding to FP64
-// (m: its mantissa before the rounding, leading bit 63; 0 for a zero vector)
-__device__ __forceinline__ double ipos_r2(long long dx, long long dy, long long dz, unsigned long long& m) {
+// (m: its mantissa before the rounding, leading bit 63; 0 for a zero vector).  d is left
+// normalised, in units of 2^-(50 + sh) bohr: its largest component lies in
+// [2^62, 2^63].
+__device__ __forceinline__ double ipos_r2(long long& dx, long long& dy, long long& dz, int& sh, unsigned long long& m) {
     const unsigned long long o = (unsigned long long)((dx ^ (dx >> 63)) | (dy ^ (dy >> 63)) | (dz ^ (dz >> 63)));
-    const int sh = __clzll((long long)o) - 1;
-    const long long nx = dx << sh, ny = dy << sh, nz = dz << sh;
-    const unsigned long long r2u = (unsigned long long)(__mul64hi(nx, nx) + __mul64hi(ny, ny)) +
-                                   (unsigned long long)__mul64hi(nz, nz);
+    sh = __clzll((long long)o) - 1;
+    dx <<= sh;
+    dy <<= sh;
+    dz <<= sh;
+    const unsigned long long r2u = (unsigned long long)(__mul64hi(dx, dx) + __mul64hi(dy, dy)) +
+                                   (unsigned long long)__mul64hi(dz, dz);
     const int lz = __clzll((long long)r2u);
     const unsigned long long mant = r2u << lz;
     m = mant;
     const unsigned long long bits = ((unsigned long long)(unsigned)(1049 - 2 * sh - lz) << 52) + (mant >> 11) +
                                     ((mant >> 10) & 1);  // (the leading bit adds one to the exponent)
     return r2u ? __longlong_as_double((long long)bits) : 0.0;
+}
+
+// a positive double cut off to FP32 on the integer pipe (from 2^-126 on; below, 2^-126)
+__device__ __forceinline__ float cut32(double x) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)(b >> 52) - 896;  // the exponent field of the FP32 number
+    return __int_as_float(e > 0 ? (e << 23) | (int)((b >> 29) & 0x7fffff) : 0x00800000);
 }
 
 // 1 - r2 y^2 in units of 2^-62 for y near r2^(-1/2) (to 2^-40 or so), r2 with mantissa m (leading

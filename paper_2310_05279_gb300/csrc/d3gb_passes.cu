@@ -85,10 +85,17 @@ __device__ __forceinline__ long long fix_value(double v, int e, int bits) {
 // (and, for the cluster-list dispersion pass, the same values beside those of
 // dv_p^(u)_a = sum_b C6ref[u][t][a][b] dW_b in w.vd)
 // (u0, us: the partner types u0, u0 + us, ... are this thread's; u0 = 0 stores the rest)
+// FP64 form over cluster lists: *rb gets bounds that hold for any partner (the weights of Eq. 3 add up to 1)
+struct RowBound {
+    int ed = -1022;                            // |dC6/dn_p| < 2^ed
+    float f = 0.f, e = 0.f, v = 0.f, g = 0.f;  // a pair's force, energy, virial and de/dC6 beyond R_cn
+    float part = 0.f;                          // |C6| over the element pair's largest
+};
 template <class T, int R>
 __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, const T* __restrict__ c6, int64_t p, int t,
                                               const T (&L)[R], const T (&Wr)[8], const T (&dWr)[8], int u0 = 0,
-                                              int us = 1) {
+                                              int us = 1, const float4* __restrict__ bound = nullptr,
+                                              RowBound* rb = nullptr) {
     if (u0 == 0) {
         store_row<T>((T*)w.W + p * c.RP, Wr, c.RP);
         store_row<T>((T*)w.dW + p * c.RP, dWr, c.RP);
@@ -96,7 +103,6 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
     T* vp = (T*)w.v + p * c.T * c.RP;
     T* dvp = (sizeof(T) == 4 && w.vd) ? (T*)w.vd + p * c.T * 2 * c.RP : nullptr;  // [T][RP][2] per atom
     constexpr int S64 = row64_len(R);
-    int edmax = -1022;  // FP64 form: |dv| < 2^edmax over all rows
     for (int u = u0; u < c.T; u += us) {
         const T* cu = c6 + ((size_t)(u * c.T + t) * R) * R;  // C6ref[u][t][a][b]
         T vr[8], dvr[8];
@@ -118,7 +124,16 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
             if (w.row64) {
                 long long* r64 = w.row64 + (p * c.T + u) * S64;
                 const int ev = fix_exponent(vr, R), ed = fix_exponent(dvr, R);
-                edmax = max(edmax, ed);
+                rb->ed = max(rb->ed, ed);
+                if ((w.tmask[w.sid[p]] >> u) & 1) {  // |C6| of p and a partner of type u is below 2^ev
+                    const float4 far = __ldg(bound + (c.T + t) * c.T + u);
+                    const float C = __ldg(&bound[t * c.T + u].x), C6 = fminf(__int_as_float((max(ev, -100) + 127) << 23), C);
+                    rb->f = fmaxf(rb->f, C6 * far.x);
+                    rb->v = fmaxf(rb->v, C6 * far.y);
+                    rb->e = fmaxf(rb->e, C6 * far.z);
+                    rb->g = fmaxf(rb->g, far.z);
+                    rb->part = fmaxf(rb->part, C > 0.0f ? C6 / C : 0.0f);
+                }
 #pragma unroll
                 for (int a = 0; a < R; ++a) {
                     r64[a] = fix_value(vr[a], ev, 63);
@@ -144,8 +159,6 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
                 q[R + a] = fix_value(dWr[a], ew, 61);
             }
             q[2 * R] = ew;
-            // |dC6/dn_p| < 2^edmax for any partner (the weights of Eq. 3 add up to 1)
-            w.kd[p] = min(900, 61 - (edmax + c.fx_eG + fix_log2_pairs(w, c, w.sid[p])));
         }
     }
     if (u0 != 0) return;
@@ -163,7 +176,7 @@ template <bool MIXED, int R>
 __device__ __forceinline__ void weights_atom(const Work& w, const Consts& c, const double* __restrict__ cnref,
                                              const int* __restrict__ nref,
                                              const typename Real<MIXED>::T* __restrict__ c6, int64_t p, int t,
-                                             double n) {
+                                             double n, const float4* __restrict__ bound, RowBound* rb) {
     using T = typename Real<MIXED>::T;
     const int nr = nref[t];
     double cr[R], x[R];
@@ -208,8 +221,50 @@ __device__ __forceinline__ void weights_atom(const Work& w, const Consts& c, con
             Wr[a] = dWr[a] = 0;
         }
     }
-    store_weights<T, R>(w, c, c6, p, t, L, Wr, dWr);
+    store_weights<T, R>(w, c, c6, p, t, L, Wr, dWr, 0, 1, bound, rb);
 }
+
+// FP64 form over cluster lists: bounds of an atom's sums, from those of its pairs (FP32; Becke-Johnson
+// damping is finite at any distance).  With C the largest |C6 reference| of the element pair,
+// i6 = 1/(r^6 + R^6) and i8 = 1/(r^8 + R^8):
+//   de/dC6  |s6| i6 + |s8| R0^2 i8        energy  C de/dC6
+//   virial  C (6 |s6| r^6 i6^2 + 8 |s8| R0^2 r^8 i8^2)        force  virial / r
+// The partners within R_cn are taken at their distance (but no nearer than a quarter of the
+// smallest R: below R force and virial fall towards r = 0 and de/dC6 is flat), the others, at
+// most as many as the fullest cluster window of the structure holds, at R_cn (RowBound).
+struct SumBound {
+    float f = 0.f, e = 0.f, v = 0.f, g = 0.f;  // sums, and the largest term of each
+    float f1 = 0.f, e1 = 0.f, v1 = 0.f;
+    // b: C, R^6, R^8, |s8| R0^2
+    __device__ __forceinline__ void add(const Consts& c, const float4& b, double r2d) {
+        const float r2 = fmaxf(cut32(r2d), c.fx_r2min), r4 = r2 * r2, r6 = r4 * r2, r8 = r4 * r4;
+        const float i6 = rcp_approx(r6 + b.y), i8 = rcp_approx(r8 + b.z);
+        const float t6 = c.fx_s6 * i6, t8 = b.w * i8;
+        const float cv = b.x * fmaf(6.0f * t6, r6 * i6, 8.0f * t8 * (r8 * i8));
+        const float ce = b.x * (t6 + t8), cf = cv * rsqrt_approx(r2);
+        g += t6 + t8;
+        e += ce;
+        v += cv;
+        f += cf;
+        e1 = fmaxf(e1, ce);
+        v1 = fmaxf(v1, cv);
+        f1 = fmaxf(f1, cf);
+    }
+    // The units of the atom's sums (Work::ks): 62 bits to the bound of a sum, so that no partial sum
+    // overflows, and 58 (force, energy) and 56 (virial) to that of a term, which k_disp_cl64's
+    // mantissas have at least.  A unit then lies below an FP64 rounding of the sum of the terms' sizes,
+    // whatever the damping, the other elements of the table and the other atoms of the structure.
+    __device__ __forceinline__ int2 units(const RowBound& rb, int nfar) const {
+        const float n = (float)nfar;
+        auto above = [](float x) { return (__float_as_int(1.05f * x) >> 23) - 126; };  // x < 2^above(x)
+        auto k = [&](int bits, float sum, float term, float beyond) {
+            const int a = 62 - above(fmaf(n, beyond, rb.part * sum)), b = bits - above(fmaxf(beyond, rb.part * term));
+            return max(-900, min(900, min(a, b)));
+        };
+        const int kD = max(-900, min(900, 62 - above(fmaf(n, rb.g, g)) - rb.ed));
+        return make_int2((k(58, f, f1, rb.f) & 0xffff) | (kD << 16), (k(58, e, e1, rb.e) & 0xffff) | (k(56, v, v1, rb.v) << 16));
+    }
+};
 
 // Mixed form of the above without FP64 (GB300 runs FP64 at 1/64 of the FP32
 // rate): the exponents -k3 (n - nref_a)^2 are formed in float-float from
@@ -288,12 +343,14 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
                                            const float2* __restrict__ cnref2, const float* __restrict__ dcr,
                                            const int* __restrict__ nref,
                                            const typename Real<MIXED>::T* __restrict__ c6,
-                                           const double* __restrict__ k1rc, const double* __restrict__ exptab64) {
+                                           const double* __restrict__ k1rc, const double* __restrict__ exptab64,
+                                           const float4* __restrict__ bound) {
     using T = typename Real<MIXED>::T;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= w.Nr) return;
     const Site<MIXED> S(w, p);
-    const StructGeo& G = w.geo[w.sid[p]];
+    const int s = w.sid[p];
+    const StructGeo& G = w.geo[s];
     const ListView LV{w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn)};
     const int cnt = w.cnt_cn[p];
     const T rc2 = MIXED ? (T)c.rc_cn2f : (T)c.rc_cn2, k1 = MIXED ? (T)c.k1f : (T)c.k1;
@@ -353,8 +410,11 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
         // kept for the chain pass. The FP64 pipe bounds the pass (80 issue slots an instruction),
         // so where positions stand as integers too, the pair vector, r^2 and the exponential are
         // formed from them: 16 FP64 instructions a pair instead of 33, 9.4 M entries 0.77 -> 0.46 ms
-        // (0.91 with the library's exp, square root and divisions).
-        const double* krow = k1rc + (S.tsrc() & 15) * c.T;
+        // (0.91 with the library's exp, square root and divisions; 0.47 with the bounds of SumBound).
+        const int t = S.tsrc() & 15;
+        const double* krow = k1rc + t * c.T;
+        const float4* brow = bound + t * c.T;
+        SumBound sb;
         double* grow = w.gcnd + (LV.p - w.nbr_cn);
         const bool ints = w.ipos != nullptr;
         longlong2 xa = make_longlong2(0, 0), xb = xa;
@@ -373,7 +433,9 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
             if (ints) {
                 const longlong2* x2 = reinterpret_cast<const longlong2*>(w.ipos + 4 * (int64_t)q);
                 const longlong2 ya = __ldg(x2), yb = __ldg(x2 + 1);
-                r2 = ipos_r2(ya.x - xa.x, ya.y - xa.y, yb.x - xb.x, mant);
+                long long nx = ya.x - xa.x, ny = ya.y - xa.y, nz = yb.x - xb.x;
+                int sh;
+                r2 = ipos_r2(nx, ny, nz, sh, mant);
                 tq = (int)yb.y;
                 const long long d = __double_as_longlong(r2) - rcb;  // (positive doubles order as their bits)
                 if (d > 64) return 0.0;
@@ -382,6 +444,7 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
                     S.dist(q, dx, dy, dz, r2, tq, rkq);
                     if (!(r2 < c.rc_cn2)) return 0.0;
                 }
+                sb.add(c, __ldg(brow + (tq & 15)), r2);
             } else {
                 double dx, dy, dz, rkq;
                 S.dist(q, dx, dy, dz, r2, tq, rkq);
@@ -410,7 +473,9 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
             *reinterpret_cast<dbl4*>(grow + list_off(k)) = g;
         }
         w.cn[p] = (double)nh;
-        weights_atom<MIXED, R>(w, c, cnref, nref, c6, p, S.tsrc() & 15, (double)nh);
+        RowBound rb;
+        weights_atom<MIXED, R>(w, c, cnref, nref, c6, p, t, (double)nh, bound, &rb);
+        if (ints) w.ks[p] = sb.units(rb, w.maxcnt[3 * s]);
     }
 }
 
@@ -909,7 +974,8 @@ cudaError_t forward_impl(const Work& w, const Consts& c, const Tabs& tb, double*
                                                               (const float*)tb.c6);
     else if (w.Nr > 0)
         k_cn<MIXED, R><<<nblk(w.Nr, w.blk_cn), w.blk_cn, 0, st>>>(w, c, tb.rcpair, tb.exptab, tb.cnref, tb.cnref2,
-                                                                  tb.dcr, tb.nref, (const T*)tb.c6, tb.k1rc, tb.exptab64);
+                                                                  tb.dcr, tb.nref, (const T*)tb.c6, tb.k1rc, tb.exptab64,
+                                                                  tb.bound);
     mark(1);  // the weights (Eq. 3) are formed inside the CN pass
     mark(2);
     if (w.cl_mode && !w_atom) {
