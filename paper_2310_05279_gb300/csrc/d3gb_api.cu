@@ -304,9 +304,7 @@ void fixed_point_bounds(d3_handle* h, std::vector<float4>& tab) {
             tab[(size_t)T * T + a * T + b] = make_float4((float)f, (float)v, (float)g, 0.f);
         }
     for (int k = 0; k < 4; ++k) ok = ok && mx[k] > 1e-30 && mx[k] < 1e30;
-    // (and listed pair vectors, in units of 2^-50 bohr, stay below 2^62)
-    const double reach = std::max(h->prm.rc_disp_A, h->prm.rc_cn_A) + std::max(0.0, h->prm.skin_A);
-    h->fx_ok = ok && h->prm.rc_cn_A >= 4.0 && reach / kBohrA < 4000.0;
+    h->fx_ok = ok && h->prm.rc_cn_A >= 4.0;
     h->fx_s6 = (float)x;
     h->fx_r2min = (float)(rmin * rmin / 16.0);
 }
@@ -464,6 +462,10 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
             G.win_cn[k] = (int)std::min<long long>(nck, (long long)std::ceil(rln / cw));
             nc_total *= nck;
         }
+        double pad = 1.0 + 2.0 * std::max(0.0, h->prm.skin_A) / kBohrA;
+        for (int k = 0; k < 3; ++k)
+            pad += G.img[k] * std::max(std::fabs(G.H[3 * k]), std::max(std::fabs(G.H[3 * k + 1]), std::fabs(G.H[3 * k + 2])));
+        G.ipad = (float)(1.001 * pad);
         if (nc_total > ((int64_t)1 << 26)) return fail(h, D3_ERR_ARG, "too many cells for structure " + std::to_string(s));
         for (int k = 0; k < 9; ++k) {
             G.Hinvf[k] = (float)G.Hinv[k];
@@ -552,6 +554,8 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     w.blk_chain = h->shape[2];
     w.build_per_sm = h->shape[3];
     w.max_natoms = maxn;
+    // listed pair vectors, in units of 2^-iucap bohr, stay below 2^62
+    w.iucap = std::min(54, 60 - std::ilogb(std::max(list_radius(h, h->prm.rc_disp_A), list_radius(h, h->prm.rc_cn_A))));
     w.max_ncell = (int)std::min<int64_t>(P.max_ncell, 1 << 26);
     w.n_fin = nfin;
     // Lists longer than this are split over a block (k_disp_cl_split) where clusters are few: 64
@@ -628,6 +632,7 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
             A(w.i64, long long, Nr * row64_len(h->R));
             A(w.ks, int2, Nr);
             A(w.tmask, int, B);
+            A(w.ixmax, int, B);
         }
         A(w.gate, int, 1);
         A(w.xref, double, 3 * Nr);

@@ -80,8 +80,9 @@ __device__ __forceinline__ void add_lattice(double (&x)[3], const StructGeo& G, 
 // wrapped position, cell and in-cell key, returns the cell.  The lattice translation that
 // wraps an atom is chosen from its FP32 fractional coordinates; the wrapped position is
 // x - sum_k n_k H_k in FP64 (x itself when the atom is inside the cell).
-__device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int64_t i, const double* __restrict__ pos,
-                                         const int32_t* __restrict__ types, float (&f)[3]) {
+__device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int s, int64_t i,
+                                         const double* __restrict__ pos, const int32_t* __restrict__ types,
+                                         float (&f)[3]) {
     double xb[3];
     bool fin = true;
 #pragma unroll
@@ -115,11 +116,14 @@ __device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int6
     if (n[0] | n[1] | n[2]) add_lattice(xw, G, -n[0], -n[1], -n[2]);
     // the exact FP32 split of positions needs |x| < 2^13 bohr (checked in FP32)
     bool far = false;
+    float xmax = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float xr = xf[a] - ((float)n[0] * G.Hh[a] + (float)n[1] * G.Hh[3 + a] + (float)n[2] * G.Hh[6 + a]);
         far = far || !(fabsf(xr) < kMaxCoordBohr);
+        xmax = fmaxf(xmax, fabsf(xr));
     }
+    if (w.ipos && __float_as_int(xmax) > w.ixmax[s]) atomicMax(&w.ixmax[s], __float_as_int(xmax));
     if (far && fin) atomicOr(w.status, ST_RANGE);
 #pragma unroll
     for (int a = 0; a < 3; ++a) w.xw[3 * i + a] = xw[a];
@@ -157,7 +161,7 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
         const int s = w.sid_in[i];
         const StructGeo& G = w.geo[s];
         float f[3];
-        const int cid = wrap_atom(w, G, i, pos, types, f);
+        const int cid = wrap_atom(w, G, s, i, pos, types, f);
         w.slot_of[i] = atomicAdd(&w.cnt_real[cid], 1);
         // occupied range: one atomic per group of lanes in the same structure
         const unsigned grp = __match_any_sync(__activemask(), s);
@@ -393,7 +397,7 @@ __global__ void k_reset(Work w) {
         w.cnt_ghost[k] = 0;
     }
     if (k < 3 * (int64_t)w.B) w.maxcnt[k] = 0;
-    if (w.ipos && k < w.B) w.tmask[k] = 0;
+    if (w.ipos && k < w.B) w.tmask[k] = w.ixmax[k] = 0;
     // occupied-range minima start at a huge float, maxima at +0
     if (k < 3 * (int64_t)w.B) {
         w.frange[k] = 0x7f7f7f7f;
@@ -447,24 +451,22 @@ __device__ inline void split_pos(const double x[3], float (&h)[3], float (&l)[3]
         l[a] = (xh - h[a]) + xl;
     }
 }
-// Positions of the FP64 form over cluster lists, in units of 2^-50 bohr: exact for
-// |x| >= 4 bohr, where an FP64 ulp is no smaller, and rounded by at most 2^-51 below
-// (the FP64 difference of two positions some bohr apart rounds by as much).
-__device__ inline void store_ipos(Work& w, int64_t q, const double x[3], int tsrc) {
+// Positions of the FP64 form over cluster lists (ipos_unit).
+__device__ inline void store_ipos(Work& w, int64_t q, int s, const double x[3], int tsrc) {
     if (!w.ipos) return;
     longlong2* d = reinterpret_cast<longlong2*>(w.ipos + 4 * q);
-    const double u = 1125899906842624.0;
+    const double u = __longlong_as_double((long long)(1023 + ipos_unit(w, s)) << 52);
     d[0] = make_longlong2(__double2ll_rn(x[0] * u), __double2ll_rn(x[1] * u));
     d[1] = make_longlong2(__double2ll_rn(x[2] * u), (long long)tsrc);
 }
-__device__ inline void store_pos(Work& w, int64_t q, const double x[3], double rk, int tsrc) {
+__device__ inline void store_pos(Work& w, int64_t q, int s, const double x[3], double rk, int tsrc) {
     w.pos64[q] = dbl4_make(x[0], x[1], x[2], rk);
     float h[3], l[3];
     split_pos(x, h, l);
     w.rec[2 * q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
     w.rec[2 * q + 1] = make_float4(l[0], l[1], l[2], (float)rk);
     w.hi[q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
-    store_ipos(w, q, x, tsrc);
+    store_ipos(w, q, s, x, tsrc);
 }
 
 // Sorted slot p of real atom i.
@@ -477,14 +479,15 @@ __device__ __forceinline__ void fill_real(Work& w, int64_t p, int i, int s, cons
     if (w.ipos && !((w.tmask[s] >> t) & 1)) atomicOr(&w.tmask[s], 1 << t);
     w.cell_sorted[p] = w.cell_of[i];
     const double x[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
-    store_pos(w, p, x, rk_tab[t], t | ((int)p << 4));
+    store_pos(w, p, s, x, rk_tab[t], t | ((int)p << 4));
 }
 // Sorted image slot q of image record g.  An image's FP64 position is its source's plus
 // the lattice translation; its split is the source's (read from the source's record: forming
 // it again took 12 of 18 FP64 instructions an image, which bound the fill) plus the
 // translation's (grid parts add exactly), moved back to the nearest grid point (|lo| <=
 // 2^-11) by whole grid steps.
-__device__ __forceinline__ void fill_image(Work& w, int64_t q, int g, const StructGeo& G) {
+__device__ __forceinline__ void fill_image(Work& w, int64_t q, int g, int s) {
+    const StructGeo& G = w.geo[s];
     const int i = w.ghost_src[g];
     int n0, n1, n2;
     unpack_shift(w.ghost_shift[g], n0, n1, n2);
@@ -509,7 +512,7 @@ __device__ __forceinline__ void fill_image(Work& w, int64_t q, int g, const Stru
     w.rec[2 * (w.Nr + q)] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
     w.rec[2 * (w.Nr + q) + 1] = make_float4(l[0], l[1], l[2], sl.w);
     w.hi[w.Nr + q] = make_float4(h[0], h[1], h[2], __int_as_float(tsrc));
-    store_ipos(w, w.Nr + q, x, tsrc);
+    store_ipos(w, w.Nr + q, s, x, tsrc);
 }
 
 // Each slot's final place in its cell is the number of smaller keys in the cell
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(256) k_fill(Work w) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= min(*w.ghost_count, w.ghost_cap)) return;
     const int g = w.gsorted[q];
-    fill_image(w, q, g, w.geo[w.ghost_sid[g]]);
+    fill_image(w, q, g, w.ghost_sid[g]);
 }
 
 // ---- the steps above in one kernel, for batches of small structures
@@ -619,7 +622,7 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
         fr[tid] = 0x7f7f7f7f;
         fr[3 + tid] = 0;
         w.maxcnt[3 * s + tid] = 0;
-        if (w.ipos) w.tmask[s] = 0;
+        if (w.ipos) w.tmask[s] = w.ixmax[s] = 0;
     }
     __syncthreads();
     for (int k0 = 0; k0 < n; k0 += kStructThreads) {
@@ -628,7 +631,7 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
         float f[3] = {0.f, 0.f, 0.f};
         if (live) {
             const int64_t i = a0 + k;
-            const int cid = wrap_atom(w, G, i, pos, types, f);
+            const int cid = wrap_atom(w, G, s, i, pos, types, f);
             w.slot_of[i] = atomicAdd(&cr[cid - c0], 1);
         }
 #pragma unroll
@@ -719,7 +722,7 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
         const int q = g0 + b + rank;
         w.gsorted[q] = u;
         w.ginv[u] = q;
-        fill_image(w, q, u, G);
+        fill_image(w, q, u, s);
     }
 }
 

@@ -12,8 +12,7 @@
 //     every lane has one;
 //   * leaves to the FP64 pipe only the damping function (18 instructions a pair).
 //     Pair vectors, r^2, the C6 interpolation and all sums are formed on the integer
-//     pipe, with 64-bit mantissas scaled by powers of two: positions in units of
-//     2^-50 bohr; W, dW and the rows v, dv with one exponent per row (Work::i64,
+//     pipe, with 64-bit mantissas scaled by powers of two: positions (ipos_unit); W, dW and the rows v, dv with one exponent per row (Work::i64,
 //     row64); products as the upper half of 64 x 64 bits.  Their relative errors are
 //     2^-57 and less (the C6 sums: 2^-61 of the row's largest value), below FP64's 2^-53;
 //   * adds everything to per-atom 64-bit fixed-point sums, which associate, so the
@@ -28,7 +27,7 @@
 // damping radii: at a1 = 0.05, a2 = 0.2 a C-C force at 5 A was off by 5e-5, at a2 = 0.003 by 1.)
 // Parameters beyond what the bounds hold in FP32 keep the per-atom-list pass.
 //
-// Measured on 128 x 1440 atoms (27.9 M pairs): 1.71 ms against 5.62 ms for the per-atom-list
+// Measured on 128 x 1440 atoms (27.9 M pairs): 1.70 ms against 5.62 ms for the per-atom-list
 // pass, 16 warps per SM (128 registers; at 142 registers and 12 warps 2.07 ms); 1.61 ms with
 // units for the whole batch, 1.78 with 61 bits to every sum and shifts in both directions.
 #include "d3gb_pair.cuh"
@@ -141,7 +140,7 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
         long long dx = ya.x - xa.x, dy = ya.y - xa.y, dz = yb.x - xb.x;
         unsigned long long mant;
         int sh;
-        const double r2 = ipos_r2(dx, dy, dz, sh, mant);
+        const double r2 = ipos_r2(dx, dy, dz, (int)wi[2 * R + 1], sh, mant);
         const double* t = trow + kDamp * (tsq & 15);
         // damping: g = -de/dC6 = s6/(r^6 + R^6) + s8 R0^2/(r^8 + R^8), fc0 = (de/dr)/(C6 r)
         const double r4 = r2 * r2, r6 = r4 * r2;
@@ -176,11 +175,11 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
         unsigned long long* aj = w.acc + 16 * src;
         red_add64(aj + 3, shr_rn(__mul64hi(mg, dCj), 1083 - eg - ed - J.kD));
         if (SITE) red_add64(aj + 4, Shift(sE - J.kE)(e));
-        // force in units 2^-sF, and i's virial from it in units 2^-(sF + sh - 14)
+        // force in units 2^-(sF + u), and i's virial from it in units 2^-(sF + sh - 64 + 2 u), u that of the positions
         const long long fC = __mul64hi(mf, C6) << 2;
         const long long ux = __mul64hi(fC, dx), uy = __mul64hi(fC, dy), uz = __mul64hi(fC, dz);
-        const int sF = 1070 + sh - ef - ec;
-        const Shift fj(sF - J.kF), fi(sF - K.kF), vi(sF + sh - 14 - K.kV);
+        const int sF = 1020 + sh - ef - ec;
+        const Shift fj(sF - J.kF), fi(sF - K.kF), vi(sF + sh - 64 - K.kV);
         red_add64(aj + 0, -fj(ux));
         red_add64(aj + 1, -fj(uy));
         red_add64(aj + 2, -fj(uz));
@@ -244,7 +243,10 @@ __global__ void __launch_bounds__(128, 4) k_disp_cl64(Work w, Consts c, const db
 __global__ void __launch_bounds__(256) k_disp_fin64(Work w) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= w.Nr) return;
-    const Units K(w.ks[p]);
+    Units K(w.ks[p]);
+    const int iu = ipos_unit(w, w.sid[p]);
+    K.kF += iu;
+    K.kV += 2 * iu;
     const long long* a = reinterpret_cast<const long long*>(w.acc) + 16 * p;
     auto value = [](long long v, int k) { return ldexp((double)v, -k); };
     ((dbl4*)w.Fd)[p] = dbl4_make(value(a[0], K.kF), value(a[1], K.kF), value(a[2], K.kF), 0.0);

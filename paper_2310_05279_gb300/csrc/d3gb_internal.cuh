@@ -73,6 +73,7 @@ struct StructGeo {
     int64_t list_base_disp, list_base_cn;
     int64_t clu_base;     // first cluster of the structure
     int64_t list_base_cl;  // first entry of the structure's cluster-list rows
+    float ipad;            // how far an image (or, with list reuse, a moved atom) may lie beyond the atoms, bohr
 };
 
 // Cells are numbered in serpentine order within a structure: planes along z,
@@ -170,10 +171,13 @@ struct Work {
     unsigned long long* acc; // fixed-point sums of the dispersion pass: mixed [Nr][8] F (3), dE/dn, site energy;
                              // FP64 [Nr][16] F (3), dE/dn, energy, virial (6), in the atom's own units (ks)
     // FP64 form over cluster lists (d3gb_cluster64.cu): 64-bit integers scaled by powers of two
-    long long* ipos;         // [Nr + ghost_cap][4] x, y, z in units of 2^-50 bohr, type | (source << 4)
+    long long* ipos;         // [Nr + ghost_cap][4] x, y, z in units of 2^-u bohr (ipos_unit), type | (source << 4)
+    int* ixmax;              // [B] float bits: the largest |coordinate| of each structure's atoms, bohr
+    int iucap;               // the finest unit of ipos that pair vectors within the cutoffs allow (u)
     long long* row64;        // [Nr][T][row64_len(R)] rows v^(t), dv^(t) and their exponents
     long long* i64;          // [Nr][row64_len(R)] W, dW/dn and its exponent
-    int2* ks;                // [Nr] units of the atom's sums, 2^-k: k of force, dE/dn (x) and energy, virial (y), 16 bits each
+    int2* ks;                // [Nr] units of the atom's sums, 2^-k: k of force, dE/dn (x) and energy, virial (y), 16 bits
+                             // each, with k of force and virial less u and 2 u of ipos
     int* tmask;              // [B] the elements of each structure, one bit each
     double* gcnd;            // FP64 form: per CN-list entry, the chain coefficient f'(r)/r (as gcn)
     float* gcn;              // mixed form: per CN-list entry, the chain coefficient f'(r)/r of Eq. 4
@@ -302,6 +306,16 @@ __host__ __device__ inline void unpack_shift(int s, int& a, int& b, int& c) {
     a = (s & 255) - 128;
     b = ((s >> 8) & 255) - 128;
     c = ((s >> 16) & 255) - 128;
+}
+
+// FP64 form over cluster lists: positions are 64-bit integers in units of 2^-u bohr, the finest in
+// which the structure's coordinates and its images' stay below 2^62 (and pair vectors within the
+// cutoffs, Work::iucap): 2^-54 up to 256 bohr, exact where |x| is at least 0.5 bohr.  (One unit of
+// 2^-50 for every structure doubled the errors of molecules at the origin: 40 of them, 2.6e-15 of
+// an atom's terms rms for FP64 positions, 5.4e-15 for 2^-50.)
+__device__ __forceinline__ int ipos_unit(const Work& w, int s) {
+    const float x = 1.01f * __int_as_float(w.ixmax[s]) + w.geo[s].ipad;
+    return min(w.iucap, 62 - ((__float_as_int(x) >> 23) - 126));  // x < 2^(exponent field - 126)
 }
 
 // Structure of input atom i (binary search over offsets).

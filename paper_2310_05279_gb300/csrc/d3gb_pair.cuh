@@ -89,12 +89,12 @@ __device__ __forceinline__ double exp64_int(long long X, const double* __restric
                                             ((m >> 10) & 1)));  // (the leading bit adds one to the exponent)
 }
 
-// |d|^2 for integer pair vectors in units of 2^-50 bohr (Work::ipos), from the vector normalised
+// |d|^2 for integer pair vectors in units of 2^-u bohr (Work::ipos), from the vector normalised
 // by its largest component: relative error a few 2^-58 before its rounding to FP64
 // (m: its mantissa before the rounding, leading bit 63; 0 for a zero vector).  d is left
-// normalised, in units of 2^-(50 + sh) bohr: its largest component lies in
+// normalised, in units of 2^-(u + sh) bohr: its largest component lies in
 // [2^62, 2^63].
-__device__ __forceinline__ double ipos_r2(long long& dx, long long& dy, long long& dz, int& sh, unsigned long long& m) {
+__device__ __forceinline__ double ipos_r2(long long& dx, long long& dy, long long& dz, int u, int& sh, unsigned long long& m) {
     const unsigned long long o = (unsigned long long)((dx ^ (dx >> 63)) | (dy ^ (dy >> 63)) | (dz ^ (dz >> 63)));
     sh = __clzll((long long)o) - 1;
     dx <<= sh;
@@ -105,7 +105,7 @@ __device__ __forceinline__ double ipos_r2(long long& dx, long long& dy, long lon
     const int lz = __clzll((long long)r2u);
     const unsigned long long mant = r2u << lz;
     m = mant;
-    const unsigned long long bits = ((unsigned long long)(unsigned)(1049 - 2 * sh - lz) << 52) + (mant >> 11) +
+    const unsigned long long bits = ((unsigned long long)(unsigned)(1149 - 2 * (u + sh) - lz) << 52) + (mant >> 11) +
                                     ((mant >> 10) & 1);  // (the leading bit adds one to the exponent)
     return r2u ? __longlong_as_double((long long)bits) : 0.0;
 }

@@ -159,6 +159,7 @@ __device__ __forceinline__ void store_weights(const Work& w, const Consts& c, co
                 q[R + a] = fix_value(dWr[a], ew, 61);
             }
             q[2 * R] = ew;
+            q[2 * R + 1] = ipos_unit(w, w.sid[p]);
         }
     }
     if (u0 != 0) return;
@@ -254,7 +255,8 @@ struct SumBound {
     // overflows, and 58 (force, energy) and 56 (virial) to that of a term, which k_disp_cl64's
     // mantissas have at least.  A unit then lies below an FP64 rounding of the sum of the terms' sizes,
     // whatever the damping, the other elements of the table and the other atoms of the structure.
-    __device__ __forceinline__ int2 units(const RowBound& rb, int nfar) const {
+    // iu: the unit of the positions.
+    __device__ __forceinline__ int2 units(const RowBound& rb, int nfar, int iu) const {
         const float n = (float)nfar;
         auto above = [](float x) { return (__float_as_int(1.05f * x) >> 23) - 126; };  // x < 2^above(x)
         auto k = [&](int bits, float sum, float term, float beyond) {
@@ -262,7 +264,8 @@ struct SumBound {
             return max(-900, min(900, min(a, b)));
         };
         const int kD = max(-900, min(900, 62 - above(fmaf(n, rb.g, g)) - rb.ed));
-        return make_int2((k(58, f, f1, rb.f) & 0xffff) | (kD << 16), (k(58, e, e1, rb.e) & 0xffff) | (k(56, v, v1, rb.v) << 16));
+        return make_int2(((k(58, f, f1, rb.f) - iu) & 0xffff) | (kD << 16),
+                         (k(58, e, e1, rb.e) & 0xffff) | ((k(56, v, v1, rb.v) - 2 * iu) << 16));
     }
 };
 
@@ -410,7 +413,7 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
         // kept for the chain pass. The FP64 pipe bounds the pass (80 issue slots an instruction),
         // so where positions stand as integers too, the pair vector, r^2 and the exponential are
         // formed from them: 16 FP64 instructions a pair instead of 33, 9.4 M entries 0.77 -> 0.46 ms
-        // (0.91 with the library's exp, square root and divisions; 0.47 with the bounds of SumBound).
+        // (0.91 with the library's exp, square root and divisions; 0.45 with the bounds of SumBound).
         const int t = S.tsrc() & 15;
         const double* krow = k1rc + t * c.T;
         const float4* brow = bound + t * c.T;
@@ -418,6 +421,7 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
         double* grow = w.gcnd + (LV.p - w.nbr_cn);
         const bool ints = w.ipos != nullptr;
         longlong2 xa = make_longlong2(0, 0), xb = xa;
+        const int iu = ints ? ipos_unit(w, s) : 0;
         if (ints) {
             xa = reinterpret_cast<const longlong2*>(w.ipos + 4 * p)[0];
             xb = reinterpret_cast<const longlong2*>(w.ipos + 4 * p)[1];
@@ -435,7 +439,7 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
                 const longlong2 ya = __ldg(x2), yb = __ldg(x2 + 1);
                 long long nx = ya.x - xa.x, ny = ya.y - xa.y, nz = yb.x - xb.x;
                 int sh;
-                r2 = ipos_r2(nx, ny, nz, sh, mant);
+                r2 = ipos_r2(nx, ny, nz, iu, sh, mant);
                 tq = (int)yb.y;
                 const long long d = __double_as_longlong(r2) - rcb;  // (positive doubles order as their bits)
                 if (d > 64) return 0.0;
@@ -475,7 +479,7 @@ __global__ void __launch_bounds__(128) k_cn(Work w, Consts c, const float4* __re
         w.cn[p] = (double)nh;
         RowBound rb;
         weights_atom<MIXED, R>(w, c, cnref, nref, c6, p, t, (double)nh, bound, &rb);
-        if (ints) w.ks[p] = sb.units(rb, w.maxcnt[3 * s]);
+        if (ints) w.ks[p] = sb.units(rb, w.maxcnt[3 * s], iu);
     }
 }
 

@@ -105,3 +105,48 @@ def test_molecules_and_dense_clouds(d3_class, damp, rc):
             for k, sl in (("F", i), ("E", s), ("W", s)) + ((("e_atom", i),) if sites else ()):
                 x, y = out[k][sl], full[k][sl]
                 assert np.abs(x - y).max() <= TOL_SUM * np.abs(y).max(), (k, s)
+
+
+def test_positions_near_the_origin(d3_class, oracle_mod):
+    """Pairs 0.2 A apart about the origin, hardly damped, so that energies go as d^-8: integer positions keep
+    what FP64 holds of small coordinates.  With positions to 2^-55 bohr (d = 0.38 bohr) 8 2^-54 / 0.38 =
+    1.2e-15, some 30 operations a side 6.7e-15."""
+    g = np.random.Generator(np.random.PCG64(13))
+    t = wl.carbon_table()
+    structs = []
+    for _ in range(200):
+        u = g.normal(size=3)
+        u *= 0.1 / np.linalg.norm(u)
+        structs.append(_open(np.array([-u, u]), [0, 0]))
+    b = wl.batch_of(structs, t)
+    prm = dict(wl.PBE_BJ, a1=0.0, a2=0.003)
+    ref = oracle_mod.compute_batch(b, prm)
+    d3 = d3_class(t, prm, precision="fp64")
+    pos, typ = to_dev(b)
+    E = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc)["E"].cpu().numpy()
+    d3.sync_status()
+    assert d3.list_stats()["list_mode"] == 1
+    assert (np.abs(E - ref["E"]) <= 8e-15 * np.abs(ref["E"])).all()
+
+
+@pytest.mark.parametrize("shift", [0.0, 150.0, 600.0, 3000.0])
+def test_positions_far_from_the_origin(d3_class, shift):
+    """Coordinates on both sides of the lines where the unit of the positions changes, up to the largest
+    ones taken: the same positions through the per-atom lists."""
+    g = np.random.Generator(np.random.PCG64(14))
+    t = wl.random_tables(wl.UNEVEN_ELEMENTS, 1003)
+    structs = [(_cloud(g, 20, 3.0, 1.0) + s * shift, g.integers(0, 6, 20).astype(np.int32), np.eye(3) * 30.0,
+                np.zeros(3, np.int32)) for s in (np.ones(3), np.array([-1.0, 0.0, 0.5]))]
+    structs.append(wl.random_structure(g, 60, wl.UNEVEN_ELEMENTS))
+    b = wl.batch_of(structs, t)
+    d3 = d3_class(t, precision="fp64")
+    pos, typ = to_dev(b)
+    full = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc, w_atom=True)
+    out = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc)
+    d3.sync_status()
+    assert d3.list_stats()["list_mode"] == 1
+    for s in range(b.nstruct):
+        i = slice(b.offsets[s], b.offsets[s + 1])
+        for k, sl in (("F", i), ("E", s), ("W", s)):
+            x, y = out[k][sl].cpu().numpy(), full[k][sl].cpu().numpy()
+            assert np.abs(x - y).max() <= TOL_SUM * np.abs(y).max(), (k, s)
