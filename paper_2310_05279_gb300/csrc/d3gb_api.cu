@@ -210,6 +210,8 @@ struct d3_handle {
     Plan plan;
     // staging buffers of the host-memory entry point
     Pinned pin;  // plan upload and sizing read-back
+    cudaEvent_t pin_copied = nullptr;  // recorded after the copies of the last upload
+    bool pin_busy = false;             // they have not been waited for
     DevBuf stage;
     size_t stage_atoms = 0, stage_structs = 0;
     double *s_pos = nullptr, *s_E = nullptr, *s_F = nullptr, *s_W = nullptr;
@@ -512,6 +514,7 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
         const cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return cuda_fail(h, e, "synchronize before a new layout");
     }
+    P.stream = st;
     const int B = P.B;
     const int64_t Nr = P.Nr, C = P.ncells, Ng = P.ghost_cap, Nt = Nr + Ng;
     int64_t ld = 0, lc = 0, lcl = 0, ncl = 0, nfin = 0, maxn = 0;
@@ -685,17 +688,32 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     int* gate = w.gate;
     w.gate = nullptr;  // the plan's own Work builds unconditionally; enqueue_build gates a copy
     P.gate = gate;
-    // geometry and offsets through page-locked memory (free again: the sizing pass that follows
-    // every upload waits for the stream); the per-atom and per-cluster indices are formed on the device
+    // geometry and offsets through page-locked memory, once the copies of the last upload are over
+    // (a batch without atoms has no sizing pass that waits for them); the per-atom and per-cluster
+    // indices are formed on the device
     const size_t ngeo = sizeof(StructGeo) * (size_t)B, noff = sizeof(int64_t) * ((size_t)B + 1);
-    e = h->pin.reserve(ngeo + noff + sizeof(int) * (3 * (size_t)B + 2));
-    if (e != cudaSuccess) return cuda_fail(h, e, "page-locked staging");
+    if (h->pin_busy) e = cudaEventSynchronize(h->pin_copied);
+    h->pin_busy = false;
+    if (e == cudaSuccess && !h->pin_copied) e = cudaEventCreateWithFlags(&h->pin_copied, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = h->pin.reserve(ngeo + noff + sizeof(int) * (3 * (size_t)B + 2));
+    if (e != cudaSuccess) {
+        P.valid = false;
+        return cuda_fail(h, e, "page-locked staging");
+    }
     std::memcpy(h->pin.p, P.geo.data(), ngeo);
     std::memcpy(h->pin.p + ngeo, P.offsets.data(), noff);
     e = cudaMemcpyAsync(dgeo, h->pin.p, ngeo, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(doff, h->pin.p + ngeo, noff, cudaMemcpyHostToDevice, st);
+    h->pin_busy = true;
+    if (cudaEventRecord(h->pin_copied, st) != cudaSuccess) {
+        cudaStreamSynchronize(st);
+        h->pin_busy = false;
+    }
     if (e == cudaSuccess) e = launch_plan_ids(dgeo, doff, B, Nr, ncl, nfin, dsid, dclu, dfin, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "geometry upload");
+    if (e != cudaSuccess) {
+        P.valid = false;
+        return cuda_fail(h, e, "geometry upload");
+    }
     return D3_OK;
 }
 
@@ -1264,6 +1282,7 @@ void d3_destroy(d3_handle* h) {
     h->plan.mem.release();
     h->plan.bwd.release();
     h->pin.release();
+    if (h->pin_copied) cudaEventDestroy(h->pin_copied);
     h->stage.release();
     h->tabmem.release();
     if (h->h_status) cudaFreeHost(h->h_status);

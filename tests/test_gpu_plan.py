@@ -1,0 +1,50 @@
+"""New geometries on one handle while earlier work is still running: calls that don't wait for the
+stream must not lose their geometry to the next call."""
+import numpy as np
+import pytest
+
+from paper_2310_05279_gb300 import workloads as wl
+
+from ._helpers import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    return torch
+
+
+def _empty(n):
+    s = (np.zeros((0, 3)), np.zeros(0, np.int32), np.eye(3) * 9.0, np.ones(3, np.int32))
+    return wl.batch_of([s] * n, wl.random_tables(wl.UNEVEN_ELEMENTS, 1003))
+
+
+@pytest.mark.parametrize("other_stream", [False, True])
+def test_empty_structures_before_the_next_geometry(torch_cuda, other_stream):
+    """Structures without atoms take no sizing pass, so the call returns while its upload waits behind
+    other work: their sums stay zero whatever geometry comes next."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3
+    a, c = wl.uneven_batch(seed=21, nstruct=6, n_range=(50, 300)), wl.uneven_batch(seed=22, nstruct=6, n_range=(40, 200))
+    e = _empty(6)
+    d3 = D3(a.tables)
+    pa, ta = to_dev(a)
+    pc, tc = to_dev(c)
+    pe, te = to_dev(e)
+    want = {k: v.clone() for k, v in D3(c.tables).compute_batch(pc, tc, c.offsets, c.cells, c.pbc).items()}
+    d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc)  # the workspace has room for all three
+    torch.cuda.synchronize()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(200_000_000)  # about 0.1 s
+        empty = d3.compute_batch(pe, te, e.offsets, e.cells, e.pbc)
+    with torch.cuda.stream(s2 if other_stream else s1):
+        got = d3.compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    torch.cuda.synchronize()
+    assert (empty["E"] == 0).all() and (empty["W"] == 0).all()
+    for k in want:
+        assert torch.equal(got[k], want[k]), k
