@@ -936,6 +936,15 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     Plan& P = h->plan;
     *built = false;
     if (same_geometry(P, B, offsets, cells, pbc) && P.sized[mode]) return D3_OK;
+    {  // refused before anything of the plan changes: a captured upload would not run
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+        if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return cuda_fail(h, e != cudaSuccess ? e : cudaErrorStreamCaptureUnsupported,
+                             "a new geometry cannot be sized while its stream is being captured: call once before");
+        }
+    }
     if (!same_geometry(P, B, offsets, cells, pbc)) {
         P.valid = false;
         P.sized[0] = P.sized[1] = false;

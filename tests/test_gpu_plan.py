@@ -48,3 +48,35 @@ def test_empty_structures_before_the_next_geometry(torch_cuda, other_stream):
     assert (empty["E"] == 0).all() and (empty["W"] == 0).all()
     for k in want:
         assert torch.equal(got[k], want[k]), k
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_new_geometry_refused_under_capture(torch_cuda, precision):
+    """A geometry that has not been sized is refused under capture, and the plan stays as it was: the same
+    geometry outside the capture, and the earlier one, give their results."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3, D3Error
+    a, c = wl.uneven_batch(seed=23, nstruct=5, n_range=(200, 400)), wl.uneven_batch(seed=24, nstruct=5, n_range=(40, 100))
+    pa, ta = to_dev(a)
+    pc, tc = to_dev(c)
+    d3 = D3(a.tables, precision=precision)
+    first = {k: v.clone() for k, v in d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc).items()}
+    want = D3(c.tables, precision=precision).compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    torch.cuda.synchronize()
+    for x, px, tx in ((c, pc, tc), (_empty(5), pc[:0], tc[:0])):
+        out = dict(E=torch.zeros(5, dtype=torch.float64, device="cuda"), F=torch.zeros_like(px),
+                   W=torch.zeros((5, 3, 3), dtype=torch.float64, device="cuda"))
+        refused = False
+        with torch.cuda.graph(torch.cuda.CUDAGraph()):
+            out["E"].add_(1.0)  # (something to capture)
+            try:
+                d3.compute_batch(px, tx, x.offsets, x.cells, x.pbc, out=out)
+            except D3Error:
+                refused = True
+        assert refused
+    got = d3.compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    again = d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc)
+    d3.sync_status()
+    for k in want:
+        assert torch.equal(got[k], want[k]), k
+        assert torch.equal(again[k], first[k]), k
