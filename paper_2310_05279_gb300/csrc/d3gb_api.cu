@@ -55,7 +55,6 @@ constexpr int kEvents = kStages + 3;  // kStages + 1 stage boundaries, 2 around 
 constexpr int32_t kDefaultShape[4] = {64, 128, 128, 16};
 constexpr int32_t kBlockCand[2] = {64, 128};
 constexpr int32_t kBuildCand[2] = {8, 16};
-constexpr int64_t kStructCells = 12000;  // cells that a block counts in shared memory (two blocks per SM)
 constexpr double kStructItems = 4500.0;  // build_by_struct
 constexpr int64_t kTuneMinAtoms = 16384;  // below this launch overhead decides, not the shape
 constexpr int kTuneReps = 3;

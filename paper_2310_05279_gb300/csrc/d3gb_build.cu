@@ -1197,8 +1197,11 @@ cudaError_t launch_build_impl(const Work& w, const double* pos, const int32_t* t
     if (w.by_struct) {
         const size_t sm = 2 * sizeof(int) * ((size_t)w.max_ncell + 1);
         const bool wide = w.B <= w.num_sms;  // a structure to itself on an SM takes twice the threads
+        // (the most that any plan needs: the limit belongs to the function, and a smaller one could be set
+        // by another handle's thread between here and the launch)
         const cudaError_t e = cudaFuncSetAttribute(wide ? k_build_struct<1024> : k_build_struct<512>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(2 * sizeof(int) * (kStructCells + 1)));
         if (e != cudaSuccess) return e;
         k_reset_struct<<<1, 1, 0, st>>>(w);
         if (wide) k_build_struct<1024><<<(unsigned)w.B, 1024, sm, st>>>(w, pos, types, rk_tab);

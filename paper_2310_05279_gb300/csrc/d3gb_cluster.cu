@@ -130,6 +130,10 @@ __device__ __forceinline__ void load_j(const Work& w, const float* __restrict__ 
 constexpr int kChunkSteps = 16;
 constexpr int kSplitForce = kChunkSteps * 3 * 32;
 constexpr int kSplitFloats = kSplitForce + 8 * 32;  // per warp
+constexpr int kSplitWarps = 8;                      // at most, per block
+// the most shared memory that a split pass needs: the limit belongs to the function, so it is never set
+// lower (another handle's thread could launch in between)
+constexpr int kSplitSmem = kMaxTypes * kMaxTypes * (int)sizeof(float4) + kSplitWarps * kSplitFloats * (int)sizeof(float);
 
 // The lane's i atom and its running sums.  step2() evaluates two steps (8 i atoms x
 // 4 list entries each) written as one block, so that their dependency chains
@@ -732,7 +736,7 @@ cudaError_t launch_disp_cl(const Work& w, const Consts& c, const void* pair_tab,
         const int TB = w.blk_disp;  // 64 or 128 threads: 2 or 4 clusters per block
         const unsigned grid = nblk(w.ncl, TB / 32);
         const size_t sm = (size_t)c.T * c.T * sizeof(float4);
-        const int nw = w.ncl <= w.num_sms ? 8 : 4;  // fewer clusters than SMs: more warps for each
+        const int nw = w.ncl <= w.num_sms ? kSplitWarps : 4;  // fewer clusters than SMs: more warps for each
         const size_t sms = sm + (size_t)nw * kSplitFloats * sizeof(float);
         const unsigned gs = (unsigned)(w.ncl < 8 * (int64_t)w.num_sms ? w.ncl : 8 * (int64_t)w.num_sms);
         const float4* pt = (const float4*)pair_tab;
@@ -740,7 +744,7 @@ cudaError_t launch_disp_cl(const Work& w, const Consts& c, const void* pair_tab,
 #define D3_CL1(RR, S, I)                                                                                   \
     {                                                                                                      \
         if (w.split_on) {                                                                                  \
-            e = cudaFuncSetAttribute(k_disp_cl_split<RR, S, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms); \
+            e = cudaFuncSetAttribute(k_disp_cl_split<RR, S, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem); \
             if (e != cudaSuccess) return e;                                                                \
             k_disp_cl_split<RR, S, I><<<gs, 32 * nw, sms, st>>>(w, c, pt);                                 \
             e = launch_overlapped(k_disp_cl<RR, S, I, true>, grid, TB, sm, st, w, c, pt);                         \

@@ -33,6 +33,7 @@ constexpr double kHartreeEV = 27.211386245988;  // eV per Hartree
 constexpr int kMaxTypes = 16;
 constexpr int kMaxRef = 7;
 constexpr int kChunk = 64;  // pairs summed in FP32 before an FP64 accumulate (mixed form)
+constexpr int64_t kStructCells = 12000;  // cells that a block counts in shared memory (k_build_struct; two blocks per SM)
 constexpr int kFinChunk = 2048;  // atoms per first-level block of the per-structure sums
 
 enum StatusBits : int {
