@@ -198,6 +198,7 @@ struct d3_handle {
     double* d_k1rc = nullptr;    // k1 k2 (Rcov_i + Rcov_j)
     double* d_exptab64 = nullptr;  // 2^(j/64), j = 0..63
     float4* d_bound = nullptr;   // FP64 form: bounds of a pair's terms (Tabs::bound)
+    bool tables_ok = false;      // the device tables hold the damping parameters of prm
     // FP64 form over cluster lists: whether the bounds can be formed, and their constants (Consts)
     bool fx_ok = false;
     float fx_s6 = 0.0f, fx_r2min = 0.0f;
@@ -313,6 +314,7 @@ void fixed_point_bounds(d3_handle* h, std::vector<float4>& tab) {
 // Upload the damping table (R^6, R^8, s6, s8 R0^2 per element pair) in both precisions.
 d3_status upload_pair_table(d3_handle* h) {
     const int T = h->T;
+    h->tables_ok = false;
     std::vector<float4> bnd;
     fixed_point_bounds(h, bnd);
     std::vector<dbl4> pd(T * T), pb(T * T);
@@ -337,6 +339,7 @@ d3_status upload_pair_table(d3_handle* h) {
     if (e == cudaSuccess) e = cudaMemcpy(h->d_pairb, pb.data(), pb.size() * sizeof(dbl4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_bound, bnd.data(), bnd.size() * sizeof(float4), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(h, e, "pair table upload");
+    h->tables_ok = true;
     return D3_OK;
 }
 
@@ -1301,7 +1304,9 @@ d3_status d3_set_damping(d3_handle* h, double s6, double s8, double a1, double a
     if (!h) return D3_ERR_ARG;
     if (!std::isfinite(s6) || !std::isfinite(s8) || !std::isfinite(a1) || !std::isfinite(a2_bohr))
         return fail(h, D3_ERR_ARG, "non-finite damping parameter");
-    if (s6 == h->prm.s6 && s8 == h->prm.s8 && a1 == h->prm.a1 && a2_bohr == h->prm.a2_bohr) return D3_OK;
+    // (nothing to do when the tables hold these values: the backward of a fit step sets its forward's again)
+    if (h->tables_ok && s6 == h->prm.s6 && s8 == h->prm.s8 && a1 == h->prm.a1 && a2_bohr == h->prm.a2_bohr)
+        return D3_OK;
     if (h->last_stream) cudaStreamSynchronize(h->last_stream);
     h->prm.s6 = s6;
     h->prm.s8 = s8;
