@@ -29,7 +29,9 @@
  *    geometry of a size class, measures the launch shapes: d3_set_autotune);
  *    later calls with the same
  *    geometry allocate nothing and do not synchronise, so they can be captured
- *    in a CUDA graph.
+ *    in a CUDA graph.  Such a graph refers to the handle's workspace: it may be
+ *    replayed until the handle takes a call with another geometry, which waits
+ *    for replays that are running, or is destroyed.
  *  - Errors: every call returns a d3_status.  Device-side problems (capacity
  *    overflow, non-finite coordinates, bad types, coordinates out of range) are
  *    recorded in a status word that d3_sync_status() reads.  The library never

@@ -148,6 +148,8 @@ struct Plan {
     int ghost_cap = 0;
     Arena mem, bwd;  // the plan's buffers; the backward's scratch
     cudaStream_t stream = nullptr;  // of the last work enqueued on them
+    bool captured = false;          // a caller's graph holds work on them: it may run on any stream
+    bool unknown = false;           // the last build enqueued went into a caller's graph: it may not have run
     Work w{};
     int* bsum = nullptr;  // scan scratch
     int* gate = nullptr;  // list-reuse gate (device int)
@@ -507,16 +509,24 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
     return D3_OK;
 }
 
+// Whether work on st is being captured, or would end the capture of a stream that st waits for.
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Lay out every device buffer of the plan for the current capacities and upload
 // its geometry on st.
 d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     ++h->plan_gen;  // a captured graph refers to the old layout
-    // work of earlier calls may still use the memory: calls on st are ordered, another stream's are waited for
-    if (P.mem.base && P.stream != st) {
-        const cudaError_t e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) return cuda_fail(h, e, "synchronize before a new layout");
-    }
+    // Work of earlier calls may still use the memory.  What runs on st is ordered before this; what runs on
+    // another stream, as a caller's graph may, is waited for by giving the memory back (cudaFree waits for
+    // the device; cudaDeviceSynchronize would fail, and end the capture, while another thread captures)
+    if (P.stream != st || P.captured) P.mem.release();
     P.stream = st;
+    P.captured = P.unknown = false;
     const int B = P.B;
     const int64_t Nr = P.Nr, C = P.ncells, Ng = P.ghost_cap, Nt = Nr + Ng;
     int64_t ld = 0, lc = 0, lcl = 0, ncl = 0, nfin = 0, maxn = 0;
@@ -789,9 +799,10 @@ d3_status enqueue_build(d3_handle* h, Plan& P, const double* pos, const int32_t*
                         bool gated = false, cudaEvent_t* lmarks = nullptr) {
     // a build in the other list mode re-sorted the atoms: the first build in
     // this mode must run whatever the displacement check would decide
-    if (P.last_mode != mode) gated = false;
+    if (P.last_mode != mode || P.unknown) gated = false;
     set_mode(P, mode);
     P.last_mode = mode;
+    P.unknown = false;
     P.stream = st;
     Work w = P.w;
     cudaError_t e = cudaSuccess;
@@ -938,15 +949,9 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     Plan& P = h->plan;
     *built = false;
     if (same_geometry(P, B, offsets, cells, pbc) && P.sized[mode]) return D3_OK;
-    {  // refused before anything of the plan changes: a captured upload would not run
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
-        if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return cuda_fail(h, e != cudaSuccess ? e : cudaErrorStreamCaptureUnsupported,
-                             "a new geometry cannot be sized while its stream is being captured: call once before");
-        }
-    }
+    if (capturing(st))  // refused before anything of the plan changes: a captured upload would not run
+        return cuda_fail(h, cudaErrorStreamCaptureUnsupported,
+                         "a new geometry cannot be sized while its stream is being captured: call once before");
     if (!same_geometry(P, B, offsets, cells, pbc)) {
         P.valid = false;
         P.sized[0] = P.sized[1] = false;
@@ -1104,10 +1109,12 @@ d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const d
     s = ensure_plan(h, B, offsets, pos, types, cells, pbc, st, mode, &built);
     if (s != D3_OK) return s;
     auto direct = [&]() { return enqueue_forward(h, pos, types, E, F, W, e_atom, cn, st, w_atom, mode, built); };
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (!h->graphs || h->prof_on || offsets[B] <= 0 || cudaStreamIsCapturing(st, &cs) != cudaSuccess ||
-        cs != cudaStreamCaptureStatusNone)
-        return direct();
+    const bool caller_captures = capturing(st);
+    if (!h->graphs || h->prof_on || offsets[B] <= 0 || caller_captures) {
+        s = direct();
+        if (caller_captures) h->plan.captured = h->plan.unknown = true;
+        return s;
+    }
     const void* key[10] = {pos, types, E, F, W, e_atom, cn, w_atom, (const void*)(intptr_t)h->plan_gen,
                            (const void*)(intptr_t)(h->param_gen * 2 + (h->accumulate ? 1 : 0))};
     const bool again = same_key(key, h->lkey);  // as in the previous call
@@ -1115,7 +1122,7 @@ d3_status forward_graph(d3_handle* h, int32_t B, const int64_t* offsets, const d
     // (the last build was in the other list mode: rebuild once directly, a
     // replayed graph would take the list-reuse decision on stale lists)
     const bool captured_before = h->gexec && same_key(key, h->gkey);
-    if (built || h->plan.last_mode != mode || !(captured_before || again)) return direct();
+    if (built || h->plan.last_mode != mode || h->plan.unknown || !(captured_before || again)) return direct();
     if (!captured_before) {
         if (!h->cap_stream && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
             h->graphs = false;
@@ -1514,6 +1521,7 @@ d3_status d3_backward(d3_handle* h, int32_t B, const int64_t* offsets, const dou
     cudaError_t e = launch_backward(P.w, c, h->d_c6d, h->d_pairb, h->d_cnref, h->d_nref, tbm, dLdE, dLdF, dLdparams,
                                     dLdpos, reinterpret_cast<double*>(P.bwd.base), P.list_cn, B, mixed, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "backward launch");
+    if (capturing(st)) P.captured = P.unknown = true;
     return D3_OK;
 }
 

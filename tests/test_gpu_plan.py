@@ -1,5 +1,7 @@
 """New geometries on one handle while earlier work is still running: calls that don't wait for the
 stream must not lose their geometry to the next call."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -80,3 +82,91 @@ def test_new_geometry_refused_under_capture(torch_cuda, precision):
     for k in want:
         assert torch.equal(got[k], want[k]), k
         assert torch.equal(again[k], first[k]), k
+
+
+def test_new_geometry_on_another_stream_while_a_thread_captures(torch_cuda):
+    """The workspace changes streams with a new geometry while another stream is being captured: the call
+    succeeds and the capture goes on."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3
+    a, c = wl.uneven_batch(seed=26, nstruct=4, n_range=(100, 200)), wl.uneven_batch(seed=27, nstruct=4, n_range=(40, 90))
+    pa, ta = to_dev(a)
+    pc, tc = to_dev(c)
+    want = D3(c.tables).compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    d3 = D3(a.tables)
+    d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc)
+    torch.cuda.synchronize()
+    x, s, got = torch.zeros(8, device="cuda"), torch.cuda.Stream(), {}
+    out = {k: torch.empty_like(v) for k, v in want.items()}
+
+    def other():
+        with torch.cuda.stream(s):
+            try:
+                d3.compute_batch(pc, tc, c.offsets, c.cells, c.pbc, out=out)
+                s.synchronize()
+                got["ok"] = True
+            except Exception as e:  # noqa: BLE001
+                got["error"] = str(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        x.add_(1.0)
+        t = threading.Thread(target=other)
+        t.start()
+        t.join()
+        x.add_(1.0)
+    assert got == {"ok": True}
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (x == 2.0).all()
+    for k in want:
+        assert torch.equal(out[k], want[k]), k
+
+
+def test_new_geometry_waits_for_a_callers_graph(torch_cuda):
+    """A caller's graph that runs on a stream the handle has not seen keeps its workspace until it is done."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3
+    a, c = wl.uneven_batch(seed=28, nstruct=6, n_range=(200, 400)), wl.uneven_batch(seed=29, nstruct=6, n_range=(100, 300))
+    pa, ta = to_dev(a)
+    pc, tc = to_dev(c)
+    d3 = D3(a.tables)
+    first = {k: v.clone() for k, v in d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc).items()}
+    want = D3(c.tables).compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    out = {k: torch.zeros_like(v) for k, v in first.items()}
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc, out=out)
+    d3.compute_batch(pa, ta, a.offsets, a.cells, a.pbc)  # the handle's last stream is the current one again
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(100_000_000)
+        graph.replay()
+    got = d3.compute_batch(pc, tc, c.offsets, c.cells, c.pbc)
+    torch.cuda.synchronize()
+    for k in first:
+        assert torch.equal(out[k], first[k]), k
+        assert torch.equal(got[k], want[k]), k
+
+
+def test_skin_after_a_captured_call_of_the_other_lists(torch_cuda):
+    """With a skin, a captured build counts as not run: the next ordinary call builds its own lists."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3
+    b = wl.uneven_batch(seed=30, nstruct=4, n_range=(60, 200))
+    pos, typ = to_dev(b)
+    d3 = D3(b.tables, skin=0.5)
+    want = {k: v.clone() for k, v in d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc).items()}
+    wa = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc, w_atom=True)  # the lists are per atom now
+    out = {k: torch.empty_like(v) for k, v in want.items()}
+    torch.cuda.synchronize()
+    n0 = d3.build_count()
+    with torch.cuda.graph(torch.cuda.CUDAGraph()):
+        d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc, out=out)
+    got = d3.compute_batch(pos, typ, b.offsets, b.cells, b.pbc)
+    d3.sync_status()
+    assert d3.build_count() == n0 + 1
+    for k in want:
+        assert torch.equal(got[k], want[k]), k
+    assert wa["w_atom"].isfinite().all()
