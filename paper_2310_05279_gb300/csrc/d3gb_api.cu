@@ -126,6 +126,17 @@ struct Pinned {
     }
 };
 
+// The largest of the last 16 ratios (at least 1, at most 8): one odd structure is forgotten after 16 geometries.
+struct CapRatio {
+    double last[16] = {};
+    int next = 0;
+    void add(double r) {
+        last[next] = r;
+        next = (next + 1) % 16;
+    }
+    double value() const { return std::min(8.0, std::max(1.0, *std::max_element(last, last + 16))); }
+};
+
 // List layout of a build: the forward takes its dispersion pairs from cluster
 // half lists (per-atom lists only within R_cn); the per-atom virial of Eq. 7, the
 // backward, and the FP64 form with parameters outside its fixed-point bounds use
@@ -235,8 +246,8 @@ struct d3_handle {
     const void* gkey[10] = {};     // pointers and generations the graph was captured with
     int64_t plan_gen = 0, param_gen = 0;
     const void* lkey[10] = {};       // key of the previous call
-    // list capacities the sizing passes settled on, over plan_geometry's estimates (largest ratio seen)
-    double cap_ratio_cn = 1.0, cap_ratio_cl = 1.0;
+    // list capacities that the last geometries needed, over plan_geometry's estimates
+    CapRatio cap_ratio_cn, cap_ratio_cl;
     // launch shapes (d3_launch_shapes): chosen per size class by the autotuner unless fixed
     int32_t shape[4] = {kDefaultShape[0], kDefaultShape[1], kDefaultShape[2], kDefaultShape[3]};
     bool autotune = true;
@@ -409,7 +420,7 @@ d3_status plan_geometry(d3_handle* h, Plan& P, int32_t B, const int64_t* offsets
     // structures streamed through one handle are alike: start from the ratios of the earlier ones, so
     // that the sizing pass rarely has to regrow and build again (up to a size where memory matters)
     const bool learn = offsets[B] <= ((int64_t)1 << 18);
-    const double ratio_cn = learn ? h->cap_ratio_cn : 1.0, ratio_cl = learn ? h->cap_ratio_cl : 1.0;
+    const double ratio_cn = learn ? h->cap_ratio_cn.value() : 1.0, ratio_cl = learn ? h->cap_ratio_cl.value() : 1.0;
     int64_t cell_base = 0;
     for (int s = 0; s < B; ++s) {
         StructGeo& G = P.geo[s];
@@ -1008,6 +1019,7 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         if (status & ST_NONFINITE) return fail(h, D3_ERR_NONFINITE, "non-finite coordinate");
         if (status & ST_TYPE) return fail(h, D3_ERR_TYPE, "atom type out of range");
         bool grow = false;
+        double need_cn = 0.0, need_cl = 0.0;  // of this geometry, over the estimates
         if (gcount > P.ghost_cap) {
             P.ghost_cap = (int)std::min<double>(2.0e9, gcount * 1.1 + 64);
             grow = true;
@@ -1015,16 +1027,18 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
         for (int s2 = 0; s2 < B; ++s2) {
             StructGeo& G = P.geo[s2];
             if (mode == kFullLists && mx[3 * s2] > G.cap_disp) { G.cap_disp = round_cap(mx[3 * s2] * 1.1 + 16); grow = true; }
-            auto regrow = [&](int n, int32_t& cap, int spare, double est, double& ratio) {
+            auto regrow = [&](int n, int32_t& cap, int spare, double est, double& need) {
+                if (est > 0) need = std::max(need, n * 1.1 / est);
                 if (n <= cap) return;
                 cap = round_cap(n * 1.1 + spare);
-                if (est > 0) ratio = std::min(8.0, std::max(ratio, n * 1.1 / est));
                 grow = true;
             };
-            regrow(mx[3 * s2 + 1], G.cap_cn, 8, P.cap_est[2 * (size_t)s2], h->cap_ratio_cn);
-            regrow(mx[3 * s2 + 2], G.cap_cl, 16, P.cap_est[2 * (size_t)s2 + 1], h->cap_ratio_cl);
+            regrow(mx[3 * s2 + 1], G.cap_cn, 8, P.cap_est[2 * (size_t)s2], need_cn);
+            regrow(mx[3 * s2 + 2], G.cap_cl, 16, P.cap_est[2 * (size_t)s2 + 1], need_cl);
         }
         if (!grow) {
+            h->cap_ratio_cn.add(need_cn);
+            if (mode == kClusterLists) h->cap_ratio_cl.add(need_cl);
             // image rows of v and dv are copies of their source's when that is cheap
             // (few images, or few types); otherwise the pass resolves each image's source
             P.vd_images = (int64_t)gcount * h->T <= 2 * P.Nr ? 1 : 0;

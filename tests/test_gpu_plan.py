@@ -170,3 +170,37 @@ def test_skin_after_a_captured_call_of_the_other_lists(torch_cuda):
     for k in want:
         assert torch.equal(got[k], want[k]), k
     assert wa["w_atom"].isfinite().all()
+
+
+def test_an_odd_structure_is_forgotten(torch_cuda):
+    """The list capacities of later geometries follow the last ones, not the oddest ever seen: a dense drop in
+    a wide cell, then twenty ordinary structures, then a large box, which takes the memory it takes alone."""
+    torch = torch_cuda
+    from paper_2310_05279_gb300 import D3
+    g = np.random.Generator(np.random.PCG64(33))
+    box = wl.mof_like_box(seed=34, ncell=36)
+    drop = g.normal(size=(400, 3))
+    drop *= 5.0 * g.uniform(0.0, 1.0, (400, 1)) ** (1 / 3) / np.linalg.norm(drop, axis=1, keepdims=True)
+    odd = wl.batch_of([(drop + 60.0, g.integers(0, 5, 400).astype(np.int32), np.eye(3) * 120.0, np.ones(3, np.int32))],
+                      box.tables)
+    small = wl.mof_like_box(seed=35, ncell=8)
+
+    def used(d3):
+        free0 = torch.cuda.mem_get_info()[0]
+        pos, typ = to_dev(box)
+        d3.compute_batch(pos, typ, box.offsets, box.cells, box.pbc)
+        d3.sync_status()
+        del pos, typ
+        torch.cuda.empty_cache()
+        return free0 - torch.cuda.mem_get_info()[0]
+
+    d3 = D3(box.tables)
+    pos, typ = to_dev(odd)
+    d3.compute_batch(pos, typ, odd.offsets, odd.cells, odd.pbc)
+    pos, typ = to_dev(small)
+    for k in range(20):
+        d3.compute_batch(pos * (1 + 0.001 * k), typ, small.offsets, small.cells * (1 + 0.001 * k), small.pbc)
+    d3.sync_status()
+    after = used(d3)
+    alone = used(D3(box.tables))
+    assert after <= 1.25 * alone
