@@ -939,7 +939,8 @@ int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
 
 // Whether the mixed form's CN pass (bit 0) and chain pass (bit 1) take 8 lanes per atom.
 // For few atoms one thread per atom is a chain of 0.55 us per list entry (64 atoms: CN pass
-// 37 us and 13 with 8 lanes, chain pass 18 and 12; 6,912 atoms: 36 and 15, 20 and 15).  Beyond,
+// 37 us and 13 with 8 lanes, chain pass 18 and 12; 6,912 atoms: 36 and 15, 20 and 15), in the
+// CN pass also for 34,560 (41 and 35), 42,592 (43 and 40) and 46,080 atoms (43 and 43).  Beyond,
 // 8 lanes cost the CN pass about half as much again per entry, and pay where a few structures'
 // lists are so long that their chains outlast the rest: where the longest list (mx: per
 // structure, as the sizing pass found them) is at least twice the mean over the atoms of their
@@ -959,6 +960,7 @@ int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
 int wide_passes(const d3_handle* h, const Plan& P, const int* mx) {
     if (h->prm.precision != D3_MIXED || P.Nr == 0) return 0;
     if (P.Nr <= 32768) return 3;
+    if (P.Nr <= 46080) return 1;
     if (P.Nr > 262144) return 0;
     double most = 0.0, sum = 0.0;
     for (int s = 0; s < P.B; ++s) {
