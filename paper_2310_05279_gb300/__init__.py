@@ -319,7 +319,7 @@ def _autograd_function():
         apply(pos, theta, d3, types, offsets, cells, pbc): pos cuda float64 (N,3) [A],
         theta cuda float64 (4,) = (s6, s8, a1, a2[bohr]).  Returns E (B,) [eV] and F (N,3)
         [eV/A].  Gradients flow to pos and theta; the backward runs in the handle's
-        precision (FP64 duals for an FP64 handle; for a mixed handle the forward's mixed
+        precision (FP64 values and tangents for an FP64 handle; for a mixed handle the forward's mixed
         arithmetic with FP32 tangents)."""
 
         @staticmethod

@@ -326,13 +326,13 @@ __global__ void __launch_bounds__(128) kb_disp(Work w, BW b, BConsts c, const db
     t6 = lanes_sum(fma(3.0, t6t, t6)); t8 = lanes_sum(t8); ta = lanes_sum(ta); tR = lanes_sum(tR);
     if (!live || lane != 0) return;
     b.dEdn[p] = Dual{dn, dnt};
-    b.F[3 * p] = Dual{Gx, 0.0};
-    b.F[3 * p + 1] = Dual{Gy, 0.0};
-    b.F[3 * p + 2] = Dual{Gz, 0.0};
-    b.th[4 * p] = Dual{0.0, 0.5 * t6};
-    b.th[4 * p + 1] = Dual{0.0, 0.5 * t8};
-    b.th[4 * p + 2] = Dual{0.0, -0.5 * ta};
-    b.th[4 * p + 3] = Dual{0.0, -0.5 * tR};
+    b.F[3 * p].v = Gx;
+    b.F[3 * p + 1].v = Gy;
+    b.F[3 * p + 2].v = Gz;
+    b.th[4 * p].t = 0.5 * t6;
+    b.th[4 * p + 1].t = 0.5 * t8;
+    b.th[4 * p + 2].t = -0.5 * ta;
+    b.th[4 * p + 3].t = -0.5 * tR;
 }
 
 // ---- mixed form of the dispersion pass of the backward: the same dual-number
@@ -742,8 +742,8 @@ __global__ void __launch_bounds__(128) kb_chain_mixed(Work w, BW b, Consts c, co
     }
 }
 
-// per-structure sums of dE/dtheta (value and tangent), fixed order
-__global__ void __launch_bounds__(256) kb_struct_sum(Work w, BW b) {
+// per-structure sums of dE/dtheta (value and tangent; in the FP64 form the values are in the tangents), fixed order
+__global__ void __launch_bounds__(256) kb_struct_sum(Work w, BW b, bool values) {
     const int s = blockIdx.x;
     const StructGeo& G = w.geo[s];
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(256) kb_struct_sum(Work w, BW b) {
         const int64_t p = G.atom_base + k;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            acc[m] += b.th[4 * p + m].v;
+            if (values) acc[m] += b.th[4 * p + m].v;
             acc[4 + m] += b.th[4 * p + m].t;
         }
     }
@@ -814,7 +814,7 @@ cudaError_t backward_impl(const Work& w, const Consts& cc, const double* c6d, co
             if (dLdx) kb_chain<<<nl, TB, 0, st>>>(w, b, c, gE, dLdx);
         }
     }
-    kb_struct_sum<<<B, 256, 0, st>>>(w, b);
+    kb_struct_sum<<<B, 256, 0, st>>>(w, b, mixed);
     if (dLdp) kb_param_grad<<<1, 256, 0, st>>>(b, B, gE, dLdp);
     return cudaGetLastError();
 }

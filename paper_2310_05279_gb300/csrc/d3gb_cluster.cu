@@ -325,7 +325,6 @@ struct ClusterRow {
     int cnt;
 };
 
-template <int R, bool SITE, bool SPLIT>
 __device__ __forceinline__ ClusterRow cluster_row(const Work& w, int64_t I, int il) {
     ClusterRow C;
     const StructGeo& G = w.geo[w.clu_sid[I]];
@@ -635,7 +634,7 @@ __global__ void __launch_bounds__(256, 1) k_disp_cl_split(Work w, Consts c, cons
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nq = w.work_ctr[2];
     for (int k = blockIdx.x; k < nq; k += gridDim.x) {
-        const ClusterRow C = cluster_row<R, SITE, true>(w, w.split_q[k], lane & 7);
+        const ClusterRow C = cluster_row(w, w.split_q[k], lane & 7);
         ClusterPass<R, SITE, true> P(w, C.p);
         cluster_setup(P, w, c, C, tab, lane);
         const int nblocks = (C.cnt + 31) >> 5, nchunks = (nblocks + 1) >> 1;

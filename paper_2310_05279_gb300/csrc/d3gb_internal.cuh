@@ -12,10 +12,8 @@
 //                split of the position (x = hi + lo, hi on a 2^-10 bohr grid),
 //                tsrc = type | (data source << 4) as int bits.  One 256-bit
 //                load fetches the whole record.
-//   lists        per structure, one row of cap_s entries per atom:
-//                entry k of sorted atom p is at list_base_s + (p - atom_base_s) * cap_s + k.
-//                A thread appends to its own row, so every 32-byte sector is
-//                filled by one thread, and reads it 4 entries per 16-byte load.
+//   lists        per atom, cap_s entries each, the rows of 32 consecutive atoms interleaved in
+//                groups of 4 entries (list_row, list_off); per cluster, one row of cap_cl entries.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -160,7 +158,7 @@ struct Work {
     int* maxcnt;             // [3*B] per structure, the longest list of an atom or cluster: disp (cluster lists:
                              // the most atoms in a cluster's window), cn, cluster
     int* work_ctr;           // [3] persistent-kernel work counters, length of split_q (zeroed before each build)
-    // cluster lists of the dispersion pass (mixed form)
+    // cluster lists of the dispersion pass
     int cl_mode;             // build: 1 = CN per-atom lists and cluster lists, 0 = both per-atom lists
     int64_t ncl;             // clusters over the batch
     const int* clu_sid;      // [ncl] structure of each cluster

@@ -655,9 +655,8 @@ __global__ void __launch_bounds__(128) k_disp(Work w, Consts c, const typename R
 // The chain-rule virial is accumulated per atom as -dE/dn_i sum_q f'(r) d(x)d/r
 // (ordered pairs; equal to the symmetric form), whose diagonal terms all have
 // one sign, so the cancellation between atoms and against the dispersion part
-// happens in FP64 (per-atom sums and the per-structure reduction).  The force
-// coefficient (dE/dn_i + dE/dn_q) f'(r)/r uses the double-single argument, the
-// exact rc and 1/r from the double-single r^2.
+// happens in FP64 (per-atom sums and the per-structure reduction).  The pair's
+// coefficient f'(r)/r is the one that the CN pass stored.
 //
 // ATOMV: also the per-atom virial of Eq. 7 (row-major, eV) into w_atom:
 //   W_i = D_i - sum_j dE/dn_j f'(r)/r d (x) d - P_i (x) G_i - sum_j f'(r)/r P_j (x) d,
@@ -666,10 +665,8 @@ __global__ void __launch_bounds__(128) k_disp(Work w, Consts c, const typename R
 // partners' site energies on r_ji through their own coordination numbers, the
 // last two the dependence through n_i and through the CNs of other partners.
 template <bool MIXED, bool ATOMV>
-__global__ void __launch_bounds__(128) k_chain(Work w, Consts c, const float4* __restrict__ rcpair,
-                                              const float2* __restrict__ exptab, double* __restrict__ F,
-                                              double* __restrict__ e_atom, double* __restrict__ cn_out,
-                                              double* __restrict__ w_atom) {
+__global__ void __launch_bounds__(128) k_chain(Work w, Consts c, double* __restrict__ F, double* __restrict__ e_atom,
+                                              double* __restrict__ cn_out, double* __restrict__ w_atom) {
     using T = typename Real<MIXED>::T;
     using T4 = typename Real<MIXED>::T4;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -680,7 +677,6 @@ __global__ void __launch_bounds__(128) k_chain(Work w, Consts c, const float4* _
     const StructGeo& G = w.geo[w.sid[p]];
     const ListView LV{w.nbr_cn + list_row(G.list_base_cn, p - G.atom_base, G.cap_cn)};
     const int cnt = w.cnt_cn[p];
-    const T rc2 = MIXED ? (T)c.rc_cn2f : (T)c.rc_cn2, k1 = MIXED ? (T)c.k1f : (T)c.k1;
     T fx = 0, fy = 0, fz = 0;
     double Sxx = 0, Syy = 0, Szz = 0, Sxy = 0, Sxz = 0, Syz = 0;
     double Tm[6] = {0, 0, 0, 0, 0, 0}, Gv[3] = {0, 0, 0}, Mm[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -1004,9 +1000,9 @@ cudaError_t forward_impl(const Work& w, const Consts& c, const Tabs& tb, double*
         if (MIXED && (w.wide & 2) && !w_atom)
             k_chain_wide<<<nblk(w.Nr * kWide, 128), 128, 0, st>>>(w, c, F, e_atom, cn_out);
         else if (w_atom)
-            k_chain<MIXED, true><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, tb.rcpair, tb.exptab, F, e_atom, cn_out, w_atom);
+            k_chain<MIXED, true><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, F, e_atom, cn_out, w_atom);
         else
-            k_chain<MIXED, false><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, tb.rcpair, tb.exptab, F, e_atom, cn_out, nullptr);
+            k_chain<MIXED, false><<<nblk(w.Nr, TB), TB, 0, st>>>(w, c, F, e_atom, cn_out, nullptr);
     }
     mark(5);
     if (B > 0 && w.max_natoms <= kFinChunk) {
