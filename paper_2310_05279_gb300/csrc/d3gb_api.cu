@@ -939,35 +939,37 @@ int build_by_struct(const d3_handle* h, const Plan& P, int gcount) {
 
 // Whether the mixed form's CN pass (bit 0) and chain pass (bit 1) take 8 lanes per atom.
 // For few atoms one thread per atom is a chain of 0.55 us per list entry (64 atoms: CN pass
-// 37 us and 13 with 8 lanes, chain pass 18 and 12; 6,912 atoms: 36 and 15, 20 and 15), in the
-// CN pass also for 34,560 (41 and 35), 42,592 (43 and 40) and 46,080 atoms (43 and 43).  Beyond,
-// 8 lanes cost the CN pass about half as much again per entry, and pay where a few structures'
-// lists are so long that their chains outlast the rest: where the longest list (mx: per
-// structure, as the sizing pass found them) is at least twice the mean over the atoms of their
-// structures' longest, up to some 250,000 atoms.  One thread and 8 lanes per atom, us:
+// 37 us and 13 with 8 lanes, chain pass 18 and 12; 6,912 atoms: 36 and 15, 20 and 15).  Beyond,
+// 8 lanes cost the CN pass about half as much again, some 1.2e-5 us per entry, and pay where the
+// longest list's chain lasts longer than that, which for even lists is up to 46,000 atoms, or
+// where it is at least twice the mean, so that a few structures outlast the rest, up to some
+// 250,000 atoms.  (mx: the longest list of each structure, from the sizing pass; the mean is that
+// over the atoms.)  One thread and 8 lanes per atom, us:
 //   longest / mean   structures, atoms
-//   149 / 36         64 uneven, 52,832                74 and  39
-//    89 / 37         16 uneven, 57,258                53 and  38
-//   156 / 45         100 of equal size, 100,037       95 and  70
-//   138 / 38         128 uneven, 112,241              91 and  70
-//    94 / 38         256 uneven, 221,102             129 and 129
+//    76 / 52         24 bilayers, 34,560               41 and  35
+//    60 / 60         a box of 42,592                   43 and  40
+//    76 / 52         32 bilayers, 46,080               43 and  43
+//   149 / 36         64 uneven, 52,832                 74 and  39
+//    89 / 37         16 uneven, 57,258                 53 and  38
+//   156 / 45         100 of equal size, 100,037        95 and  70
+//   138 / 38         128 uneven, 112,241               91 and  70
+//    94 / 38         256 uneven, 221,102              129 and 129
 //   103 / 74         128 uneven of one element, 122,742   96 and 115
 //   109 / 77         256 uneven of one element, 210,601  151 and 193
-//    76 / 52         64 bilayers, 92,160              51 and  77
+//    76 / 52         64 bilayers, 92,160               51 and  77
 //    61 / 59         64 and 128 equal frames of five elements, 87,808 and 175,616   62 and 73, 108 and 134
 // (512 uneven, 497,680 atoms: 245 and 274).  The chain pass does not gain there (208,635 atoms:
 // 76 and 146).
 int wide_passes(const d3_handle* h, const Plan& P, const int* mx) {
     if (h->prm.precision != D3_MIXED || P.Nr == 0) return 0;
     if (P.Nr <= 32768) return 3;
-    if (P.Nr <= 46080) return 1;
     if (P.Nr > 262144) return 0;
     double most = 0.0, sum = 0.0;
     for (int s = 0; s < P.B; ++s) {
         most = std::max(most, (double)mx[3 * (size_t)s + 1]);
         sum += (double)mx[3 * (size_t)s + 1] * P.geo[s].natoms;
     }
-    return most * (double)P.Nr >= 2.0 * sum ? 1 : 0;
+    return most * (double)P.Nr >= 2.0 * sum || 0.55 * most > 1.2e-5 * sum ? 1 : 0;
 }
 
 // Make the plan match the geometry; on a new geometry run the build once
