@@ -80,9 +80,9 @@ __device__ __forceinline__ void add_lattice(double (&x)[3], const StructGeo& G, 
 // wrapped position, cell and in-cell key, returns the cell.  The lattice translation that
 // wraps an atom is chosen from its FP32 fractional coordinates; the wrapped position is
 // x - sum_k n_k H_k in FP64 (x itself when the atom is inside the cell).
-__device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int s, int64_t i,
-                                         const double* __restrict__ pos, const int32_t* __restrict__ types,
-                                         float (&f)[3]) {
+// *xmax: its largest |coordinate|, *type: its element, one bit.
+__device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int64_t i, const double* __restrict__ pos,
+                                         const int32_t* __restrict__ types, float (&f)[3], float* xmax, int* type) {
     double xb[3];
     bool fin = true;
 #pragma unroll
@@ -96,6 +96,7 @@ __device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int 
     }
     const int t = types[i];
     if (t < 0 || t >= w.T) atomicOr(w.status, ST_TYPE);
+    *type = 1 << (t < 0 || t >= w.T ? 0 : t);
     const float xf[3] = {(float)xb[0], (float)xb[1], (float)xb[2]};
     int n[3] = {0, 0, 0};
 #pragma unroll
@@ -116,14 +117,13 @@ __device__ __forceinline__ int wrap_atom(const Work& w, const StructGeo& G, int 
     if (n[0] | n[1] | n[2]) add_lattice(xw, G, -n[0], -n[1], -n[2]);
     // the exact FP32 split of positions needs |x| < 2^13 bohr (checked in FP32)
     bool far = false;
-    float xmax = 0.0f;
+    *xmax = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float xr = xf[a] - ((float)n[0] * G.Hh[a] + (float)n[1] * G.Hh[3 + a] + (float)n[2] * G.Hh[6 + a]);
         far = far || !(fabsf(xr) < kMaxCoordBohr);
-        xmax = fmaxf(xmax, fabsf(xr));
+        *xmax = fmaxf(*xmax, fabsf(xr));
     }
-    if (w.ipos && __float_as_int(xmax) > w.ixmax[s]) atomicMax(&w.ixmax[s], __float_as_int(xmax));
     if (far && fin) atomicOr(w.status, ST_RANGE);
 #pragma unroll
     for (int a = 0; a < 3; ++a) w.xw[3 * i + a] = xw[a];
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
     // A block within one structure (most, where structures are large) puts its range together
     // in shared memory: atomics on one structure's six words, one set a warp, were most of this
     // kernel on a single box (1,048,576 atoms 160 us, now 32).
-    __shared__ int blo[3], bhi[3];
+    __shared__ int blo[3], bhi[3], bx, bt;
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x, i = i0 + threadIdx.x;
     if (skip_build(w)) return;  // the whole grid
     const int s0 = w.sid_in[i0];
@@ -155,13 +155,16 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
     if (threadIdx.x < 3) {
         blo[threadIdx.x] = 0x7f800000;  // above every fraction
         bhi[threadIdx.x] = 0;
+        bx = bt = 0;
     }
     __syncthreads();
     if (i < w.Nr) {
         const int s = w.sid_in[i];
         const StructGeo& G = w.geo[s];
         float f[3];
-        const int cid = wrap_atom(w, G, s, i, pos, types, f);
+        float xmax;
+        int type;
+        const int cid = wrap_atom(w, G, i, pos, types, f, &xmax, &type);
         w.slot_of[i] = atomicAdd(&w.cnt_real[cid], 1);
         // occupied range: one atomic per group of lanes in the same structure
         const unsigned grp = __match_any_sync(__activemask(), s);
@@ -176,8 +179,19 @@ __global__ void __launch_bounds__(256) k_wrap(Work w, const double* __restrict__
                 atomicMax(one ? &bhi[k] : &w.frange[3 * (w.B + s) + k], hi);
             }
         }
+        if (w.ipos) {
+            const int x = __reduce_max_sync(grp, __float_as_int(xmax)), t = __reduce_or_sync(grp, type);
+            if (leader) {
+                atomicMax(one ? &bx : &w.ixmax[s], x);
+                atomicOr(one ? &bt : &w.tmask[s], t);
+            }
+        }
     }
     __syncthreads();
+    if (w.ipos && one && threadIdx.x == 0) {
+        atomicMax(&w.ixmax[s0], bx);
+        atomicOr(&w.tmask[s0], bt);
+    }
     if (one && threadIdx.x < 3 && w.geo[s0].pbc[threadIdx.x]) {
         atomicMin(&w.frange[3 * s0 + threadIdx.x], blo[threadIdx.x]);
         atomicMax(&w.frange[3 * (w.B + s0) + threadIdx.x], bhi[threadIdx.x]);
@@ -476,7 +490,7 @@ __device__ __forceinline__ void fill_real(Work& w, int64_t p, int i, int s, cons
     if (t < 0 || t >= w.T) t = 0;
     w.perm[p] = i;
     w.sid[p] = s;
-    if (w.ipos && !((w.tmask[s] >> t) & 1)) atomicOr(&w.tmask[s], 1 << t);
+    if (w.ipos && !((w.tmask[s] >> t) & 1)) atomicOr(&w.tmask[s], 1 << t);  // (an element new to kept lists)
     w.cell_sorted[p] = w.cell_of[i];
     const double x[3] = {w.xw[3 * i], w.xw[3 * i + 1], w.xw[3 * i + 2]};
     store_pos(w, p, s, x, rk_tab[t], t | ((int)p << 4));
@@ -609,7 +623,7 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
                                                                     const int32_t* __restrict__ types,
                                                                     const double* __restrict__ rk_tab) {
     extern __shared__ int counts[];  // [2][ncell + 1]: atoms and images per cell, then their starts
-    __shared__ int fr[6], seg[2], wsum[kStructThreads / 32];
+    __shared__ int fr[6], seg[2], xt[2], wsum[kStructThreads / 32];
     const int s = blockIdx.x, tid = threadIdx.x;
     const StructGeo& G = w.geo[s];
     const int n = G.natoms;
@@ -622,16 +636,17 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
         fr[tid] = 0x7f7f7f7f;
         fr[3 + tid] = 0;
         w.maxcnt[3 * s + tid] = 0;
-        if (w.ipos) w.tmask[s] = w.ixmax[s] = 0;
+        xt[0] = xt[1] = 0;
     }
     __syncthreads();
     for (int k0 = 0; k0 < n; k0 += kStructThreads) {
         const int k = k0 + tid;
         const bool live = k < n;
-        float f[3] = {0.f, 0.f, 0.f};
+        float f[3] = {0.f, 0.f, 0.f}, xmax = 0.0f;
+        int type = 0;
         if (live) {
             const int64_t i = a0 + k;
-            const int cid = wrap_atom(w, G, s, i, pos, types, f);
+            const int cid = wrap_atom(w, G, i, pos, types, f, &xmax, &type);
             w.slot_of[i] = atomicAdd(&cr[cid - c0], 1);
         }
 #pragma unroll
@@ -644,8 +659,19 @@ __global__ void __launch_bounds__(kStructThreads, 1024 / kStructThreads) k_build
                 atomicMax(&fr[3 + m], hi);
             }
         }
+        if (w.ipos) {
+            const int x = __reduce_max_sync(0xffffffffu, __float_as_int(xmax)), t = __reduce_or_sync(0xffffffffu, type);
+            if ((tid & 31) == 0) {
+                atomicMax(&xt[0], x);
+                atomicOr(&xt[1], t);
+            }
+        }
     }
     __syncthreads();
+    if (w.ipos && tid == 0) {
+        w.ixmax[s] = xt[0];
+        w.tmask[s] = xt[1];
+    }
     // images: the block's total first (one segment of slots), then the records
     int mine = 0;
     for (int k = tid; k < n; k += kStructThreads) mine += ImageRange(w, G, a0 + k, fr, fr + 3).count;
