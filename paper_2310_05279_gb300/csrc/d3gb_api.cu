@@ -223,8 +223,9 @@ struct d3_handle {
     Plan plan;
     // staging buffers of the host-memory entry point
     Pinned pin;  // plan upload and sizing read-back
-    cudaEvent_t pin_copied = nullptr;  // recorded after the copies of the last upload
-    bool pin_busy = false;             // they have not been waited for
+    // its last copies: over, pending before pin_copied, or of a call that failed before it waited for them
+    enum { kPinFree, kPinEvent, kPinUnknown } pin_state = kPinFree;
+    cudaEvent_t pin_copied = nullptr;
     DevBuf stage;
     size_t stage_atoms = 0, stage_structs = 0;
     double *s_pos = nullptr, *s_E = nullptr, *s_F = nullptr, *s_W = nullptr;
@@ -535,7 +536,7 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     // Work of earlier calls may still use the memory.  What runs on st is ordered before this; what runs on
     // another stream, as a caller's graph may, is waited for by giving the memory back (cudaFree waits for
     // the device; cudaDeviceSynchronize would fail, and end the capture, while another thread captures)
-    if (P.stream != st || P.captured) P.mem.release();
+    if (P.stream != st || P.captured || h->pin_state == d3_handle::kPinUnknown) P.mem.release();
     P.stream = st;
     P.captured = P.unknown = false;
     const int B = P.B;
@@ -711,13 +712,13 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     int* gate = w.gate;
     w.gate = nullptr;  // the plan's own Work builds unconditionally; enqueue_build gates a copy
     P.gate = gate;
-    // geometry and offsets through page-locked memory, once the copies of the last upload are over
-    // (a batch without atoms has no sizing pass that waits for them); the per-atom and per-cluster
-    // indices are formed on the device
+    // geometry and offsets through page-locked memory, once the copies of the last upload are over:
+    // the sizing pass waits for them, but a batch without atoms has none, and its event is waited for
+    // here; the per-atom and per-cluster indices are formed on the device
     const size_t ngeo = sizeof(StructGeo) * (size_t)B, noff = sizeof(int64_t) * ((size_t)B + 1);
-    if (h->pin_busy) e = cudaEventSynchronize(h->pin_copied);
-    h->pin_busy = false;
-    if (e == cudaSuccess && !h->pin_copied) e = cudaEventCreateWithFlags(&h->pin_copied, cudaEventDisableTiming);
+    if (h->pin_state == d3_handle::kPinEvent) e = cudaEventSynchronize(h->pin_copied);
+    h->pin_state = d3_handle::kPinFree;
+    if (e == cudaSuccess && Nr == 0 && !h->pin_copied) e = cudaEventCreateWithFlags(&h->pin_copied, cudaEventDisableTiming);
     if (e == cudaSuccess) e = h->pin.reserve(ngeo + noff + sizeof(int) * (3 * (size_t)B + 2));
     if (e != cudaSuccess) {
         P.valid = false;
@@ -727,11 +728,8 @@ d3_status plan_alloc(d3_handle* h, Plan& P, cudaStream_t st) {
     std::memcpy(h->pin.p + ngeo, P.offsets.data(), noff);
     e = cudaMemcpyAsync(dgeo, h->pin.p, ngeo, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(doff, h->pin.p + ngeo, noff, cudaMemcpyHostToDevice, st);
-    h->pin_busy = true;
-    if (cudaEventRecord(h->pin_copied, st) != cudaSuccess) {
-        cudaStreamSynchronize(st);
-        h->pin_busy = false;
-    }
+    h->pin_state = d3_handle::kPinUnknown;
+    if (Nr == 0 && cudaEventRecord(h->pin_copied, st) == cudaSuccess) h->pin_state = d3_handle::kPinEvent;
     if (e == cudaSuccess) e = launch_plan_ids(dgeo, doff, B, Nr, ncl, nfin, dsid, dclu, dfin, st);
     if (e != cudaSuccess) {
         P.valid = false;
@@ -1019,6 +1017,7 @@ d3_status ensure_plan(d3_handle* h, int32_t B, const int64_t* offsets, const dou
             e = cudaMemcpyAsync(mx + 3 * (size_t)B + 1, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(h, e, "sizing pass");
+        h->pin_state = d3_handle::kPinFree;
         const int gcount = mx[3 * (size_t)B], status = mx[3 * (size_t)B + 1];
         if (status & ST_NONFINITE) return fail(h, D3_ERR_NONFINITE, "non-finite coordinate");
         if (status & ST_TYPE) return fail(h, D3_ERR_TYPE, "atom type out of range");
