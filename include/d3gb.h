@@ -80,7 +80,7 @@ enum { D3_FP64 = 0, D3_MIXED = 1 };
  * dispersion pass forms its C6 interpolation and its sums in 64-bit fixed
  * point, each atom's sums in units below an FP64 rounding of the sum of their
  * terms' sizes; for an atom without a partner within R_cn the unit follows
- * terms at R_cn, up to 2e-14 of a lone pair's force at 11 A.  Damping radii
+ * terms at R_cn, up to 3e-14 of a lone pair's force at 11 A.  Damping radii
  * beyond 1e-3 to 1e4 bohr, R_cn below 4 A and coefficients out of FP32 range
  * take FP64 sums instead). */
 typedef struct d3_params {
